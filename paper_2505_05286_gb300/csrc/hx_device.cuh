@@ -146,7 +146,6 @@ struct WarpShared {
   int64_t q[HX_MAX_INST];       // t_queue: Eq. comp summed over requests dispatched and unfinished
   uint64_t ekey[HX_MAX_INST];   // next completion event key per instance
   int32_t erid[HX_MAX_INST];    // its request id
-  int64_t orew[HX_MAX_INST];    // cached (1 - alpha) * reward per instance (its owner lane's)
   int32_t hoff[HX_MAX_INST];    // local queue: heap offset in the arena
   int32_t hsize[HX_MAX_INST];   //              heap size
   uint8_t cnt[HX_MAX_INST];     // running calls (the first cnt of the instance's slot keys)
@@ -156,10 +155,9 @@ struct WarpShared {
   int32_t pest[HX_MAX_K];
   // per-simulation constants
   int32_t A, one_minus_a;        // alpha and 1 - alpha, fixed point
-  int32_t rewards, oob;          // 1 when dispatch scores need the reward term; an index check
-                                // failed (bounds-checked build)
   int64_t G, beta;
-  float betaf, pad3;            // beta as a float (the reward quotient's numerator)
+  longlong2 tie;                // t_queue up to which the least cost alone decides a dispatch; cost mask
+  float4 fscore;                // the score filter's constants (score_range)
   int64_t frest[kFRows];        // rest-of-path cost of the budget denominator by fcode
   int32_t lpol, dpol, recj, kcap, rr, bump;
   // this warp's scratch slices and the current trace's offsets

@@ -98,6 +98,39 @@ __device__ __forceinline__ int64_t reward_of(int64_t beta, int64_t q) {
   return r < kRewardCap ? r : kRewardCap;
 }
 
+__device__ __forceinline__ float warp_max_f32(float v) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+// Bounds of the score (1 - alpha) * min(floor(beta / max(q, 1)), cap) - alpha * e
+// in single precision, f = ((1 - alpha) beta, (1 - alpha) cap, 2 (1 - alpha)):
+// with t the reward term, u the cost term and w = t + u, the conversions of q
+// and e, the approximate reciprocal (1 ulp), the rounded constants and the
+// products leave t within 5 * 2^-24 and u within 2^-23 of their values without
+// the floor, the difference adds 2^-24 w and the bounds' own rounding 2^-23 w,
+// less than 2^-20 w together; the floor lowers the score by less than 1 - alpha.
+// So lo - (1 - alpha) <= score <= hi - (1 - alpha), and an instance whose hi is
+// below the largest lo loses.  neg_a = -inf (no instance): lo = -inf, hi = NaN,
+// below everything.  One 32-bit reduction and no division in place of a 64-bit
+// division pass per changed queue and a three-step 64-bit argmax: an event is a
+// chain of dependent instructions, and these were the longest part of it (19
+// traces x 5003 queries x 512 points on 32 instances 159.2 -> 127.3 ms, 8 x
+// 20000 x 1024 on 64 instances 566.0 -> 529.4 ms).
+struct ScoreRange {
+  float lo, hi;
+};
+
+__device__ __forceinline__ ScoreRange score_range(int64_t q, int e, float4 f, float neg_a) {
+  float rq;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rq) : "f"((float)(q > 1 ? q : 1)));
+  const float t = fminf(f.x * rq, f.y), nu = neg_a * (float)e;
+  const float s = t + nu, w = t - nu;
+  constexpr float kErr = 1.0f / (1 << 20);
+  return {fmaf(w, -kErr, s), fmaf(w, kErr, s + f.z)};
+}
+
 // (num * tb) / d truncated toward zero, for |num| < 2^41 and 1 <= tb <= d < 2^33:
 // splitting num = q1 * d + r1 keeps every product below 2^63.
 __device__ __forceinline__ int64_t scaled_div(int64_t num, int64_t tb, int64_t d) {
@@ -465,6 +498,21 @@ __device__ __forceinline__ int2 push_pop(WarpShared* W, const CallRec* rec, int6
   return make_int2(top.rid, top.svc);
 }
 
+// The dispatch winner from exact scores, for the dispatches whose float bounds
+// overlap: highest score, ties to the lowest instance.  All lanes call.
+__device__ __noinline__ int exact_winner(const WarpShared* W, int64_t q0, int64_t q1, int e0, int e1, bool ok0, bool ok1,
+                                         int lane) {
+  const uint64_t beta = (uint64_t)W->beta;
+  const float betaf = u64_to_float(beta);
+  const int64_t A = W->A, oma = W->one_minus_a;
+  const uint64_t r0 = udiv_trial_f(beta, betaf, q0 > 1 ? (uint64_t)q0 : 1ull);
+  const uint64_t r1 = udiv_trial_f(beta, betaf, q1 > 1 ? (uint64_t)q1 : 1ull);
+  const int64_t s0 = ok0 ? oma * (int64_t)(r0 < (uint64_t)kRewardCap ? r0 : kRewardCap) - A * e0 : INT64_MIN;
+  const int64_t s1 = ok1 ? oma * (int64_t)(r1 < (uint64_t)kRewardCap ? r1 : kRewardCap) - A * e1 : INT64_MIN;
+  const bool take1 = s1 > s0;
+  return warp_argmax_s64(take1 ? s1 : s0, take1 ? lane + 32 : lane);
+}
+
 // All lanes: a query's evaluation call finished at `now` (Sec. 4.3's metrics).
 __device__ __forceinline__ void finish_query(WarpShared* W, int& dn, int32_t qid, int64_t now, int64_t arrival,
                                             int64_t deadline, int lane) {
@@ -574,7 +622,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     // per-instance state that every lane reads later: written before the
     // barrier below
     for (int m = lane; m < 64; m += 32) {
-      W->q[m] = 0;
+      W->q[m] = m < N ? 0 : INT64_MAX;
       W->hoff[m] = 0;
       W->hcl[m] = 0;
       W->hsize[m] = 0;
@@ -608,11 +656,17 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       const int64_t A = a.alpha[p];
       W->A = (int32_t)A;
       W->one_minus_a = (int32_t)(kScale - A);
-      // rewards carry no weight at alpha = 1 and are unused by round robin
-      W->rewards = (A != kScale && !(kGeneric && a.dpol[p] == HX_DISPATCH_RR)) ? 1 : 0;
       W->G = a.gamma[p];
-      W->beta = a.beta[p];
-      W->betaf = u64_to_float((uint64_t)a.beta[p]);
+      const int64_t beta = a.beta[p], oma = kScale - A;
+      W->beta = beta;
+      W->fscore = make_float4((float)((double)oma * (double)beta), (float)oma * (float)kRewardCap, 2.0f * (float)oma, 0.0f);
+      // t_queue up to which instances share the greatest reward and beat every
+      // other one whatever its cost (below 2^28): all of them when rewards have
+      // no weight (alpha = 1); the idle ones (max(t_queue, 1) = 1) when the step
+      // from beta to the next reward, at most beta / 2, outweighs any cost
+      // difference; else none.  Instances past N hold INT64_MAX.
+      const bool idle_top = oma * (reward_of(beta, 1) - reward_of(beta, 2)) > A << 28;
+      W->tie = make_longlong2(A == kScale ? INT64_MAX - 1 : idle_top ? 1 : -1, A != 0 ? 0xffffffffll : 0ll);
       W->lpol = a.lpol[p];
       W->dpol = a.dpol[p];
       W->recj = a.rec_map ? a.rec_map[sim] : -1;
@@ -640,19 +694,10 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     // this lane's instances m0 = lane and m1 = lane + 32: t_queue in W->q[m]
     // and the next completion's event key and request id in W->ekey[m] and
     // W->erid[m] (every change stored alike by every lane; the owner reads
-    // the keys at the loop top), the cached (1 - alpha) * reward in
-    // W->orew[m] (the owner lane alone) and its staleness in dirty0 / dirty1;
-    // shared memory rather than registers leaves the allocator room.
-    // Instances past N start with a reward far below any real score
-    // (|alpha * est| < 2^52), so the argmax needs no validity test.
-    const int32_t oma32 = W->one_minus_a;
-    // rewards carry weight (alpha < 1 with workload-balanced dispatch): kept in
-    // a predicate register rather than re-read at every queue-cost change
-    const bool rewards_on = W->rewards != 0;
-    const int64_t orew_idle = (int64_t)oma32 * reward_of(W->beta, 0);
-    W->orew[m0] = valid0 ? orew_idle : -(int64_t(1) << 62);
-    W->orew[m1] = valid1 ? orew_idle : -(int64_t(1) << 62);
-    bool dirty0 = false, dirty1 = false;
+    // its own); shared memory rather than registers leaves the allocator room.
+    // -alpha as the score filter's cost weight; -inf keeps instances past N out of it
+    const float neg_a0 = valid0 ? -(float)W->A : -INFINITY;
+    const float neg_a1 = valid1 ? -(float)W->A : -INFINITY;
     W->ekey[m0] = kKeyInf;
     W->ekey[m1] = kKeyInf;
     // this event's dispatches, entry j on lane j
@@ -771,9 +816,6 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         set_key(m, head);
         {
           W->q[m] = W->q[m] - est_m;  // every lane stores the same value
-          const bool stale = rewards_on;
-          dirty0 = lane == m ? stale : dirty0;
-          dirty1 = lane + 32 == m ? stale : dirty1;
         }
         // the freed slot needs a batch boundary only if requests wait for it
         if (hs_m > 0) touched |= 1ull << m;
@@ -850,19 +892,6 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         // Eq. (comp) and the service time on this lane's two instances
         const int2 ev0 = r->ev[ty0], ev1 = r->ev[ty1];
         const int e0 = ev0.x, e1 = ev1.x, v0 = ev0.y, v1 = ev1.y;
-        // SIMT division passes: each lane refreshes one stale reward of its
-        // instances per pass (two passes at most)
-        const uint64_t beta = (uint64_t)W->beta;
-        while (__any_sync(kFull, dirty0 || dirty1)) {
-          const bool rj = dirty0 || dirty1;
-          const int64_t q = W->q[dirty0 ? m0 : m1];
-          const uint64_t res = udiv_trial_f(rj ? beta : 0ull, rj ? W->betaf : 0.0f, (rj && q > 1) ? (uint64_t)q : 1ull);
-          const int64_t orew =
-              (int64_t)W->one_minus_a * (res < (uint64_t)kRewardCap ? (int64_t)res : kRewardCap);
-          if (rj) W->orew[dirty0 ? m0 : m1] = orew;
-          if (dirty0) dirty0 = false;
-          else dirty1 = false;
-        }
         int m;
         // a re-issued request avoids the instance it timed out on
         const int excl = kGeneric ? W->excl : -1;
@@ -872,15 +901,30 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
           __syncwarp();
           if (lane == 0) W->rr = (m + 1 == N) ? 0 : m + 1;
         } else {
-          const int32_t A = W->A;
-          int64_t s0 = W->orew[m0] - (int64_t)A * e0;
-          int64_t s1 = W->orew[m1] - (int64_t)A * e1;
-          if (kGeneric && excl >= 0) {
-            if (m0 == excl) s0 = INT64_MIN;
-            if (m1 == excl) s1 = INT64_MIN;
+          const int64_t q0 = W->q[m0], q1 = W->q[m1];
+          // instances that tie in their reward and beat all others: the least cost wins
+          // (the lowest instance at alpha = 0, where costs have no weight)
+          const longlong2 tie = W->tie;
+          const int64_t q_top = tie.x;
+          const uint32_t cost_mask = (uint32_t)tie.y;
+          const bool top0 = q0 <= q_top, top1 = q1 <= q_top;
+          if (__any_sync(kFull, top0 || top1) && excl < 0) {
+            const uint32_t c0 = top0 ? (uint32_t)e0 & cost_mask : 0xffffffffu, c1 = top1 ? (uint32_t)e1 & cost_mask : 0xffffffffu;
+            const uint32_t least = __reduce_min_sync(kFull, c0 < c1 ? c0 : c1);
+            const unsigned b0 = __ballot_sync(kFull, c0 == least), b1 = __ballot_sync(kFull, c1 == least);
+            m = b0 ? __ffs(b0) - 1 : __ffs(b1) + 31;
+          } else {
+            const float4 f = W->fscore;
+            const ScoreRange a0 = score_range(q0, e0, f, neg_a0), a1 = score_range(q1, e1, f, neg_a1);
+            const float lo = warp_max_f32(fmaxf(a0.lo, a1.lo));
+            const unsigned b0 = __ballot_sync(kFull, a0.hi >= lo), b1 = __ballot_sync(kFull, a1.hi >= lo);
+            // one instance's score can reach the best lower bound: it wins
+            if ((((b0 & (b0 - 1)) | (b1 & (b1 - 1))) == 0) && ((b0 == 0) != (b1 == 0)) && excl < 0) {
+              m = b0 ? __ffs(b0) - 1 : __ffs(b1) + 31;
+            } else {
+              m = exact_winner(W, q0, q1, e0, e1, m0 < N && m0 != excl, m1 < N && m1 != excl, lane);
+            }
           }
-          const bool take1 = s1 > s0;
-          m = warp_argmax_s64(take1 ? s1 : s0, take1 ? m1 : m0);
         }
         if (kGeneric) W->excl = -1;
         HX_BOUND(m >= 0 && m < N)
@@ -889,9 +933,6 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         const int svc_m = __shfl_sync(kFull, m < 32 ? v0 : v1, m & 31);
         {
           W->q[m] = W->q[m] + est_m;  // every lane stores the same value
-          const bool stale = rewards_on;
-          dirty0 = lane == m ? stale : dirty0;
-          dirty1 = lane + 32 == m ? stale : dirty1;
         }
         if (kGeneric) {
           const int recj = W->recj;
