@@ -86,17 +86,26 @@ int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 // the record says.
 constexpr int kMaxDevices = 64;
 std::mutex g_smem_mu;
-int g_smem_limit[kMaxDevices][2] = {};  // [device][0: hx_sim_kernel, 1: hx_sim_kernel_lean]
+constexpr int kSimKernels = 6;
+int g_smem_limit[kMaxDevices][kSimKernels] = {};  // [device][instantiation]
 
-int ensure_dyn_smem(bool generic, int bytes) {
+using SimKernel = void (*)(hx::SimArgs, hx::ClusterK);
+constexpr SimKernel kSimKernel[kSimKernels] = {hx::hx_sim_kernel_lean,   hx::hx_sim_kernel,   hx::hx_sim_kernel_faults,
+                                               hx::hx_sim_kernel_lean32, hx::hx_sim_kernel32, hx::hx_sim_kernel_faults32};
+
+// The instantiation of the simulation kernel a cluster runs on.
+int sim_kernel_of(bool generic, const hx::ClusterK& ck) {
+  return (!generic ? 0 : ck.n_faults == 0 ? 1 : 2) + (ck.n_inst <= 32 ? 3 : 0);
+}
+
+int ensure_dyn_smem(int kernel, int bytes) {
   int dev = 0;
   HX_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxDevices) return fail(HX_ERR_INVALID, "device index out of range");
   std::lock_guard<std::mutex> lock(g_smem_mu);
-  int& cur = g_smem_limit[dev][generic ? 0 : 1];
+  int& cur = g_smem_limit[dev][kernel];
   const int want = std::max(cur, bytes);
-  const void* kfn = generic ? (const void*)hx::hx_sim_kernel : (const void*)hx::hx_sim_kernel_lean;
-  if (cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, want) != cudaSuccess) {
+  if (cudaFuncSetAttribute((const void*)kSimKernel[kernel], cudaFuncAttributeMaxDynamicSharedMemorySize, want) != cudaSuccess) {
     cudaGetLastError();
     return fail(HX_ERR_CUDA, "cannot reserve " + std::to_string(want) +
                                  " bytes of shared memory for the simulation kernel");
@@ -177,7 +186,8 @@ struct hx_sim {
   std::vector<int32_t> record_sims;
   // launch shape
   int blocks = 0, resident_warps = 0, smem_per_block = 0;
-  bool generic = true;  // which instantiation of the simulation kernel runs
+  bool generic = true;
+  int kernel = 1;  // which instantiation of the simulation kernel runs (kSimKernel)
   int64_t scratch_bytes = 0, device_bytes = 0;
   cudaStream_t last_stream = nullptr;
   bool ran = false;
@@ -476,11 +486,11 @@ int upload_traces(hx_sim* h, const hx_trace* traces, cudaStream_t s) {
   return HX_OK;
 }
 
-// WarpShared with its trailing slot array sized for the cluster (and one
-// fail flag per slot when the cluster has fault windows)
-int per_warp_smem(int total_slots, bool faults) {
-  const int64_t ts = std::max(total_slots, 1);
-  return (int)align_up((int64_t)offsetof(hx::WarpShared, slot) + 8 * ts + (faults ? ts : 0), 16);
+// WarpShared and the instance states and slot entries that follow it.
+int per_warp_smem(const hx::ClusterK& ck) {
+  const int64_t slot = ck.n_faults > 0 ? sizeof(hx::Slot64) : sizeof(hx::Slot32);
+  return (int)align_up((int64_t)sizeof(hx::WarpShared) + (ck.n_inst <= 32 ? 32 : 64) * (int64_t)sizeof(hx::InstState) +
+                       slot * ck.slot_entries, 16);
 }
 
 // Kernel-parameter copy of a validated cluster.
@@ -514,7 +524,7 @@ void fill_cluster(const hx_cluster* cluster, hx::ClusterK& ck) {
       ck.cnt[ty]++;
     }
   }
-  ck.total_slots = base;
+  ck.slot_entries = ck.n_inst <= 32 ? 16 * 32 : base + 16;
   // per-tenant SLO multipliers replace slo_mult_fp when given
   ck.n_tenants = std::max(cluster->n_tenants, 1);
   for (int t = 0; t < HX_MAX_TENANTS; ++t)
@@ -530,7 +540,7 @@ void fill_cluster(const hx_cluster* cluster, hx::ClusterK& ck) {
     ck.faults[f].inst = F.inst;
     ck.faults[f].pad = 0;
   }
-  ck.smem_per_warp = per_warp_smem(base, cluster->n_faults > 0);
+  ck.smem_per_warp = per_warp_smem(ck);
 }
 
 // The simulations of opt->sim_subset, checked (in range, distinct) and sorted
@@ -694,10 +704,11 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
     return bail(rc);
 
   h->generic = needs_generic(grid, ck, opt && opt->n_record > 0, opt && opt->force_generic, h->checked);
-  const void* kfn = h->generic ? (const void*)hx::hx_sim_kernel : (const void*)hx::hx_sim_kernel_lean;
+  h->kernel = sim_kernel_of(h->generic, ck);
+  const void* kfn = (const void*)kSimKernel[h->kernel];
   // launch shape of the simulation kernel and its per-warp scratch
   h->smem_per_block = hx::kWarpsPerBlock * ck.smem_per_warp;
-  if ((rc = ensure_dyn_smem(h->generic, h->smem_per_block))) return bail(rc);
+  if ((rc = ensure_dyn_smem(h->kernel, h->smem_per_block))) return bail(rc);
   int bps = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kfn, hx::kWarpsPerBlock * 32, h->smem_per_block) !=
           cudaSuccess ||
@@ -869,16 +880,13 @@ static int hx_sim_run_impl(hx_sim* h, void* stream) {
   ba.point_sums = h->d_point_sums;
 
   const int prep_blocks = (int)std::max<int64_t>(1, (h->n_q + 255) / 256);
-  if (int rc = ensure_dyn_smem(h->generic, h->smem_per_block)) return rc;
+  if (int rc = ensure_dyn_smem(h->kernel, h->smem_per_block)) return rc;
   cudaEvent_t* ev = h->timing ? h->run_ev(h->runs) : nullptr;
   if (ev) HX_CUDA(cudaEventRecord(ev[0], s));
   hx::hx_prep_kernel<<<prep_blocks, 256, 0, s>>>(pa, h->ck);
   HX_CUDA(cudaGetLastError());
   if (ev) HX_CUDA(cudaEventRecord(ev[1], s));
-  if (h->generic)
-    hx::hx_sim_kernel<<<h->blocks, hx::kWarpsPerBlock * 32, h->smem_per_block, s>>>(sa, h->ck);
-  else
-    hx::hx_sim_kernel_lean<<<h->blocks, hx::kWarpsPerBlock * 32, h->smem_per_block, s>>>(sa, h->ck);
+  kSimKernel[h->kernel]<<<h->blocks, hx::kWarpsPerBlock * 32, h->smem_per_block, s>>>(sa, h->ck);
   HX_CUDA(cudaGetLastError());
   if (ev) HX_CUDA(cudaEventRecord(ev[2], s));
   hx::hx_best_kernel<<<h->n_traces + 1, 256, 0, s>>>(ba);
@@ -1233,8 +1241,9 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
   HX_CUDA(cudaGetDeviceProperties(&prop, dev));
   const int smem_per_block = hx::kWarpsPerBlock * ck.smem_per_warp;
   const bool generic = needs_generic(grid, ck, false, false, false);
-  const void* kfn = generic ? (const void*)hx::hx_sim_kernel : (const void*)hx::hx_sim_kernel_lean;
-  if ((rc = ensure_dyn_smem(generic, smem_per_block))) return rc;
+  const int kernel = sim_kernel_of(generic, ck);
+  const void* kfn = (const void*)kSimKernel[kernel];
+  if ((rc = ensure_dyn_smem(kernel, smem_per_block))) return rc;
   int bps = 0;
   HX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kfn, hx::kWarpsPerBlock * 32, smem_per_block));
   if (bps < 1) return fail(HX_ERR_CUDA, "simulation kernel does not fit on an SM");
@@ -1339,10 +1348,7 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
 
   hx::hx_prep_kernel<<<(unsigned)std::max<int64_t>(1, (nq + 255) / 256), 256, 0, s>>>(pa, ck);
   HX_CUDA(cudaGetLastError());
-  if (generic)
-    hx::hx_sim_kernel<<<(unsigned)blocks, hx::kWarpsPerBlock * 32, smem_per_block, s>>>(sa, ck);
-  else
-    hx::hx_sim_kernel_lean<<<(unsigned)blocks, hx::kWarpsPerBlock * 32, smem_per_block, s>>>(sa, ck);
+  kSimKernel[kernel]<<<(unsigned)blocks, hx::kWarpsPerBlock * 32, smem_per_block, s>>>(sa, ck);
   HX_CUDA(cudaGetLastError());
   hx::hx_best_kernel<<<2, 256, 0, s>>>(ba);
   HX_CUDA(cudaGetLastError());

@@ -21,14 +21,14 @@ namespace hx {
 constexpr int64_t kScale = 1000000;       // fixed point of alpha, gamma, slo_mult
 constexpr int64_t kUsPerS = 1000000;      // prefill throughput is per second
 constexpr int64_t kRewardCap = (int64_t(1) << 43) - 1;
-constexpr uint64_t kKeyInf = ~0ull;
-// Event keys (time << 7 | instance) stay below 2^46: every time is below 2^39.
-constexpr uint64_t kNoEvent = 1ull << 46;
-constexpr int64_t kTimeInf = INT64_MAX;
 constexpr int kWarpsPerBlock = 4;
 constexpr unsigned kFull = 0xffffffffu;
-constexpr uint64_t kArrivalTag = 64;      // event-key tag: after every instance
 constexpr int kFRows = 18;                // S, G/C with 0..15 corrections done, E
+
+// What a completion does: release the k calls from `next` on, end a chain of
+// the query (the last of its k chains releases `next`), end the query.
+enum { kDoneRelease = 0, kDoneChain = 1, kDoneQuery = 2 };
+constexpr int kDoneShift = 24;  // of the last four bytes as one word
 
 // One call as the simulator reads it: 64 bytes, 16-byte aligned.
 struct __align__(16) CallRec {
@@ -37,11 +37,12 @@ struct __align__(16) CallRec {
   int64_t deadline;   // query arrival + T_slo
   int64_t arrival;    // query arrival
   int32_t tbar;       // mean of est over the instances
-  int32_t next;       // S: unused; G/C: next correction's id, or ~(E's id) at chain end
+  int32_t next;       // S: G_0; G/C: the next correction, or E at the end of the chain
   int32_t qid;        // query index within the trace
-  uint8_t stage, u, k, fcode;  // stage, corrections done incl. this call (E: the query's
-                               // tenant), k of the query, row of the rest-of-path table:
-                               // S 0, G/C 1 + u, E 17
+  uint8_t k, u, fcode, done;  // calls that its completion releases, or at a chain's end the
+                              // query's chains; corrections done incl. this call (E: the
+                              // query's tenant); row of the rest-of-path table: S 0, G/C 1 + u,
+                              // E 17; what its completion does (kDone*)
 };
 static_assert(sizeof(CallRec) == 64, "CallRec is one 64-byte unit");
 
@@ -64,12 +65,12 @@ struct ClusterK {
   int64_t slo_mult_fp;
   int32_t prefill[HX_MAX_TYPES], decode[HX_MAX_TYPES], slots[HX_MAX_TYPES], cnt[HX_MAX_TYPES];
   int32_t ref_prompt[4], ref_out[4];
-  int32_t total_slots;
+  int32_t slot_entries;     // slot entries per warp
   int32_t smem_per_warp;
   uint8_t inst_type[HX_MAX_INST];
   uint8_t inst_slots[HX_MAX_INST];
   uint16_t slot_base[HX_MAX_INST];
-  // tenants and faults (only the generic simulation kernel handles faults)
+  // tenants and faults (only hx_sim_kernel_faults handles faults)
   int32_t n_tenants, n_faults;
   int64_t tenant_mult[HX_MAX_TENANTS];
   int64_t timeout_mult_fp;
@@ -117,7 +118,7 @@ struct SimArgs {
   unsigned long long* work_counter;
   HeapEnt* arena;           // per resident warp: arena_per_warp entries
   int64_t arena_per_warp;
-  uint8_t* chains;          // per resident warp: chains_per_warp bytes
+  uint8_t* chains;          // per resident warp: chains_per_warp bytes (a multiple of 16)
   int64_t chains_per_warp;
   int64_t* topk;            // per resident warp: topk_per_warp latencies
   int64_t topk_per_warp;
@@ -137,50 +138,63 @@ struct SimArgs {
   int32_t checked;          // check the scheduler's invariants after every event (generic kernel)
 };
 
-// Per-warp shared memory of one simulation: per-instance local-queue and
-// slot state, per-simulation constants and lane-0 accumulators, then one
-// 64-bit (end << 24 | request id) key per batch slot of the cluster.  An
-// instance's running calls occupy the first cnt of its slots in ascending key
-// order, so the next completion on it is always its first slot.
-struct WarpShared {
-  int64_t q[HX_MAX_INST];       // t_queue: Eq. comp summed over requests dispatched and unfinished
-  uint64_t ekey[HX_MAX_INST];   // next completion event key per instance
-  int32_t erid[HX_MAX_INST];    // its request id
-  int32_t hoff[HX_MAX_INST];    // local queue: heap offset in the arena
-  int32_t hsize[HX_MAX_INST];   //              heap size
-  uint8_t cnt[HX_MAX_INST];     // running calls (the first cnt of the instance's slot keys)
-  uint8_t hcl[HX_MAX_INST];     // local queue: heap capacity 8 << hcl (0: none yet)
-  // this event's dispatches in order: (request id, service time), Eq. (comp) on the winner
-  int2 prs[HX_MAX_K];
-  int32_t pest[HX_MAX_K];
-  // per-simulation constants
-  int32_t A, one_minus_a;        // alpha and 1 - alpha, fixed point
-  int64_t G, beta;
+// A running call in its batch slot: end time and request id << 8 | slot.
+struct __align__(8) Slot32 {
+  uint32_t end, tag;
+};
+struct __align__(16) Slot64 {
+  uint64_t end;
+  uint32_t tag, fail;           // fail: the attempt times out at `end`
+};
+
+// One instance as every lane reads it (one 16-byte load).  Its t_queue and next
+// completion are in its owner lane's registers.
+struct __align__(16) InstState {
+  uint32_t free;                // free batch slots, one bit each
+  int32_t hsize;                // local queue: heap size
+  uint32_t heap;                // local queue: heap offset in the arena, capacity code << 27
+                                // (8 << code entries; 0: none yet)
+  uint32_t cfg;                 // its slots' mask, first slot << 16
+};
+constexpr int kHeapCodeShift = 27;  // the arena holds at most 4 * 2^24 + 1024 entries
+constexpr uint32_t kHeapOffMask = (1u << kHeapCodeShift) - 1;
+
+// Per-warp shared memory of one simulation: per-simulation constants and
+// warp-uniform state, then an InstState per lane and instance of it and the
+// slot entries: an instance's are read 16 at a time, so up to 32 instances have
+// 16 each; more have their own slots only, and 16 entries follow the last.
+struct __align__(16) WarpShared {
+  int4 pend[HX_MAX_K];          // this event's waiting dispatches: request id, service time and
+                                // Eq. (comp) on the instance, instance
+  uint4 dterm[16];              // digest terms waiting to be hashed: 32 of (relative time, id
+                                // tag), with 64-bit times 16
   longlong2 tie;                // t_queue up to which the least cost alone decides a dispatch; cost mask
   float4 fscore;                // the score filter's constants (score_range)
+  // per-simulation constants
+  int64_t G, beta;
   int64_t frest[kFRows];        // rest-of-path cost of the budget denominator by fcode
-  int32_t lpol, dpol, recj, kcap, rr, bump;
+  int32_t A, one_minus_a;       // alpha and 1 - alpha, fixed point
+  int32_t lpol, kcap, rr, bump;
   // this warp's scratch slices and the current trace's offsets
   HeapEnt* arena;
-  uint8_t* chains;
+  uint8_t* chains;              // finished chains per query
   int64_t* topk;
   int64_t qb, cb;
   int32_t nq, nc;
   int64_t sim, clk0;            // result index and start clock of the simulation
-  uint64_t akey;                // next arrival's event key (written alike by every lane)
-  int32_t qa, trace;            // arrivals taken so far (likewise); the simulation's trace
-  // lane-0 accumulators
+  int64_t base;                 // what the 32-bit event times are relative to (written alike by every lane)
+  int64_t next_arrival;         // time of the next arrival (likewise)
+  int32_t arrivals, trace;      // arrivals taken so far (likewise); the simulation's trace
   uint64_t digest;
   int64_t makespan;
-  int32_t n_done, slo_met, events, tk;
+  int32_t n_done, slo_met, pad, tk;
   int64_t tkmin;                // root of the full top-K heap (written alike by every lane)
-  longlong2 dterm[16];          // digest terms waiting to be hashed: (time, id tag)
   int32_t tslo[HX_MAX_TENANTS], tdone[HX_MAX_TENANTS];  // per-tenant counts (generic kernel)
   int32_t ttk[HX_MAX_TENANTS];  // per-tenant top-K heaps: entries (generic kernel with tenants)
   int64_t ttkmin[HX_MAX_TENANTS];  //                 and roots once full
   int32_t reissued, excl;       // timed-out attempts; the instance a re-issue avoids (-1: none)
-  uint64_t slot[1];             // [total_slots], then with faults one fail flag byte per slot
 };
+static_assert(sizeof(WarpShared) % 16 == 0, "InstState follows");
 
 struct BestCand {
   int64_t p95;
@@ -200,11 +214,16 @@ struct BestArgs {
 };
 
 __global__ void hx_prep_kernel(PrepArgs a, ClusterK c);
-// hx_sim_kernel: any mix of dispatch and local-queue policies and per-call
-// logs; hx_sim_kernel_lean: every point workload-balanced with the urgency
-// queue, nothing logged (the same simulation with those branches removed).
-__global__ void hx_sim_kernel(SimArgs a, ClusterK c);
+// hx_sim_kernel_lean: every point workload-balanced with the urgency queue,
+// nothing logged; hx_sim_kernel: any mix of dispatch and local-queue policies,
+// tenants and per-call logs; hx_sim_kernel_faults: those with fault windows.
+// Each for clusters of up to 64 instances, two a lane, and of up to 32, one a lane.
 __global__ void hx_sim_kernel_lean(SimArgs a, ClusterK c);
+__global__ void hx_sim_kernel_lean32(SimArgs a, ClusterK c);
+__global__ void hx_sim_kernel(SimArgs a, ClusterK c);
+__global__ void hx_sim_kernel32(SimArgs a, ClusterK c);
+__global__ void hx_sim_kernel_faults(SimArgs a, ClusterK c);
+__global__ void hx_sim_kernel_faults32(SimArgs a, ClusterK c);
 __global__ void hx_best_kernel(BestArgs a);
 __global__ void hx_selftest_div_kernel(const uint64_t* n, const uint64_t* d, uint64_t* q, uint64_t* q_ref,
                                        int64_t count);

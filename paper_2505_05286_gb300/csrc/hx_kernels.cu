@@ -236,16 +236,18 @@ __global__ void __launch_bounds__(256) hx_prep_kernel(PrepArgs a, ClusterK c) {
     r.deadline = deadline;
     r.arrival = arr;
     r.qid = qid;
-    r.stage = (uint8_t)st;
-    r.k = (uint8_t)k;
     if (st == HX_STAGE_S) {
       r.u = 0;
       r.fcode = 0;
-      r.next = -1;
+      r.done = kDoneRelease;
+      r.next = (int32_t)(j + 1 - cbase);
+      r.k = (uint8_t)k;
     } else if (st == HX_STAGE_E) {
       r.u = (uint8_t)tenant;
       r.fcode = kFRows - 1;
-      r.next = -1;
+      r.done = kDoneQuery;
+      r.next = 0;
+      r.k = 0;
     } else {
       const int cd = a.cand[j];
       int32_t nx;
@@ -256,7 +258,9 @@ __global__ void __launch_bounds__(256) hx_prep_kernel(PrepArgs a, ClusterK c) {
         r.u = a.retry[j];
         nx = (j + 1 < e - 1 && a.stage[j + 1] == HX_STAGE_C && a.cand[j + 1] == cd) ? (int32_t)(j + 1 - cbase) : -1;
       }
-      r.next = nx >= 0 ? nx : ~e_rid;
+      r.done = nx >= 0 ? kDoneRelease : kDoneChain;
+      r.next = nx >= 0 ? nx : e_rid;
+      r.k = (uint8_t)(nx >= 0 ? 1 : k);
       r.fcode = (uint8_t)(1 + r.u);
     }
     const int4* src = reinterpret_cast<const int4*>(&r);
@@ -271,23 +275,64 @@ __global__ void __launch_bounds__(256) hx_prep_kernel(PrepArgs a, ClusterK c) {
 // -------------------------------------------------------- simulation kernel
 namespace {
 
-// The digest is a sum of terms, so they are hashed 16 at a time: every lane
-// calls with the same (t, tag); lane 0 appends it, and a full batch is hashed
-// one term per lane and summed into W->digest.
+// Event times of one simulation.  Without fault windows an attempt runs less
+// than 2^28 us, so 32 bits relative to a base (moved up every 2^31 us) order
+// the running calls and one 32-bit warp minimum finds the next completion;
+// with fault windows an attempt can outlast that and times are 64-bit, base 0.
+template <bool kWide>
+struct Times {
+  using T = uint32_t;
+  using Slot = Slot32;
+};
+template <>
+struct Times<true> {
+  using T = uint64_t;
+  using Slot = Slot64;
+};
+
+// Running calls complete by (end, request id); a tag is request id << 8 | slot.
+__device__ __forceinline__ bool before(uint32_t e0, uint32_t tag0, uint32_t e1, uint32_t tag1) {
+  return ((uint64_t)e0 << 32 | tag0) < ((uint64_t)e1 << 32 | tag1);
+}
+__device__ __forceinline__ bool before(uint64_t e0, uint32_t tag0, uint64_t e1, uint32_t tag1) {
+  return (e0 < e1) | ((e0 == e1) & (tag0 < tag1));
+}
+
+__device__ __forceinline__ uint32_t warp_min(uint32_t v) { return __reduce_min_sync(kFull, v); }
+__device__ __forceinline__ uint64_t warp_min(uint64_t v) { return warp_min_u64(v); }
+
+// The digest is a sum of terms, so they are hashed a batch at a time: every
+// lane calls with the same (t, tag) and stores the same pair; a full batch is
+// hashed one term per lane and summed into W->digest.
+template <bool kWide>
 __device__ __noinline__ void digest_flush(WarpShared* W, int n, int lane) {
   __syncwarp();
-  const longlong2 e = W->dterm[lane < n ? lane : 0];
-  uint64_t y = lane < n ? digest_term((uint64_t)e.x, (uint64_t)e.y) : 0ull;
+  uint64_t t, tag;
+  if (kWide) {
+    const ulonglong2 e = reinterpret_cast<const ulonglong2*>(W->dterm)[lane < n ? lane : 0];
+    t = e.x;
+    tag = e.y;
+  } else {
+    const uint2 e = reinterpret_cast<const uint2*>(W->dterm)[lane < n ? lane : 0];
+    t = (uint64_t)W->base + e.x;
+    tag = e.y;
+  }
+  uint64_t y = lane < n ? digest_term(t, tag) : 0ull;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(kFull, y, o);
   if (lane == 0) W->digest += y;
   __syncwarp();
 }
 
-__device__ __forceinline__ void digest_push(WarpShared* W, int& dn, int64_t t, uint32_t tag, int lane) {
-  W->dterm[dn] = make_longlong2(t, (long long)tag);  // every lane writes the same pair
-  if (++dn == 16) {
-    digest_flush(W, 16, lane);
+template <bool kWide, class T>
+__device__ __forceinline__ void digest_push(WarpShared* W, int& dn, T t, uint32_t tag, int lane) {
+  constexpr int kBatch = kWide ? 16 : 32;
+  if (kWide)
+    reinterpret_cast<ulonglong2*>(W->dterm)[dn] = make_ulonglong2(t, tag);
+  else
+    reinterpret_cast<uint2*>(W->dterm)[dn] = make_uint2((uint32_t)t, tag);
+  if (++dn == kBatch) {
+    digest_flush<kWide>(W, kBatch, lane);
     dn = 0;
   }
 }
@@ -410,9 +455,6 @@ __device__ __noinline__ void topk_insert_warp(int64_t* h, int32_t* size, int kca
   }
 }
 
-// Queue this event's dispatches to instance m (pending entries on the lanes of
-// mask pm) in m's heap, re-homing the heap in the arena when it is full.
-// All lanes call.  Returns HX_OK or HX_ERR_CAPACITY.
 __device__ __noinline__ int64_t budget_wide(int64_t num, int64_t tb, int64_t d) { return scaled_div(num, tb, d); }
 
 // t_slo of Eq. (budget): (deadline - now) * tbar / (tbar + F), truncated
@@ -425,36 +467,33 @@ __device__ __forceinline__ int64_t slo_budget(int64_t num, int64_t tb, int64_t d
   return budget_wide(num, tb, dd);
 }
 
-// Local-queue key, higher first, of pending entry j: Eq. (priority) with
-// the budget at send time (now) and the common now dropped; FCFS: earliest
+// Local-queue key, higher first, of a request dispatched now: Eq. (priority)
+// with the budget at send time (now) and the common now dropped; FCFS: earliest
 // enqueue; LLF: least deadline - now - remaining work, again with the common
-// now dropped.
-__device__ __forceinline__ long long pending_key(const WarpShared* W, const CallRec* rec, int64_t now, int lpol,
-                                                 int j) {
-  const CallRec* r = rec + W->prs[j].x;
+// now dropped.  est is its Eq. (comp) on the instance.
+__device__ __forceinline__ long long queue_key(const WarpShared* W, const CallRec* r, int est, int64_t now, int lpol) {
   const int64_t dl = r->deadline;
   const int4 tail = *reinterpret_cast<const int4*>(&r->tbar);
   const int64_t tb = tail.x;
-  const int64_t dd = tb + W->frest[(uint32_t)tail.w >> 24];
-  return lpol == HX_LOCAL_PQ     ? (long long)(kScale * ((int64_t)W->pest[j] - slo_budget(dl - now, tb, dd)) - W->G * now)
+  const int64_t dd = tb + W->frest[(tail.w >> 16) & 0xff];
+  return lpol == HX_LOCAL_PQ     ? (long long)(kScale * ((int64_t)est - slo_budget(dl - now, tb, dd)) - W->G * now)
          : lpol == HX_LOCAL_FCFS ? (long long)(-now)
                                  : (long long)(dd - dl);
 }
 
-// The instance's new requests (pending entries, bits of pm) join its local
-// queue, their keys formed one per lane.
-__device__ __forceinline__ int push_pending(WarpShared* W, const CallRec* rec, int64_t now, int lpol,
-                                        int64_t arena_per_warp, int m, unsigned pm, int lane) {
-  const long long key = ((pm >> lane) & 1u) ? pending_key(W, rec, now, lpol, lane) : 0;
+// The instance's new requests (this lane's: p, its key: key; on the lanes of
+// pm) join its local queue, which moves to a region of twice the size when it
+// is full.  All lanes call.  Returns HX_OK or HX_ERR_CAPACITY.
+__device__ __forceinline__ int push_pending(WarpShared* W, InstState* I, int4 p, long long key, unsigned pm,
+                                            int64_t arena_per_warp, int lane) {
   HeapEnt* const arena = W->arena;
   while (pm) {
     const int j = __ffs(pm) - 1;
     pm &= pm - 1;
-    const long long kj = __shfl_sync(kFull, key, j);
-    const int2 rs = W->prs[j];
-    const int rid = rs.x, svc = rs.y;
-    const int size = W->hsize[m], hcl = W->hcl[m], off = W->hoff[m], bump = W->bump;
-    const int cap = hcl ? 8 << hcl : 0;
+    const int size = I->hsize;
+    const uint32_t heap = I->heap;
+    const int hcl = (int)(heap >> kHeapCodeShift), cap = hcl ? 8 << hcl : 0, bump = W->bump;
+    const int off = (int)(heap & kHeapOffMask);
     __syncwarp();
     int hoff = off;
     if (size == cap) {
@@ -463,68 +502,41 @@ __device__ __forceinline__ int push_pending(WarpShared* W, const CallRec* rec, i
       hoff = bump;
       for (int i = lane; i < size; i += 32) arena[hoff + i] = arena[off + i];
       __syncwarp();
-      if (lane == 0) {
-        W->bump = bump + ncap;
-        W->hoff[m] = hoff;
-        W->hcl[m] = (uint8_t)(hcl + 1);
-      }
+      W->bump = bump + ncap;  // every lane writes the same values
+      I->heap = (uint32_t)hoff | (uint32_t)(hcl + 1) << kHeapCodeShift;
     }
-    if (lane == 0) {
-      heap_push(arena + hoff, size, kj, rid, svc);
-      W->hsize[m] = size + 1;
-    }
+    if (lane == j) heap_push(arena + hoff, size, key, p.x, p.y);
+    I->hsize = size + 1;
     __syncwarp();
   }
   return HX_OK;
 }
 
-// One new request (the single bit of pm) meets an instance with one free slot
-// and a non-empty local queue: the more urgent of it and the queue's top
-// starts and the other waits, i.e. a push and a pop in one sift (the new
-// request replaces the top).  Returns the started (request id, service time).
-__device__ __forceinline__ int2 push_pop(WarpShared* W, const CallRec* rec, int64_t now, int lpol, int m, unsigned pm,
-                                     int lane) {
-  const int j = __ffs(pm) - 1;
-  const long long key = pending_key(W, rec, now, lpol, j);  // the same on every lane
-  const int2 rs = W->prs[j];
-  HeapEnt* const h = W->arena + W->hoff[m];
-  const HeapEnt top = h[0];
-  if (ent_better(key, rs.x, top.key, top.rid)) return rs;
-  HeapEnt e;
-  e.key = key;
-  e.rid = rs.x;
-  e.svc = rs.y;
-  heap_sift_warp(h, W->hsize[m], e, lane);
-  return make_int2(top.rid, top.svc);
-}
-
 // The dispatch winner from exact scores, for the dispatches whose float bounds
 // overlap: highest score, ties to the lowest instance.  All lanes call.
+template <int J>
 __device__ __noinline__ int exact_winner(const WarpShared* W, int64_t q0, int64_t q1, int e0, int e1, bool ok0, bool ok1,
                                          int lane) {
   const uint64_t beta = (uint64_t)W->beta;
   const float betaf = u64_to_float(beta);
   const int64_t A = W->A, oma = W->one_minus_a;
   const uint64_t r0 = udiv_trial_f(beta, betaf, q0 > 1 ? (uint64_t)q0 : 1ull);
-  const uint64_t r1 = udiv_trial_f(beta, betaf, q1 > 1 ? (uint64_t)q1 : 1ull);
   const int64_t s0 = ok0 ? oma * (int64_t)(r0 < (uint64_t)kRewardCap ? r0 : kRewardCap) - A * e0 : INT64_MIN;
+  if (J == 1) return warp_argmax_s64(s0, lane);
+  const uint64_t r1 = udiv_trial_f(beta, betaf, q1 > 1 ? (uint64_t)q1 : 1ull);
   const int64_t s1 = ok1 ? oma * (int64_t)(r1 < (uint64_t)kRewardCap ? r1 : kRewardCap) - A * e1 : INT64_MIN;
   const bool take1 = s1 > s0;
   return warp_argmax_s64(take1 ? s1 : s0, take1 ? lane + 32 : lane);
 }
 
 // All lanes: a query's evaluation call finished at `now` (Sec. 4.3's metrics).
-__device__ __forceinline__ void finish_query(WarpShared* W, int& dn, int32_t qid, int64_t now, int64_t arrival,
-                                            int64_t deadline, int lane) {
-  {
-    // every lane reads the counters, then every lane writes the same new values
-    const int32_t slo = W->slo_met + (now <= deadline ? 1 : 0), nd = W->n_done + 1;
-    __syncwarp();
-    W->slo_met = slo;
-    W->n_done = nd;
-    W->makespan = now;
-  }
-  digest_push(W, dn, now, query_tag(qid), lane);
+__device__ __forceinline__ void finish_query(WarpShared* W, int64_t now, int64_t arrival, int64_t deadline, int lane) {
+  // every lane reads the counters, then every lane writes the same new values
+  const int32_t slo = W->slo_met + (now <= deadline ? 1 : 0), nd = W->n_done + 1;
+  __syncwarp();
+  W->slo_met = slo;
+  W->n_done = nd;
+  W->makespan = now;
   // most latencies of a full heap fall below its root and change nothing
   const int64_t v = now - arrival;
   if (W->tk < W->kcap || v > W->tkmin) topk_insert_warp(W->topk, &W->tk, W->kcap, &W->tkmin, v, lane);
@@ -537,17 +549,19 @@ __device__ __noinline__ void log_dispatch(const SimArgs& a, int recj, int rid, i
   a.rec_budget[o] = budget;
 }
 
-
 }  // namespace
 
-// Resident blocks per SM the register allocation aims for (4 warps each).
+// Resident blocks per SM the register allocation aims for (4 warps each): 8
+// with one instance per lane; with two, 7, whose 72 registers hold a
+// simulation's state without spills (8 spill 48 bytes in the event loop: 8
+// traces x 20000 queries x 1024 points 503 ms against 458 ms).
 #ifndef HX_SIM_MIN_BLOCKS
-#define HX_SIM_MIN_BLOCKS 8
+#define HX_SIM_MIN_BLOCKS(J) ((J) == 1 ? 8 : 7)
 #endif
 
 // Bounds-checked build (-DHX_CHECKED): before every shared- or global-memory
 // access whose index the simulation forms from its own state (instance,
-// request id, query id, slot count, heap offset and size, top-K size), the
+// request id, query id, slot, heap offset and size, top-K size), the
 // index is range-checked; a failed check sets the simulation's status to
 // HX_ERR_BOUNDS and leaves the loop it is in instead of making the access,
 // and the simulation stops after that event.  Every checked value is the
@@ -566,12 +580,35 @@ __device__ __noinline__ void log_dispatch(const SimArgs& a, int recj, int rid, i
 #define HX_STOP_IF_FAILED()
 #endif
 
-template <bool kGeneric>
+// One warp, one simulation.  J instances per lane: lane l owns l and, with J = 2,
+// l + 32.
+//
+// An event is a chain of dependent warp instructions, and their number bounds
+// both a lone simulation (5 to 7 cycles per instruction) and a full GPU (issue
+// slots 80 to 85 % busy).  So the state that only scores and the next event need
+// stays in the owner lane's registers, where an update is a select; event times
+// are 32-bit, so one warp reduction finds the next completion; running calls sit
+// unsorted in their slots under a free mask, so a start is one store and one
+// comparison, and a completion one reduction over the instance's slots; and up
+// to 32 instances take one lane each (half the per-lane work).  Against sorted
+// 64-bit slot keys and per-instance arrays in shared memory: 342 -> 178
+// warp-instructions per call event (8 traces x 2000 queries x 64 points, 8
+// instances: 14.2 -> 10.9 ms); 32 instances, 19 x 5003 x 512: 127 -> 89 ms; 64
+// instances, 8 x 20000 x 1024: 529 -> 460 ms.
+template <int J, bool kGeneric, bool kFaults>
 __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
+  using T = typename Times<kFaults>::T;
+  using Slot = typename Times<kFaults>::Slot;
+  constexpr T kIdle = ~T(0);                      // no running call; no arrival in range
+  constexpr T kFar = kFaults ? kIdle : T(1) << 31;  // an event this far moves the base up first
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
+  // volatile: read once and kept, not read again wherever it is used
+  int lane;
+  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
   WarpShared* const W = reinterpret_cast<WarpShared*>(smem_raw + warp * c.smem_per_warp);
+  InstState* const inst = reinterpret_cast<InstState*>(W + 1);
+  Slot* const slots = reinterpret_cast<Slot*>(inst + 32 * J);
   if (lane == 0) {
     // this warp's slices of the scratch arrays (kept in shared memory to spare registers)
     const int64_t gw = (int64_t)blockIdx.x * kWarpsPerBlock + warp;
@@ -580,10 +617,12 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     W->topk = a.topk + gw * a.topk_per_warp;
   }
   const int N = c.n_inst;
-  const int m0 = lane, m1 = lane + 32;
-  const bool valid0 = m0 < N, valid1 = m1 < N;
-  const int ty0 = valid0 ? c.inst_type[m0] : 0;
-  const int ty1 = valid1 ? c.inst_type[m1] : 0;
+  // an instance's slots are read one per lane of the lower half warp
+  const int l16 = lane & 15;
+  const uint32_t lbit = lane < 16 ? 1u << lane : 0u;
+  uint32_t lrec[J];  // byte offset of this lane's type in a call record
+#pragma unroll
+  for (int j = 0; j < J; ++j) lrec[j] = lane + 32 * j < N ? 8u * c.inst_type[lane + 32 * j] : 0u;
 
   for (;;) {
     unsigned long long work = 0;
@@ -621,14 +660,14 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
 
     // per-instance state that every lane reads later: written before the
     // barrier below
-    for (int m = lane; m < 64; m += 32) {
-      W->q[m] = m < N ? 0 : INT64_MAX;
-      W->hoff[m] = 0;
-      W->hcl[m] = 0;
-      W->hsize[m] = 0;
-      W->cnt[m] = 0;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const int m = lane + 32 * j;
+      const uint32_t mask = m < N ? (1u << c.inst_slots[m]) - 1 : 0u;
+      inst[m] = InstState{mask, 0, 0u, mask | (m < N ? (uint32_t)c.slot_base[m] << 16 : 0u)};
     }
-    for (int j = lane; j < c.total_slots; j += 32) W->slot[j] = kKeyInf;
+    // no chain of any query has finished
+    for (int i = 16 * lane; i < nq; i += 512) *reinterpret_cast<uint4*>(W->chains + i) = make_uint4(0, 0, 0, 0);
     if (lane < kFRows) {
       // rest of the request's own path after it (the budget denominator minus
       // its own mean cost): stage reference costs, i.e. means over instances of
@@ -668,8 +707,6 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       const bool idle_top = oma * (reward_of(beta, 1) - reward_of(beta, 2)) > A << 28;
       W->tie = make_longlong2(A == kScale ? INT64_MAX - 1 : idle_top ? 1 : -1, A != 0 ? 0xffffffffll : 0ll);
       W->lpol = a.lpol[p];
-      W->dpol = a.dpol[p];
-      W->recj = a.rec_map ? a.rec_map[sim] : -1;
       W->kcap = nq - (95 * nq + 99) / 100 + 1;
       W->rr = 0;
       W->bump = 0;
@@ -677,7 +714,6 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       W->makespan = 0;
       W->n_done = 0;
       W->slo_met = 0;
-      W->events = 0;
       W->tk = 0;
       W->tkmin = 0;
       for (int t = 0; t < HX_MAX_TENANTS; ++t) {
@@ -691,26 +727,42 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     }
     __syncwarp();
 
-    // this lane's instances m0 = lane and m1 = lane + 32: t_queue in W->q[m]
-    // and the next completion's event key and request id in W->ekey[m] and
-    // W->erid[m] (every change stored alike by every lane; the owner reads
-    // its own); shared memory rather than registers leaves the allocator room.
-    // -alpha as the score filter's cost weight; -inf keeps instances past N out of it
-    const float neg_a0 = valid0 ? -(float)W->A : -INFINITY;
-    const float neg_a1 = valid1 ? -(float)W->A : -INFINITY;
-    W->ekey[m0] = kKeyInf;
-    W->ekey[m1] = kKeyInf;
-    // this event's dispatches, entry j on lane j
-    int pend_m = -1;
+    // What this lane keeps of its instances, in registers: t_queue, the end of
+    // the next completion (kIdle: nothing runs) and its tag (request id << 8 |
+    // slot).  An instance past N has t_queue INT64_MAX and cost weight -inf in the
+    // score filter, and never wins.
+    int64_t q[J];
+    T next_end[J];
+    uint32_t next_tag[J];
+    float neg_a[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const bool on = lane + 32 * j < N;
+      q[j] = on ? 0 : INT64_MAX;
+      next_end[j] = kIdle;
+      next_tag[j] = 0;
+      neg_a[j] = on ? -(float)W->A : -INFINITY;
+    }
 
-    W->qa = 0;
-    W->akey = nq > 0 ? (((uint64_t)a.arrival[qb] << 7) | kArrivalTag) : kKeyInf;
-    int64_t now = 0;
+    // the record slot of a logged simulation, or -1; the dispatch policy
+    const int recj = kGeneric && a.rec_map ? a.rec_map[sim] : -1;
+    const bool round_robin = kGeneric && a.dpol[p] == HX_DISPATCH_RR;
+
+    // times are relative to base; an arrival 2^32 us or more past it reads as kIdle
+    W->base = 0;
+    auto rel = [&](int64_t t_abs) -> T {
+      if (kFaults) return (T)t_abs;
+      const uint64_t d = (uint64_t)(t_abs - W->base);
+      return (d >> 32) ? kIdle : (T)d;
+    };
+    auto absolute = [&](T t) -> int64_t { return kFaults ? (int64_t)t : W->base + (int64_t)t; };
+    W->arrivals = 0;
+    W->next_arrival = nq > 0 ? a.arrival[qb] : 0;
+    T arr = nq > 0 ? rel(a.arrival[qb]) : kIdle;
+    T now = 0;
     int32_t status = HX_OK, npend = 0;
-    uint64_t touched = 0;
     // event bound; re-issued attempts add events while fault windows last
-    const bool faults = kGeneric && c.n_faults > 0;
-    int32_t steps_left = nc + nq + 8 + (faults ? 16 * nc + 4096 : 0);
+    int32_t steps_left = nc + nq + 8 + (kFaults ? 16 * nc + 4096 : 0);
 #ifdef HX_CHECKED
     // the warp's scratch slices must hold this trace's chain counters and top-K
     if (!(nq <= a.chains_per_warp && W->kcap <= a.topk_per_warp && (a.tenant_kcap == nullptr ||
@@ -718,345 +770,396 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       status = HX_ERR_BOUNDS;
 #endif
 
-    // Request rid starts on instance m now and runs until now + svc: its key
-    // joins the cn sorted keys of m's running calls at sl.
+    // one instance per lane: 16 slot entries each, so that no load gives the first
+    auto first_slot = [&](int m, const InstState& I) -> uint32_t { return J == 1 ? 16u * m : I.cfg >> 16; };
+    // Request rid starts on instance m now in the highest of its free slots;
+    // svc is its service time on m (on m's lane at least).  The slots stay
+    // unsorted: a start is one store and a comparison with the instance's next
+    // completion.  Returns the remaining free slots.
     int dn = 0;  // digest terms waiting in W->dterm
-    auto start_call = [&](uint64_t* sl, int m, int cn, int rid, int svc) {
-      int64_t run = svc;
+    auto start_call = [&](int m, uint32_t free, uint32_t slot_base, int rid, int svc) -> uint32_t {
+      T run = (T)svc;
       bool fail = false;
-      if (faults) {
+      if (kFaults) {
         // the first fault window of m that covers now, and the timeout (Sec. 3.3)
+        int64_t r64 = svc;
         bool in_window = false, down = false;
         for (int f = 0; f < c.n_faults; ++f) {
           const FaultK& F = c.faults[f];
-          if (F.inst == m && now >= F.t0 && now < F.t1) {
+          if (F.inst == m && (int64_t)now >= F.t0 && (int64_t)now < F.t1) {
             in_window = true;
             if (F.slow == 0) down = true;
-            else run = (run * F.slow + kScale - 1) / kScale;
+            else r64 = (r64 * F.slow + kScale - 1) / kScale;
             break;
           }
         }
         if (in_window && c.timeout_mult_fp > 0) {
           const int64_t timeout = ((int64_t)rec[rid].ev[c.inst_type[m]].x * c.timeout_mult_fp) / kScale;
-          if (down || run > timeout) {
+          if (down || r64 > timeout) {
             fail = true;
-            run = timeout;
+            r64 = timeout;
           }
         }
+        run = (T)r64;
       }
-      const uint64_t nk = ((uint64_t)(now + run) << 24) | (uint64_t)(uint32_t)rid;
-      const uint64_t cur = lane < cn ? sl[lane] : kKeyInf;
-      uint8_t* const fl = faults ? reinterpret_cast<uint8_t*>(W->slot + c.total_slots) + (sl - W->slot) : nullptr;
-      const uint8_t fcur = (faults && lane < cn) ? fl[lane] : 0;
-      const int pos = __popc(__ballot_sync(kFull, cur < nk));
-      if (lane >= pos && lane < cn) sl[lane + 1] = cur;
-      if (lane == pos) sl[pos] = nk;
-      if (faults) {
-        if (lane >= pos && lane < cn) fl[lane + 1] = fcur;
-        if (lane == pos) fl[pos] = fail ? 1 : 0;
-      }
-      digest_push(W, dn, now, call_tag(rid, m), lane);
-      if (kGeneric && lane == 0) {
-        const int recj = W->recj;
-        if (recj >= 0) {
-          a.rec_start[(int64_t)recj * a.rec_stride + rid] = now;
-          a.rec_end[(int64_t)recj * a.rec_stride + rid] = now + run;
+      const int s = 31 - __clz(free);
+      const uint32_t tag = (uint32_t)rid << 8 | (uint32_t)s;
+      const T end = now + run;
+      if (lane == (m & 31)) {
+        Slot e;
+        e.end = end;
+        e.tag = tag;
+        if constexpr (kFaults) e.fail = fail ? 1u : 0u;
+        slots[slot_base + s] = e;
+        if (kGeneric && recj >= 0) {
+          a.rec_start[(int64_t)recj * a.rec_stride + rid] = absolute(now);
+          a.rec_end[(int64_t)recj * a.rec_stride + rid] = absolute(end);
         }
       }
-      __syncwarp();
-    };
-
-    auto set_key = [&](int m, uint64_t nk) {
-      // an empty instance (nk all ones) maps to a key at or above kNoEvent
-      W->ekey[m] = ((nk >> 24) << 7) | (uint64_t)m;  // every lane stores the same key
-      W->erid[m] = (int32_t)(nk & 0xffffffull);
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        // the lowest request id completes first among equal ends
+        const bool first = (lane + 32 * j == m) & before(end, tag, next_end[j], next_tag[j]);
+        next_end[j] = first ? end : next_end[j];
+        next_tag[j] = first ? tag : next_tag[j];
+      }
+      free ^= 1u << s;
+      inst[m].free = free;  // every lane stores the same mask
+      digest_push<kFaults>(W, dn, now, call_tag(rid, m), lane);
+      return free;
     };
 
     for (;;) {
       HX_STOP_IF_FAILED()
-      const uint64_t k0 = W->ekey[m0], k1 = W->ekey[m1];
-      const uint64_t ck = warp_min_u64(k0 < k1 ? k0 : k1);
-      const uint64_t akey = W->akey;
-      if (ck >= kNoEvent && akey == kKeyInf) break;
-      if (--steps_left < 0) {
-        status = HX_ERR_STEP_LIMIT;
-        break;
+      __syncwarp();
+      const T mn = warp_min(J == 2 && next_end[J - 1] < next_end[0] ? next_end[J - 1] : next_end[0]);
+      if (((mn < arr ? mn : arr) >= kFar) | (steps_left == 0)) {
+        // the end, too many events, or nothing within 2^31 us of the base, which
+        // then moves to the next event
+        const bool more = W->arrivals < nq;
+        if (mn == kIdle && !more) break;
+        if (steps_left-- == 0) {
+          status = HX_ERR_STEP_LIMIT;
+          break;
+        }
+        ++steps_left;
+        if (!kFaults) {
+          digest_flush<kFaults>(W, dn, lane);
+          dn = 0;
+          const int64_t base = W->base, at = W->next_arrival;
+          int64_t nb = mn == kIdle ? at : base + (int64_t)mn;
+          if (more && at < nb) nb = at;
+          const T shift = (T)(nb - base);
+#pragma unroll
+          for (int j = 0; j < J; ++j) next_end[j] = next_end[j] == kIdle ? kIdle : next_end[j] - shift;
+          for (int j = lane; j < c.slot_entries; j += 32) slots[j].end -= shift;
+          __syncwarp();
+          W->base = nb;  // every lane writes the same value
+          arr = more ? rel(at) : kIdle;
+          continue;
+        }
       }
-      touched = 0;
+      --steps_left;
       npend = 0;
+      int cm = 0, waiting = 0;  // the instance whose slot this event frees, and the requests waiting for it
       // requests released by this event: rel_first .. rel_first + rel_count - 1
       int32_t rel_first = 0, rel_count = 0;
-      if (ck < akey) {
-        // completion on instance m
-        const int m = (int)(ck & 127ull);
-        now = (int64_t)(ck >> 7);
-        HX_BOUND(m < N)
-        uint64_t* const sl = W->slot + c.slot_base[m];
-        const int cn = W->cnt[m];
-        HX_BOUND(cn >= 1 && cn <= c.inst_slots[m] && c.slot_base[m] + cn <= c.total_slots)
-        // the finishing call heads m's sorted slots; its id is kept beside
-        // m's event key, so that its record load need not wait for the slot
-        const int32_t rid = W->erid[m];
+      if (mn <= arr) {
+        // completion on the lowest instance that has one at mn
+        now = mn;
+        const unsigned b0 = __ballot_sync(kFull, next_end[0] == mn);
+        const unsigned b1 = J == 2 ? __ballot_sync(kFull, next_end[J - 1] == mn) : 0u;
+        const bool low = J == 1 || b0 != 0;
+        const int ml = __ffs(low ? b0 : b1) - 1, m = low ? ml : ml + 32;
+        HX_BOUND(ml >= 0 && m < N)
+        const uint32_t tag = __shfl_sync(kFull, low ? next_tag[0] : next_tag[J - 1], ml);
+        const int32_t rid = (int32_t)(tag >> 8);
+        const int hole = (int)(tag & 0xffu);
         HX_BOUND(rid < nc)
-        // the finished call's record: issued now, used after the slot shift
-        const CallRec* r = rec + rid;
+        const CallRec* const r = rec + rid;
         const int4 tail = *reinterpret_cast<const int4*>(&r->tbar);
-        const int64_t est_m = r->ev[c.inst_type[m]].x;
-        const int hs_m = W->hsize[m];
-        // remove it: the remaining keys move down one slot
-        const uint64_t nxt = lane + 1 < cn ? sl[lane + 1] : kKeyInf;
-        const uint64_t head = cn > 1 ? sl[1] : kKeyInf;
-        uint8_t* const fl = faults ? reinterpret_cast<uint8_t*>(W->slot + c.total_slots) + (sl - W->slot) : nullptr;
-        const bool failed = faults && fl[0] != 0;
-        const uint8_t fnxt = (faults && lane + 1 < cn) ? fl[lane + 1] : 0;
-        __syncwarp();
-        if (lane < cn) sl[lane] = nxt;
-        if (faults && lane < cn) fl[lane] = fnxt;
-        W->cnt[m] = cn - 1;  // every lane writes the same count
-        set_key(m, head);
-        {
-          W->q[m] = W->q[m] - est_m;  // every lane stores the same value
+        const int est = *reinterpret_cast<const int*>(reinterpret_cast<const char*>(r) + (low ? lrec[0] : lrec[J - 1]));
+        const InstState I = inst[m];
+        const uint32_t slot_base = first_slot(m, I);
+        HX_BOUND((int)slot_base + 16 <= c.slot_entries && hole < 16 && ((I.cfg & ~I.free) >> hole & 1u))
+        // the slot is free; the next completion is the earliest of those still running
+        const uint32_t free = I.free | 1u << hole;
+        const bool failed = kFaults && reinterpret_cast<const Slot64*>(slots)[slot_base + hole].fail != 0;
+        const Slot e = slots[slot_base + l16];
+        const bool runs = (I.cfg & ~free & 0xffffu & lbit) != 0;
+        const T nmin = warp_min(runs ? e.end : kIdle);
+        unsigned nb = __ballot_sync(kFull, runs & (e.end == nmin));
+        if (nb & (nb - 1)) {
+          // equal ends: the lowest request id
+          const uint32_t id = runs & (e.end == nmin) ? e.tag : 0xffffffffu;
+          nb = __ballot_sync(kFull, id == __reduce_min_sync(kFull, id));
+        }
+        const uint32_t ntag = __shfl_sync(kFull, e.tag, 31 - __clz(nb));
+        inst[m].free = free;  // every lane stores the same mask
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+          const bool own = lane + 32 * j == m;
+          next_end[j] = own ? nmin : next_end[j];
+          next_tag[j] = own ? ntag : next_tag[j];
+          q[j] -= own ? est : 0;
         }
         // the freed slot needs a batch boundary only if requests wait for it
-        if (hs_m > 0) touched |= 1ull << m;
-        const int stg = tail.w & 0xff;
+        cm = m;
+        waiting = I.hsize;
+        const uint32_t what = (uint32_t)tail.w >> kDoneShift;
         const int32_t qid = tail.z;
         HX_BOUND(qid >= 0 && qid < nq)
-        if (faults && failed) {
+        if (kFaults && failed) {
           // the attempt timed out: the request goes out again, avoiding m
-          if (lane == 0) W->reissued++;
+          const int32_t n = W->reissued + 1;
+          __syncwarp();
+          W->reissued = n;
           W->excl = c.n_inst > 1 ? m : -1;
           rel_first = rid;
           rel_count = 1;
-        } else if (stg == HX_STAGE_S) {
-          const int k = (tail.w >> 16) & 0xff;
-          HX_BOUND(k >= 1 && k <= HX_MAX_K && rid + k < nc)
-          W->chains[qid] = (uint8_t)k;  // every lane writes the same byte
-          rel_first = rid + 1;
-          rel_count = k;
-        } else if (stg == HX_STAGE_E) {
-          const int64_t dl = r->deadline;
-          const int64_t arr = r->arrival;
+        } else if (what == kDoneRelease) {
+          rel_first = tail.y;
+          rel_count = tail.w & 0xff;
+        } else if (what == kDoneChain) {
+          // a chain of the query ended: the last one releases the evaluation
+          uint8_t* const chains = W->chains + qid;
+          const int ended = *chains + 1;
+          __syncwarp();
+          *chains = (uint8_t)ended;  // every lane writes the same byte
+          rel_first = tail.y;
+          rel_count = ended == (tail.w & 0xff) ? 1 : 0;
+        } else {
+          const int64_t t_abs = absolute(now), dl = r->deadline, at = r->arrival;
           if (kGeneric) {
             const int ten = (tail.w >> 8) & 0xff;
             HX_BOUND(ten < HX_MAX_TENANTS)
             if (lane == 0) {
               W->tdone[ten]++;
-              W->tslo[ten] += now <= dl ? 1 : 0;
+              W->tslo[ten] += t_abs <= dl ? 1 : 0;
             }
             if (a.tenant_kcap) {
               // this tenant's own top-K, for its P95 (Sec. 5's per-tenant tail latency)
               const int kc = a.tenant_kcap[(int64_t)W->trace * HX_MAX_TENANTS + ten];
               HX_BOUND(W->trace < a.n_traces && kc <= a.tenant_topk_off[0])
-              const int64_t v = now - arr;
+              const int64_t v = t_abs - at;
               __syncwarp();
               if (W->ttk[ten] < kc || v > W->ttkmin[ten])
                 topk_insert_warp(W->topk + a.tenant_topk_off[ten], &W->ttk[ten], kc, &W->ttkmin[ten], v, lane);
             }
           }
-          finish_query(W, dn, qid, now, arr, dl, lane);
-        } else {
-          const int32_t nx = tail.y;
-          HX_BOUND(nx >= 0 ? nx < nc : ~nx < nc)
-          if (nx >= 0) {
-            rel_first = nx;
-            rel_count = 1;
-          } else {
-            uint8_t* const chains = W->chains;
-            const int left = chains[qid] - 1;
-            __syncwarp();
-            chains[qid] = (uint8_t)left;  // every lane writes the same byte
-            rel_first = ~nx;
-            rel_count = left == 0 ? 1 : 0;
-          }
+          digest_push<kFaults>(W, dn, now, query_tag(qid), lane);
+          finish_query(W, t_abs, at, dl, lane);
         }
+        HX_BOUND(rel_first >= 0 && rel_count <= HX_MAX_K && rel_first + rel_count <= nc)
       } else {
-        now = (int64_t)(akey >> 7);
+        now = arr;
         const int64_t qbase = W->qb;
-        const int32_t qa = W->qa;
+        const int32_t qa = W->arrivals;
         HX_BOUND(qa < W->nq)
         rel_first = (int32_t)(a.qcall[qbase + qa] - W->cb);
         HX_BOUND(rel_first >= 0 && rel_first < nc)
         rel_count = 1;
-        W->qa = qa + 1;
-        W->akey = qa + 1 < W->nq ? (((uint64_t)a.arrival[qbase + qa + 1] << 7) | kArrivalTag) : kKeyInf;
+        __syncwarp();
+        W->arrivals = qa + 1;  // every lane writes the same values
+        const int64_t at = qa + 1 < W->nq ? a.arrival[qbase + qa + 1] : 0;
+        W->next_arrival = at;
+        arr = qa + 1 < W->nq ? rel(at) : kIdle;
       }
 
       // Sec. 4.1 for each released request, in request-id order: score every
       // instance and send it to the winner (its Sec. 4.2 key is formed at the
       // batch boundary below, and only if it has to wait).
-      for (int32_t jr = 0; jr < rel_count; ++jr) {
-        const int32_t rid = rel_first + jr;
+      for (int32_t rid = rel_first; rel_count > 0; ++rid, --rel_count) {
         HX_BOUND(rid < nc)
-        const CallRec* r = rec + rid;
-        // Eq. (comp) and the service time on this lane's two instances
-        const int2 ev0 = r->ev[ty0], ev1 = r->ev[ty1];
-        const int e0 = ev0.x, e1 = ev1.x, v0 = ev0.y, v1 = ev1.y;
+        const CallRec* const r = rec + rid;
+        // Eq. (comp) and the service time on this lane's instances
+        int2 ev[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) ev[j] = *reinterpret_cast<const int2*>(reinterpret_cast<const char*>(r) + lrec[j]);
         int m;
         // a re-issued request avoids the instance it timed out on
-        const int excl = kGeneric ? W->excl : -1;
-        if (kGeneric && W->dpol == HX_DISPATCH_RR) {
+        const int excl = kFaults ? W->excl : -1;
+        if (kGeneric && round_robin) {
           m = W->rr;
           if (m == excl) m = (m + 1 == N) ? 0 : m + 1;
           __syncwarp();
-          if (lane == 0) W->rr = (m + 1 == N) ? 0 : m + 1;
+          W->rr = (m + 1 == N) ? 0 : m + 1;  // every lane writes the same value
         } else {
-          const int64_t q0 = W->q[m0], q1 = W->q[m1];
           // instances that tie in their reward and beat all others: the least cost wins
           // (the lowest instance at alpha = 0, where costs have no weight)
           const longlong2 tie = W->tie;
-          const int64_t q_top = tie.x;
-          const uint32_t cost_mask = (uint32_t)tie.y;
-          const bool top0 = q0 <= q_top, top1 = q1 <= q_top;
-          if (__any_sync(kFull, top0 || top1) && excl < 0) {
-            const uint32_t c0 = top0 ? (uint32_t)e0 & cost_mask : 0xffffffffu, c1 = top1 ? (uint32_t)e1 & cost_mask : 0xffffffffu;
-            const uint32_t least = __reduce_min_sync(kFull, c0 < c1 ? c0 : c1);
-            const unsigned b0 = __ballot_sync(kFull, c0 == least), b1 = __ballot_sync(kFull, c1 == least);
-            m = b0 ? __ffs(b0) - 1 : __ffs(b1) + 31;
+          uint32_t cost[J];
+#pragma unroll
+          for (int j = 0; j < J; ++j) cost[j] = q[j] <= tie.x ? (uint32_t)ev[j].x & (uint32_t)tie.y : 0xffffffffu;
+          const uint32_t least = __reduce_min_sync(kFull, J == 2 && cost[J - 1] < cost[0] ? cost[J - 1] : cost[0]);
+          unsigned b0, b1 = 0;
+          if ((least != 0xffffffffu) & (excl < 0)) {
+            b0 = __ballot_sync(kFull, cost[0] == least);
+            if (J == 2) b1 = __ballot_sync(kFull, cost[J - 1] == least);
+            m = J == 1 || b0 ? __ffs(b0) - 1 : __ffs(b1) + 31;
           } else {
             const float4 f = W->fscore;
-            const ScoreRange a0 = score_range(q0, e0, f, neg_a0), a1 = score_range(q1, e1, f, neg_a1);
-            const float lo = warp_max_f32(fmaxf(a0.lo, a1.lo));
-            const unsigned b0 = __ballot_sync(kFull, a0.hi >= lo), b1 = __ballot_sync(kFull, a1.hi >= lo);
+            ScoreRange s[J];
+#pragma unroll
+            for (int j = 0; j < J; ++j) s[j] = score_range(q[j], ev[j].x, f, neg_a[j]);
+            const float lo = warp_max_f32(J == 2 ? fmaxf(s[0].lo, s[J - 1].lo) : s[0].lo);
+            b0 = __ballot_sync(kFull, s[0].hi >= lo);
+            if (J == 2) b1 = __ballot_sync(kFull, s[J - 1].hi >= lo);
             // one instance's score can reach the best lower bound: it wins
-            if ((((b0 & (b0 - 1)) | (b1 & (b1 - 1))) == 0) && ((b0 == 0) != (b1 == 0)) && excl < 0) {
-              m = b0 ? __ffs(b0) - 1 : __ffs(b1) + 31;
+            if ((((b0 & (b0 - 1)) | (b1 & (b1 - 1))) == 0) & ((b0 == 0) != (b1 == 0)) & (excl < 0)) {
+              m = J == 1 || b0 ? __ffs(b0) - 1 : __ffs(b1) + 31;
             } else {
-              m = exact_winner(W, q0, q1, e0, e1, m0 < N && m0 != excl, m1 < N && m1 != excl, lane);
+              m = exact_winner<J>(W, q[0], q[J - 1], ev[0].x, ev[J - 1].x, lane < N && lane != excl,
+                                  J == 2 && lane + 32 < N && lane + 32 != excl, lane);
             }
           }
         }
-        if (kGeneric) W->excl = -1;
+        if (kFaults) W->excl = -1;
         HX_BOUND(m >= 0 && m < N)
-        // the winner's costs, from the lane that owns it
-        const int64_t est_m = __shfl_sync(kFull, m < 32 ? e0 : e1, m & 31);
-        const int svc_m = __shfl_sync(kFull, m < 32 ? v0 : v1, m & 31);
-        {
-          W->q[m] = W->q[m] + est_m;  // every lane stores the same value
+        const bool low = J == 1 || m < 32;
+        // the winner's costs, on its lane
+        const int est = low ? ev[0].x : ev[J - 1].x, svc = low ? ev[0].y : ev[J - 1].y;
+#pragma unroll
+        for (int j = 0; j < J; ++j) q[j] += lane + 32 * j == m ? est : 0;
+        if (kGeneric && recj >= 0) {
+          HX_BOUND(rid < a.rec_stride)
+          const int4 tail = *reinterpret_cast<const int4*>(&r->tbar);
+          const int64_t t_abs = absolute(now);
+          const int64_t budget = slo_budget(r->deadline - t_abs, tail.x, tail.x + W->frest[(tail.w >> 16) & 0xff]);
+          if (lane == 0) log_dispatch(a, recj, rid, m, t_abs, budget);
         }
-        if (kGeneric) {
-          const int recj = W->recj;
-          if (recj >= 0) {
-            HX_BOUND(rid < a.rec_stride)
-            const int4 tail = *reinterpret_cast<const int4*>(&r->tbar);
-            const int64_t budget = slo_budget(r->deadline - now, tail.x, tail.x + W->frest[(uint32_t)tail.w >> 24]);
-            if (lane == 0) log_dispatch(a, recj, rid, m, now, budget);
-          }
-        }
-        if (npend == 0) {
-          // nothing of this event waits yet, m's queue is empty and m has a
-          // free slot for this request and every one still to be dispatched in
-          // this event: the batch boundary below would start it now whatever
-          // the others do, so it starts at once
-          uint64_t* const sl = W->slot + c.slot_base[m];
-          __syncwarp();
-          const int cn = W->cnt[m];
-          if (W->hsize[m] == 0 && cn + (rel_count - jr) <= c.inst_slots[m]) {
-            start_call(sl, m, cn, rid, svc_m);
-            W->cnt[m] = cn + 1;  // every lane writes the same count
-            set_key(m, sl[0]);
-            continue;
-          }
+        // nothing of this event waits yet, m's queue is empty and m has a free
+        // slot for this request and every one still to be dispatched in this
+        // event: the batch boundary below would start it now whatever the others
+        // do, so it starts at once
+        const InstState I = inst[m];
+        if (((npend | I.hsize) == 0) & (__popc(I.free) >= rel_count)) {
+          start_call(m, I.free, first_slot(m, I), rid, svc);
+          continue;
         }
         // the local-queue key is formed only if the request has to wait
         HX_BOUND(npend < HX_MAX_K)
-        pend_m = lane == npend ? m : pend_m;
-        W->prs[npend] = make_int2(rid, svc_m);  // every lane writes the same entry
-        W->pest[npend] = (int32_t)est_m;
+        if (lane == (m & 31)) W->pend[npend] = make_int4(rid, svc, est, m);
         npend++;
-        touched |= 1ull << m;
       }
       HX_STOP_IF_FAILED()
 
-      // Batch boundary on every touched instance: its free slots go to the most
-      // urgent of the waiting requests and this event's new ones.
-      uint64_t tm = touched;
-      while (tm) {
-        const int m = __ffsll((long long)tm) - 1;
-        tm &= tm - 1;
-        HX_BOUND(m < N)
-#ifdef HX_CHECKED
-        {
-          // m's heap lies inside the warp's arena and holds at most its capacity
-          const int64_t cap = W->hcl[m] ? (int64_t)8 << W->hcl[m] : 0;
-          HX_BOUND(W->hoff[m] >= 0 && W->hoff[m] + cap <= a.arena_per_warp && W->hsize[m] <= cap &&
-                   W->cnt[m] <= c.inst_slots[m])
-        }
-#endif
-        uint64_t* const sl = W->slot + c.slot_base[m];
-        const int ns = c.inst_slots[m];
-        const unsigned pm = __ballot_sync(kFull, lane < npend && pend_m == m);
+      // Batch boundary on the instance with a freed slot and requests waiting
+      // for it, and on every instance this event's requests wait for: its free
+      // slots go to the most urgent of the waiting requests and the new ones.
+      if (npend | waiting) {
         __syncwarp();
-        int cn = W->cnt[m];
-        const int hs = W->hsize[m];
-        // fast paths: an empty queue with room for all of this event's arrivals;
-        // one arrival, one free slot and a waiting queue (one sift)
-        const int npm = __popc(pm);
-        const bool direct = hs == 0 && npm <= ns - cn;
-        const bool fused = !direct && npm == 1 && ns - cn == 1;
+        const int4 pe = lane < npend ? W->pend[lane] : make_int4(0, 0, 0, -1);
+        unsigned left = (1u << npend) - 1;
         const int lpol = kGeneric ? W->lpol : HX_LOCAL_PQ;
-        unsigned bits = direct ? pm : 0u;
-        int2 fst = make_int2(0, 0);
-        if (fused) {
-          fst = push_pop(W, rec, now, lpol, m, pm, lane);
-          bits = 1u;
-        } else if (!direct && pm) {
-          status = push_pending(W, rec, now, lpol, a.arena_per_warp, m, pm, lane);
-          if (status != HX_OK) break;
-        }
-        for (;;) {
-          int rid, svc;
-          if (direct || fused) {
-            if (!bits) break;
-            const int j = __ffs(bits) - 1;
-            bits &= bits - 1;
-            const int2 rs = fused ? fst : W->prs[j];
-            rid = rs.x;
-            svc = rs.y;
-          } else {
-            const int n = W->hsize[m];
-            __syncwarp();
-            if (cn >= ns || n == 0) break;
-            const HeapEnt top = heap_sift_warp(W->arena + W->hoff[m], n - 1, W->arena[W->hoff[m] + n - 1], lane);
-            W->hsize[m] = n - 1;  // every lane writes the same size
-            rid = top.rid;
-            svc = top.svc;
+        const int64_t t_abs = absolute(now);
+        while (waiting | left) {
+          const int m = waiting ? cm : __shfl_sync(kFull, pe.w, __ffs(left) - 1);
+          waiting = 0;
+          const unsigned pm = __ballot_sync(kFull, pe.w == m);
+          left &= ~pm;
+          HX_BOUND(m < N)
+          __syncwarp();
+          const InstState I = inst[m];
+          uint32_t free = I.free;
+          const uint32_t slot_base = first_slot(m, I);
+          const int hs = I.hsize, nf = __popc(free), npm = __popc(pm);
+#ifdef HX_CHECKED
+          {
+            // m's heap lies inside the warp's arena and holds at most its capacity
+            const int hcl = (int)(I.heap >> kHeapCodeShift);
+            const int64_t off = I.heap & kHeapOffMask, cap = hcl ? (int64_t)8 << hcl : 0;
+            HX_BOUND(off + cap <= a.arena_per_warp && hs >= 0 && hs <= cap && (free & ~I.cfg & 0xffffu) == 0)
           }
-          HX_BOUND(rid >= 0 && rid < nc && cn < ns)
-          start_call(sl, m, cn, rid, svc);
-          ++cn;
+#endif
+          HeapEnt* h = W->arena + (I.heap & kHeapOffMask);
+          if (hs == 0 && npm <= nf) {
+            // an empty queue with room for all of this event's requests
+            unsigned bits = pm;
+            while (bits) {
+              const int j = __ffs(bits) - 1;
+              bits &= bits - 1;
+              const int rid = __shfl_sync(kFull, pe.x, j), svc = __shfl_sync(kFull, pe.y, j);
+              HX_BOUND(rid >= 0 && rid < nc && free != 0)
+              free = start_call(m, free, slot_base, rid, svc);
+            }
+          } else if (npm == 1 && nf == 1 && hs > 0) {
+            // one new request, one free slot and a waiting queue: the more
+            // urgent of the request and the queue's top starts and the other
+            // waits, i.e. a push and a pop in one sift
+            const int j = __ffs(pm) - 1;
+            const int4 n1 = make_int4(__shfl_sync(kFull, pe.x, j), __shfl_sync(kFull, pe.y, j),
+                                      __shfl_sync(kFull, pe.z, j), 0);
+            HX_BOUND(n1.x >= 0 && n1.x < nc)
+            const long long key = queue_key(W, rec + n1.x, n1.z, t_abs, lpol);  // the same on every lane
+            const HeapEnt top = h[0];
+            int rid = n1.x, svc = n1.y;
+            if (!ent_better(key, rid, top.key, top.rid)) {
+              HeapEnt e;
+              e.key = key;
+              e.rid = rid;
+              e.svc = svc;
+              heap_sift_warp(h, hs, e, lane);
+              rid = top.rid;
+              svc = top.svc;
+            }
+            HX_BOUND(rid >= 0 && rid < nc)
+            start_call(m, free, slot_base, rid, svc);
+          } else {
+            if (pm) {
+              const long long key = (pm >> lane) & 1u ? queue_key(W, rec + pe.x, pe.z, t_abs, lpol) : 0;
+              status = push_pending(W, inst + m, pe, key, pm, a.arena_per_warp, lane);
+              if (status != HX_OK) break;
+              h = W->arena + (inst[m].heap & kHeapOffMask);
+            }
+            int n = hs + npm;
+            while (free != 0 && n > 0) {
+              const HeapEnt top = heap_sift_warp(h, n - 1, h[n - 1], lane);
+              --n;
+              inst[m].hsize = n;  // every lane writes the same size
+              HX_BOUND(top.rid >= 0 && top.rid < nc)
+              free = start_call(m, free, slot_base, top.rid, top.svc);
+            }
+          }
+          HX_STOP_IF_FAILED()
         }
-        HX_STOP_IF_FAILED()
-        W->cnt[m] = cn;  // every lane writes the same count
-        set_key(m, cn ? sl[0] : kKeyInf);
+        if (status != HX_OK) break;
       }
-      if (kGeneric && a.checked && status == HX_OK) {
-        // after every event: no instance runs more calls than it has slots or
-        // keeps a slot free while requests wait in its queue (Sec. 4.2: free
-        // slots take waiting requests at every batch boundary), and t_queue
-        // stays non-negative
+      HX_STOP_IF_FAILED()
+      if (kGeneric && a.checked) {
+        // after every event: no instance keeps a slot free while requests wait
+        // in its queue (Sec. 4.2: free slots take waiting requests at every
+        // batch boundary) or has slots that are not its own, and t_queue stays
+        // non-negative
         __syncwarp();
         bool bad = false;
-        for (int m = lane; m < N; m += 32) {
-          const int cn = W->cnt[m], ns = c.inst_slots[m];
-          bad |= cn > ns || (cn < ns && W->hsize[m] > 0) || W->q[m] < 0;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+          const InstState I = inst[lane + 32 * j];
+          bad |= (I.free != 0 && I.hsize > 0) || (I.free & ~I.cfg) != 0 || q[j] < 0;
         }
-        if (__any_sync(kFull, bad)) status = HX_ERR_INVARIANT;
+        if (__any_sync(kFull, bad)) {
+          status = HX_ERR_INVARIANT;
+          break;
+        }
       }
-      if (status != HX_OK) break;
     }
 
-    digest_flush(W, dn, lane);
+    digest_flush<kFaults>(W, dn, lane);
     // conservation at the end: every dispatched request finished (t_queue back
     // to zero, no running call, no waiting request)
     bool left = false;
-    for (int m = lane; m < N; m += 32) left |= W->q[m] != 0 || W->cnt[m] != 0 || W->hsize[m] != 0;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const InstState I = inst[lane + 32 * j];
+      left |= (lane + 32 * j < N && q[j] != 0) || I.free != (I.cfg & 0xffffu) || I.hsize != 0;
+    }
     const bool leftover = __any_sync(kFull, left);
     if (lane == 0) {
       int st = status;
       const int32_t n_done = W->n_done;
-      const int32_t steps0 = W->nc + nq + 8 + (kGeneric && c.n_faults > 0 ? 16 * W->nc + 4096 : 0);
-      const int64_t events = (steps0 - steps_left) - W->qa - (kGeneric ? W->reissued : 0);
+      const int32_t steps0 = W->nc + nq + 8 + (kFaults ? 16 * W->nc + 4096 : 0);
+      const int64_t events = (steps0 - steps_left) - W->arrivals - (kFaults ? W->reissued : 0);
       // every query and every call completed exactly once
       if (st == HX_OK && (leftover || n_done != nq || events != W->nc)) st = HX_ERR_INVARIANT;
       hx_result res;
@@ -1088,13 +1191,17 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
   }
 }
 
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, HX_SIM_MIN_BLOCKS) hx_sim_kernel(SimArgs a, ClusterK c) {
-  sim_body<true>(a, c);
-}
-
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, HX_SIM_MIN_BLOCKS) hx_sim_kernel_lean(SimArgs a, ClusterK c) {
-  sim_body<false>(a, c);
-}
+#define HX_SIM_KERNEL(name, J, generic, faults)                                                              \
+  __global__ void __launch_bounds__(kWarpsPerBlock * 32, HX_SIM_MIN_BLOCKS(J)) name(SimArgs a, ClusterK c) { \
+    sim_body<J, generic, faults>(a, c);                                                                      \
+  }
+HX_SIM_KERNEL(hx_sim_kernel_lean, 2, false, false)
+HX_SIM_KERNEL(hx_sim_kernel_lean32, 1, false, false)
+HX_SIM_KERNEL(hx_sim_kernel, 2, true, false)
+HX_SIM_KERNEL(hx_sim_kernel32, 1, true, false)
+HX_SIM_KERNEL(hx_sim_kernel_faults, 2, true, true)
+HX_SIM_KERNEL(hx_sim_kernel_faults32, 1, true, true)
+#undef HX_SIM_KERNEL
 
 // ---------------------------------------------------------- best kernel
 namespace {

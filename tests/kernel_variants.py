@@ -5,7 +5,7 @@ mention were measured (GPU only).
 
     python -m tests.kernel_variants FAMILY [--traces 64] [--reps 3] [--out FILE]
 
-Family `occupancy`: 7 or 6 resident 4-warp blocks per SM instead of 8 (the
+Family `occupancy`: 8, 7 or 6 resident 4-warp blocks per SM (the
 register budget follows).
 
 A variant is a list of edits ((anchor, replacement) in hx_kernels.cu, or
@@ -34,7 +34,7 @@ NVCC = ["nvcc", "-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo"
         "-fPIC", "-I", os.path.join(ROOT, "include")]
 
 VARIANTS = {
-    "occupancy": {"blocks7": ([], ["-DHX_SIM_MIN_BLOCKS=7"]), "blocks6": ([], ["-DHX_SIM_MIN_BLOCKS=6"])},
+    "occupancy": {"blocks8": ([], ["-DHX_SIM_MIN_BLOCKS(J)=8"]), "blocks7": ([], ["-DHX_SIM_MIN_BLOCKS(J)=7"]), "blocks6": ([], ["-DHX_SIM_MIN_BLOCKS(J)=6"])},
 }
 
 

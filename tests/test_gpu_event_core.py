@@ -1,0 +1,82 @@
+"""The simulation kernel's event loop at the edges of its representation, against
+the oracle: times around and past 2^31 and 2^32 us (event times are 32-bit,
+relative to a base that moves), calls that end at the same time in one and in
+many slots, queries of more call records than one sweep of the warp fetches."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2505_05286_gb300 import build as B
+from paper_2505_05286_gb300 import hxsim as H
+from paper_2505_05286_gb300 import workloads as W
+
+FIELDS = ["p95_us", "makespan_us", "events", "digest", "slo_met", "n_done", "status"]
+INST = [1, 16, 32, 33, 64]
+
+
+def _check(tr, cl, generic):
+    B.build()
+    n = 6
+    lpol = (np.arange(n) % 3).astype(np.uint8) if generic else np.zeros(n, np.uint8)
+    grid = W.Grid(np.array([0, W.SCALE // 7, W.SCALE // 2, W.SCALE * 6 // 7, W.SCALE, W.SCALE], np.int64),
+                  np.array([W.SCALE, 0, 2 * W.SCALE, W.SCALE, W.SCALE // 4, 4 * W.SCALE], np.int64),
+                  np.array([0, 1, 2, 3, 15, 0], np.int32), np.full(n, 300_000 ** 2, np.int64), lpol,
+                  np.zeros(n, np.uint8))
+    wl = W.Workload("core", [tr], cl, grid, W.OBJ_P95)
+    sim = H.Sim(wl.traces, wl.cluster, wl.grid)
+    assert sim.info()["generic_kernel"] == int(generic or cl.faults is not None)
+    sim.run()
+    got, want = sim.results(), oracle.run(wl)
+    sim.close()
+    for f in FIELDS:
+        assert np.array_equal(got[f], want[f]), f
+
+
+def _cluster(n_inst, slots=(1, 3, 16), rmax=2):
+    cl = W.make_cluster(W.RECIPES[1])
+    cl.inst_type = (np.arange(n_inst) % 3).astype(np.uint8)
+    cl.slots = np.array(slots, np.int32)
+    cl.rmax = rmax
+    return cl
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["lean", "generic", "faults"])
+@pytest.mark.parametrize("n_inst", INST)
+def test_times_past_32_bits(n_inst, kind):
+    tr = W.make_trace(W.RECIPES[1], 1, 40 + n_inst, n_queries=160)
+    # bursts at the edges of 31 and 32 bits and gaps of more than 2^32 us between them,
+    # with calls of up to 100 s running across
+    at = np.array([0, 2 ** 31 - 10_000_000, 2 ** 31 - 1, 2 ** 31, 2 ** 32 - 3, 2 ** 32 + 2 ** 31 - 1,
+                   3 * 2 ** 32 + 5, 9 * 2 ** 32 - 1], np.int64)
+    tr.arrival_us = np.sort(np.concatenate([at + (i * 997) * (i % 5) for i in range(20)]))
+    tr.prompt[::17] = 1_000_000
+    cl = _cluster(n_inst)
+    if kind == "faults":
+        cl.timeout_mult_fp = 2 * W.SCALE
+        cl.faults = np.zeros(2, W.FAULT_DTYPE)
+        cl.faults[0] = (0, 0, 2 ** 31 - 20_000_000, 2 ** 31 + 20_000_000, 0)
+        cl.faults[1] = (n_inst - 1, 0, 2 ** 32 - 5, 2 ** 32 + 60_000_000, 4 * W.SCALE)
+    _check(tr, cl, kind == "generic")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("generic", [False, True])
+@pytest.mark.parametrize("slots", [(1, 1, 1), (16, 16, 16), (2, 15, 16)])
+@pytest.mark.parametrize("n_inst", INST)
+def test_equal_completion_times(n_inst, slots, generic):
+    tr = W.make_trace(W.RECIPES[1], 1, 60 + n_inst, n_queries=120)
+    tr.prompt[:] = 2000
+    tr.out[:] = 100
+    tr.out_est[:] = 100
+    tr.arrival_us = (np.arange(120) // 15 * 400_000).astype(np.int64)
+    _check(tr, _cluster(n_inst, slots), generic)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_inst", [4, 64])
+def test_queries_of_many_calls(n_inst):
+    r = W.Recipe(**{**W.EXTRA["paper-shaped"].__dict__, "p_err": 0.97, "rmax": 15})
+    tr = W.make_trace(r, 17, 5, n_queries=40)
+    assert int(np.diff(tr.call_base).max()) > 64
+    _check(tr, _cluster(n_inst, rmax=15), False)
