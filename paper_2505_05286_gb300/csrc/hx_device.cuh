@@ -135,6 +135,7 @@ struct SimArgs {
   int64_t tenant_topk_off[HX_MAX_TENANTS];  // tenant t's top-K heap within the warp's topk slice
   const int64_t* subset;    // [n_work] sims to run in work order, or NULL: all n_sims
   int64_t n_work;
+  int32_t prefetch;         // fetch a query's records into L1 as it arrives
   int32_t checked;          // check the scheduler's invariants after every event (generic kernel)
 };
 
@@ -187,7 +188,7 @@ struct __align__(16) WarpShared {
   int32_t arrivals, trace;      // arrivals taken so far (likewise); the simulation's trace
   uint64_t digest;
   int64_t makespan;
-  int32_t n_done, slo_met, pad, tk;
+  int32_t n_done, slo_met, sink, tk;  // sink: where prefetched records are copied to
   int64_t tkmin;                // root of the full top-K heap (written alike by every lane)
   int32_t tslo[HX_MAX_TENANTS], tdone[HX_MAX_TENANTS];  // per-tenant counts (generic kernel)
   int32_t ttk[HX_MAX_TENANTS];  // per-tenant top-K heaps: entries (generic kernel with tenants)

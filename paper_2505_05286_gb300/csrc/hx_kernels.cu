@@ -959,6 +959,14 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         rel_first = (int32_t)(a.qcall[qbase + qa] - W->cb);
         HX_BOUND(rel_first >= 0 && rel_first < nc)
         rel_count = 1;
+        if (a.prefetch) {
+          // the query's records into L1, 32 bytes a lane (a copy that nobody reads)
+          const char* pa = reinterpret_cast<const char*>(rec + rel_first);
+          const char* const pe = reinterpret_cast<const char*>(rec + (a.qcall[qbase + qa + 1] - W->cb));
+          const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&W->sink);
+          for (pa += 32 * lane; pa < pe; pa += 1024)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(pa) : "memory");
+        }
         __syncwarp();
         W->arrivals = qa + 1;  // every lane writes the same values
         const int64_t at = qa + 1 < W->nq ? a.arrival[qbase + qa + 1] : 0;
