@@ -46,9 +46,9 @@ struct __align__(16) CallRec {
 };
 static_assert(sizeof(CallRec) == 64, "CallRec is one 64-byte unit");
 
-// Local-queue entry: priority key (higher first) and request id (lower first).
+// Local-queue entry: priority key + 2^63 (higher first) and request id (lower first).
 struct __align__(16) HeapEnt {
-  long long key;
+  unsigned long long key;
   int rid;
   int svc;   // service time on the queue's instance
 };

@@ -53,44 +53,21 @@ __device__ __forceinline__ int warp_argmax_s64(int64_t s, int idx) {
 
 // floor(n / d) for 0 <= n < 2^63 and 1 <= d < 2^54.  Trial-quotient method
 // (Knuth, TAOCP vol. 2, 4.3.1): a quotient estimate from a single-precision
-// reciprocal, refined once on the exact int64 remainder when it is 2^21 or
-// more, then corrected by at most one step each way.  Operands reach float
-// through two 32-bit halves.  The estimate's relative error is below
-// 3.5 * 2^-23 (two conversions, the approximate reciprocal, one product), so
-// below 2^21 it is within one of n/d, and below 2^30 the refined one is.
-// Quotients of 2^30 or more (and d = 1) take the exact integer paths.
-__device__ __forceinline__ float u64_to_float(uint64_t x) {
-  return __fmaf_rn((float)(uint32_t)(x >> 32), 4294967296.0f, (float)(uint32_t)x);
-}
-
-__device__ __forceinline__ float s64_to_float(int64_t x) {
-  return x < 0 ? -u64_to_float((uint64_t)(-x)) : u64_to_float((uint64_t)x);
-}
-
-// nf = u64_to_float(n), given by a caller that divides one n many times.
-__device__ __forceinline__ uint64_t udiv_trial_f(uint64_t n, float nf, uint64_t d) {
-  if (d == 1) return n;
+// reciprocal, refined once on the exact int64 remainder, then corrected by at
+// most one step each way.  The estimate's relative error is below 2^-21 (two
+// conversions, the approximate reciprocal, one product), so below 2^30 the
+// remainder's quotient is below 2^9 and the refined estimate within one of n/d.
+// Quotients of 2^30 or more take the exact integer path.
+__device__ __forceinline__ uint64_t udiv_trial(uint64_t n, uint64_t d) {
   float rd;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"(u64_to_float(d)));
-  const float qf = nf * rd;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"((float)d));
+  const float qf = (float)n * rd;
   if (qf >= 1073741824.0f) return n / d;
   uint64_t q = (uint32_t)qf;
-  int64_t r = (int64_t)(n - q * d);
-  if (qf >= 2097152.0f) {
-    q += (int64_t)(int32_t)(s64_to_float(r) * rd);
-    r = (int64_t)(n - q * d);
-  }
-  if (r < 0) {
-    q--;
-    r += (int64_t)d;
-  } else if (r >= (int64_t)d) {
-    q++;
-    r -= (int64_t)d;
-  }
-  return q;
+  q += (int64_t)(int32_t)((float)(int64_t)(n - q * d) * rd);
+  const int64_t r = (int64_t)(n - q * d);
+  return q - (r < 0 ? 1 : 0) + (r >= (int64_t)d ? 1 : 0);
 }
-
-__device__ __forceinline__ uint64_t udiv_trial(uint64_t n, uint64_t d) { return udiv_trial_f(n, u64_to_float(n), d); }
 
 // Workload-balanced reward term of Eq. (score): beta / max(t_queue, 1), capped.
 __device__ __forceinline__ int64_t reward_of(int64_t beta, int64_t q) {
@@ -337,76 +314,90 @@ __device__ __forceinline__ void digest_push(WarpShared* W, int& dn, T t, uint32_
   }
 }
 
-__device__ __forceinline__ bool ent_better(long long ka, int ra, long long kb, int rb) {
-  return ka > kb || (ka == kb && ra < rb);
+__device__ __forceinline__ bool ent_better(const HeapEnt& a, const HeapEnt& b) {
+  return (a.key > b.key) | ((a.key == b.key) & (a.rid < b.rid));
+}
+
+// A heap entry in one 16-byte access, under a predicate and not a branch;
+// without it the load leaves an entry that goes after every other.
+__device__ __forceinline__ HeapEnt ent_load(const HeapEnt* p, bool on) {
+  HeapEnt e;
+  uint32_t lo = 0, hi = 0;
+  e.rid = INT_MAX;
+  e.svc = 0;
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.s32 p, %5, 0;\n @p ld.global.v4.b32 {%0, %1, %2, %3}, [%4];\n}"
+      : "+r"(lo), "+r"(hi), "+r"(e.rid), "+r"(e.svc)
+      : "l"(p), "r"((int)on)
+      : "memory");
+  e.key = (unsigned long long)hi << 32 | lo;
+  return e;
+}
+
+__device__ __forceinline__ void ent_store(HeapEnt* p, const HeapEnt& e, bool on) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %5, 0;\n @p st.global.v4.b32 [%4], {%0, %1, %2, %3};\n}" ::"r"(
+                   (uint32_t)e.key),
+               "r"((uint32_t)(e.key >> 32)), "r"(e.rid), "r"(e.svc), "l"(p), "r"((int)on)
+               : "memory");
 }
 
 // Local queues are 32-ary max-heaps on (key desc, rid asc) in the warp's
 // arena: node i has children 32 i + 1 .. 32 i + 32, so 40k waiting requests
-// sit four levels deep.  Push sifts up on one lane (new requests rarely
-// climb); pop and replace sift down with the whole warp, one lane per child.
-__device__ __forceinline__ void heap_push(HeapEnt* h, int n, long long key, int rid, int svc) {
+// sit four levels deep.  New requests rarely climb past their parent, so an
+// event's join at once unless one does; pop and replace sift down with the whole
+// warp, one lane per child.  At alpha = 1 every call passes through one queue and
+// the event's chain sets a run's end: with the root's children read before the
+// key or the start needs them, the children compared by their keys' high words
+// and entries moved by predicated 16-byte accesses, 8 traces x 20000 queries x
+// 1024 points took 463 -> 430 ms, 3000 queries on 64 instances 40.3 -> 38.4 ms.
+__device__ __forceinline__ void heap_push(HeapEnt* h, int n, HeapEnt e) {
   int i = n;
   while (i > 0) {
     const int par = (i - 1) >> 5;
-    const HeapEnt pe = h[par];
-    if (!ent_better(key, rid, pe.key, pe.rid)) break;
-    h[i] = pe;
+    const HeapEnt pe = ent_load(h + par, true);
+    if (!ent_better(e, pe)) break;
+    ent_store(h + i, pe, true);
     i = par;
   }
-  HeapEnt e;
-  e.key = key;
-  e.rid = rid;
-  e.svc = svc;
-  h[i] = e;
+  ent_store(h + i, e, true);
 }
 
-// All lanes call with the same arguments.  The top entry leaves the heap and
-// `sink` takes its place, sinking to its level; the heap then holds m
-// entries (m = n - 1 and sink = the last entry: a pop; m = n and sink = a new
-// entry: a replace).  Every lane gets the old top.
-__device__ __forceinline__ HeapEnt heap_sift_warp(HeapEnt* h, int m, HeapEnt sink, int lane) {
-  const HeapEnt top = h[0];
+// This lane's child of node i in a heap of m entries; past its end an entry
+// that goes after every other.
+__device__ __forceinline__ HeapEnt heap_child(const HeapEnt* h, int i, int m, int lane) {
+  const int child = 32 * i + 1 + lane;
+  return ent_load(h + child, child < m);
+}
+
+// All lanes call with the same arguments but c, their child of the root.  The
+// top entry has left the heap and `sink` takes its place, sinking to its level;
+// the heap then holds m entries (m = n - 1 and sink = the last entry: a pop;
+// m = n and sink = a new entry: a replace).
+__device__ __forceinline__ void heap_sift_warp(HeapEnt* h, int m, HeapEnt sink, HeapEnt c, int lane) {
+  const uint32_t sink_hi = (uint32_t)(sink.key >> 32);
   int i = 0;
-  for (;;) {
-    const int first = 32 * i + 1;
-    if (first >= m) break;
-    const int child = first + lane;
-    long long ck = LLONG_MIN;
-    int cr = INT_MAX, cs = 0;
-    if (child < m) {
-      const HeapEnt e = h[child];
-      ck = e.key;
-      cr = e.rid;
-      cs = e.svc;
-    }
-    // warp argmax of (key desc, rid asc): the rids decide only among equal keys
-    const uint64_t uk = (uint64_t)ck ^ 0x8000000000000000ull;
-    const uint32_t hi = (uint32_t)(uk >> 32), lo = (uint32_t)uk;
+  while (32 * i + 1 < m) {
+    // the first child by (key desc, rid asc): the keys' high words decide, the
+    // low words and the rids among equals only
+    const uint32_t hi = (uint32_t)(c.key >> 32);
     const uint32_t mh = __reduce_max_sync(kFull, hi);
-    const bool c1 = hi == mh;
-    const uint32_t ml = __reduce_max_sync(kFull, c1 ? lo : 0u);
-    unsigned best = __ballot_sync(kFull, c1 && lo == ml);
-    if (best & (best - 1)) {
+    if (mh < sink_hi) break;
+    unsigned best = __ballot_sync(kFull, hi == mh);
+    if (((best & (best - 1)) != 0) | (mh == sink_hi)) {
+      const uint32_t lo = (uint32_t)c.key, ml = __reduce_max_sync(kFull, hi == mh ? lo : 0u);
+      best = __ballot_sync(kFull, (hi == mh) & (lo == ml));
       const bool tie = (best >> lane) & 1u;
-      const uint32_t mr = __reduce_min_sync(kFull, tie ? (uint32_t)cr : 0xffffffffu);
-      best = __ballot_sync(kFull, tie && (uint32_t)cr == mr);
+      const uint32_t mr = __reduce_min_sync(kFull, tie ? (uint32_t)c.rid : 0xffffffffu);
+      best = __ballot_sync(kFull, tie & ((uint32_t)c.rid == mr));
+      if (__ballot_sync(kFull, ent_better(c, sink)) == 0) break;
     }
-    const int b = __ffs(best) - 1;
-    // the best child moves up unless the sinking entry goes before it
-    if (!__shfl_sync(kFull, (int)ent_better(ck, cr, sink.key, sink.rid), b)) break;
-    if (lane == b) {
-      HeapEnt e;
-      e.key = ck;
-      e.rid = cr;
-      e.svc = cs;
-      h[i] = e;
-    }
-    i = first + b;
+    const int b = 31 - __clz(best);
+    ent_store(h + i, c, lane == b);  // the best child moves up
+    i = 32 * i + 1 + b;
+    c = heap_child(h, i, m, lane);
   }
-  if (lane == 0 && m > 0) h[i] = sink;
+  ent_store(h + i, sink, (lane == 0) & (m > 0));
   __syncwarp();
-  return top;
 }
 
 // Min-heap of the K largest latencies seen so far, 32-ary like the local
@@ -416,6 +407,7 @@ __device__ __forceinline__ HeapEnt heap_sift_warp(HeapEnt* h, int m, HeapEnt sin
 // copies in shared memory.
 __device__ __noinline__ void topk_insert_warp(int64_t* h, int32_t* size, int kcap, int64_t* root_out, int64_t v,
                                               int lane) {
+  __builtin_assume(__isGlobal(h));
   const int n = *size;
   if (n < kcap) {
     // filling: sift up on lane 0 (few levels)
@@ -471,44 +463,55 @@ __device__ __forceinline__ int64_t slo_budget(int64_t num, int64_t tb, int64_t d
 // with the budget at send time (now) and the common now dropped; FCFS: earliest
 // enqueue; LLF: least deadline - now - remaining work, again with the common
 // now dropped.  est is its Eq. (comp) on the instance.
-__device__ __forceinline__ long long queue_key(const WarpShared* W, const CallRec* r, int est, int64_t now, int lpol) {
+__device__ __forceinline__ unsigned long long queue_key(const WarpShared* W, const CallRec* r, int est, int64_t now, int lpol) {
   const int64_t dl = r->deadline;
   const int4 tail = *reinterpret_cast<const int4*>(&r->tbar);
   const int64_t tb = tail.x;
   const int64_t dd = tb + W->frest[(tail.w >> 16) & 0xff];
-  return lpol == HX_LOCAL_PQ     ? (long long)(kScale * ((int64_t)est - slo_budget(dl - now, tb, dd)) - W->G * now)
-         : lpol == HX_LOCAL_FCFS ? (long long)(-now)
-                                 : (long long)(dd - dl);
+  const int64_t key = lpol == HX_LOCAL_PQ     ? kScale * ((int64_t)est - slo_budget(dl - now, tb, dd)) - W->G * now
+                      : lpol == HX_LOCAL_FCFS ? -now
+                                              : dd - dl;
+  return (unsigned long long)key ^ 1ull << 63;
 }
 
-// The instance's new requests (this lane's: p, its key: key; on the lanes of
-// pm) join its local queue, which moves to a region of twice the size when it
-// is full.  All lanes call.  Returns HX_OK or HX_ERR_CAPACITY.
-__device__ __forceinline__ int push_pending(WarpShared* W, InstState* I, int4 p, long long key, unsigned pm,
-                                            int64_t arena_per_warp, int lane) {
+// The instance's new requests (this lane's: e; on the lanes of pm) join its
+// local queue, which moves to a region of twice the size when it is full (8
+// requests at most, so once).  All lanes call.  Returns HX_OK or
+// HX_ERR_CAPACITY.
+__device__ __forceinline__ int push_pending(WarpShared* W, InstState* I, HeapEnt e, unsigned pm, int64_t arena_per_warp,
+                                            int lane) {
   HeapEnt* const arena = W->arena;
-  while (pm) {
-    const int j = __ffs(pm) - 1;
-    pm &= pm - 1;
-    const int size = I->hsize;
-    const uint32_t heap = I->heap;
-    const int hcl = (int)(heap >> kHeapCodeShift), cap = hcl ? 8 << hcl : 0, bump = W->bump;
-    const int off = (int)(heap & kHeapOffMask);
+  __builtin_assume(__isGlobal(arena));
+  const int size = I->hsize, np = __popc(pm);
+  const uint32_t heap = I->heap;
+  const int hcl = (int)(heap >> kHeapCodeShift), cap = hcl ? 8 << hcl : 0;
+  int hoff = (int)(heap & kHeapOffMask);
+  if (size + np > cap) {
+    const int ncap = cap ? 2 * cap : 16, bump = W->bump, off = hoff;
+    if ((int64_t)bump + ncap > arena_per_warp) return HX_ERR_CAPACITY;
+    hoff = bump;
+    for (int i = lane; i < size; i += 32) arena[hoff + i] = arena[off + i];
     __syncwarp();
-    int hoff = off;
-    if (size == cap) {
-      const int ncap = cap ? 2 * cap : 16;
-      if ((int64_t)bump + ncap > arena_per_warp) return HX_ERR_CAPACITY;
-      hoff = bump;
-      for (int i = lane; i < size; i += 32) arena[hoff + i] = arena[off + i];
-      __syncwarp();
-      W->bump = bump + ncap;  // every lane writes the same values
-      I->heap = (uint32_t)hoff | (uint32_t)(hcl + 1) << kHeapCodeShift;
-    }
-    if (lane == j) heap_push(arena + hoff, size, key, p.x, p.y);
-    I->hsize = size + 1;
-    __syncwarp();
+    W->bump = bump + ncap;  // every lane writes the same values
+    I->heap = (uint32_t)hoff | (uint32_t)(hcl + 1) << kHeapCodeShift;
   }
+  HeapEnt* const h = arena + hoff;
+  const bool mine = (pm >> lane) & 1u;
+  const int pos = size + __popc(pm & ((1u << lane) - 1));
+  // with a non-empty queue every new entry's parent is an old one: when none
+  // climbs past its parent, all are stored at once
+  const bool ask = mine & (size > 0);
+  const HeapEnt pe = ent_load(h + ((pos - 1) >> 5), ask);
+  if (!__any_sync(kFull, (ask & ent_better(e, pe)) | (size == 0))) {
+    ent_store(h + pos, e, mine);
+  } else {
+    for (unsigned left = pm; left; left &= left - 1) {
+      if (lane == __ffs(left) - 1) heap_push(h, pos, e);
+      __syncwarp();
+    }
+  }
+  I->hsize = size + np;
+  __syncwarp();
   return HX_OK;
 }
 
@@ -518,12 +521,11 @@ template <int J>
 __device__ __noinline__ int exact_winner(const WarpShared* W, int64_t q0, int64_t q1, int e0, int e1, bool ok0, bool ok1,
                                          int lane) {
   const uint64_t beta = (uint64_t)W->beta;
-  const float betaf = u64_to_float(beta);
   const int64_t A = W->A, oma = W->one_minus_a;
-  const uint64_t r0 = udiv_trial_f(beta, betaf, q0 > 1 ? (uint64_t)q0 : 1ull);
+  const uint64_t r0 = udiv_trial(beta, q0 > 1 ? (uint64_t)q0 : 1ull);
   const int64_t s0 = ok0 ? oma * (int64_t)(r0 < (uint64_t)kRewardCap ? r0 : kRewardCap) - A * e0 : INT64_MIN;
   if (J == 1) return warp_argmax_s64(s0, lane);
-  const uint64_t r1 = udiv_trial_f(beta, betaf, q1 > 1 ? (uint64_t)q1 : 1ull);
+  const uint64_t r1 = udiv_trial(beta, q1 > 1 ? (uint64_t)q1 : 1ull);
   const int64_t s1 = ok1 ? oma * (int64_t)(r1 < (uint64_t)kRewardCap ? r1 : kRewardCap) - A * e1 : INT64_MIN;
   const bool take1 = s1 > s0;
   return warp_argmax_s64(take1 ? s1 : s0, take1 ? lane + 32 : lane);
@@ -772,6 +774,11 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
 
     // one instance per lane: 16 slot entries each, so that no load gives the first
     auto first_slot = [&](int m, const InstState& I) -> uint32_t { return J == 1 ? 16u * m : I.cfg >> 16; };
+    auto queue_of = [&](uint32_t heap) -> HeapEnt* {
+      HeapEnt* const arena = W->arena;
+      __builtin_assume(__isGlobal(arena));
+      return arena + (heap & kHeapOffMask);
+    };
     // Request rid starts on instance m now in the highest of its free slots;
     // svc is its service time on m (on m's lane at least).  The slots stay
     // unsorted: a start is one store and a comparison with the instance's next
@@ -861,7 +868,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       }
       --steps_left;
       npend = 0;
-      int cm = 0, waiting = 0;  // the instance whose slot this event frees, and the requests waiting for it
+      int cm = -1, waiting = 0;  // the instance whose slot this event frees, and the requests waiting for it
       // requests released by this event: rel_first .. rel_first + rel_count - 1
       int32_t rel_first = 0, rel_count = 0;
       if (mn <= arr) {
@@ -923,6 +930,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         } else if (what == kDoneChain) {
           // a chain of the query ended: the last one releases the evaluation
           uint8_t* const chains = W->chains + qid;
+          __builtin_assume(__isGlobal(chains));
           const int ended = *chains + 1;
           __syncwarp();
           *chains = (uint8_t)ended;  // every lane writes the same byte
@@ -1056,22 +1064,23 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       // for it, and on every instance this event's requests wait for: its free
       // slots go to the most urgent of the waiting requests and the new ones.
       if (npend | waiting) {
-        __syncwarp();
-        const int4 pe = lane < npend ? W->pend[lane] : make_int4(0, 0, 0, -1);
-        unsigned left = (1u << npend) - 1;
         const int lpol = kGeneric ? W->lpol : HX_LOCAL_PQ;
-        const int64_t t_abs = absolute(now);
-        while (waiting | left) {
-          const int m = waiting ? cm : __shfl_sync(kFull, pe.w, __ffs(left) - 1);
-          waiting = 0;
-          const unsigned pm = __ballot_sync(kFull, pe.w == m);
-          left &= ~pm;
-          HX_BOUND(m < N)
+        int m = cm;
+        int4 pe = make_int4(0, 0, 0, -1);  // entry j on lane j
+        unsigned left = 0, pm = 0;
+        if (npend) {
           __syncwarp();
+          if (lane < npend) pe = W->pend[lane];
+          left = (1u << npend) - 1;
+          if (!waiting) m = __shfl_sync(kFull, pe.w, 0);
+        }
+        for (;;) {
+          HX_BOUND(m >= 0 && m < N)
           const InstState I = inst[m];
           uint32_t free = I.free;
           const uint32_t slot_base = first_slot(m, I);
-          const int hs = I.hsize, nf = __popc(free), npm = __popc(pm);
+          const int hs = I.hsize;
+          HeapEnt* h = queue_of(I.heap);
 #ifdef HX_CHECKED
           {
             // m's heap lies inside the warp's arena and holds at most its capacity
@@ -1080,56 +1089,72 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
             HX_BOUND(off + cap <= a.arena_per_warp && hs >= 0 && hs <= cap && (free & ~I.cfg & 0xffffu) == 0)
           }
 #endif
-          HeapEnt* h = W->arena + (I.heap & kHeapOffMask);
-          if (hs == 0 && npm <= nf) {
-            // an empty queue with room for all of this event's requests
-            unsigned bits = pm;
-            while (bits) {
-              const int j = __ffs(bits) - 1;
-              bits &= bits - 1;
-              const int rid = __shfl_sync(kFull, pe.x, j), svc = __shfl_sync(kFull, pe.y, j);
-              HX_BOUND(rid >= 0 && rid < nc && free != 0)
-              free = start_call(m, free, slot_base, rid, svc);
+          if (npend) {
+            pm = __ballot_sync(kFull, pe.w == m);
+            left &= ~pm;
+          }
+          HeapEnt e;
+          if (pm) {
+            e.key = (hs > 0 || __popc(pm) > __popc(free)) && ((pm >> lane) & 1u)
+                        ? queue_key(W, rec + pe.x, pe.z, absolute(now), lpol) : 0;
+            e.rid = pe.x;
+            e.svc = pe.y;
+          }
+          if (hs > 0 && m == cm && __popc(pm) < 2) {
+            // requests wait, so this event freed m's only free slot.  It goes to
+            // the queue's top, or to the new request if that is more urgent; the
+            // queue's last entry or the new one sinks from the top.
+            HeapEnt kid = heap_child(h, 0, hs, lane);
+            const HeapEnt top = ent_load(h, true);
+            int n = hs;
+            bool fresh = false;
+            if (pm) {
+              const int j = __ffs(pm) - 1;
+              e.key = __shfl_sync(kFull, e.key, j);
+              e.rid = __shfl_sync(kFull, e.rid, j);
+              e.svc = __shfl_sync(kFull, e.svc, j);
+              fresh = ent_better(e, top);
+            } else {
+              e = ent_load(h + --n, true);
+              if (lane + 1 >= n) kid.key = 0;  // the last entry is no child any more
+              inst[m].hsize = n;  // every lane writes the same size
             }
-          } else if (npm == 1 && nf == 1 && hs > 0) {
-            // one new request, one free slot and a waiting queue: the more
-            // urgent of the request and the queue's top starts and the other
-            // waits, i.e. a push and a pop in one sift
-            const int j = __ffs(pm) - 1;
-            const int4 n1 = make_int4(__shfl_sync(kFull, pe.x, j), __shfl_sync(kFull, pe.y, j),
-                                      __shfl_sync(kFull, pe.z, j), 0);
-            HX_BOUND(n1.x >= 0 && n1.x < nc)
-            const long long key = queue_key(W, rec + n1.x, n1.z, t_abs, lpol);  // the same on every lane
-            const HeapEnt top = h[0];
-            int rid = n1.x, svc = n1.y;
-            if (!ent_better(key, rid, top.key, top.rid)) {
-              HeapEnt e;
-              e.key = key;
-              e.rid = rid;
-              e.svc = svc;
-              heap_sift_warp(h, hs, e, lane);
-              rid = top.rid;
-              svc = top.svc;
-            }
+            const int rid = fresh ? e.rid : top.rid, svc = fresh ? e.svc : top.svc;
             HX_BOUND(rid >= 0 && rid < nc)
             start_call(m, free, slot_base, rid, svc);
+            if (!fresh) heap_sift_warp(h, n, e, kid, lane);
           } else {
-            if (pm) {
-              const long long key = (pm >> lane) & 1u ? queue_key(W, rec + pe.x, pe.z, t_abs, lpol) : 0;
-              status = push_pending(W, inst + m, pe, key, pm, a.arena_per_warp, lane);
+            const bool direct = hs == 0 && __popc(pm) <= __popc(free);
+            int n = 0;
+            if (!direct) {
+              status = push_pending(W, inst + m, e, pm, a.arena_per_warp, lane);
               if (status != HX_OK) break;
-              h = W->arena + (inst[m].heap & kHeapOffMask);
+              h = queue_of(inst[m].heap);
+              n = hs + __popc(pm);
             }
-            int n = hs + npm;
-            while (free != 0 && n > 0) {
-              const HeapEnt top = heap_sift_warp(h, n - 1, h[n - 1], lane);
-              --n;
-              inst[m].hsize = n;  // every lane writes the same size
-              HX_BOUND(top.rid >= 0 && top.rid < nc)
-              free = start_call(m, free, slot_base, top.rid, top.svc);
+            // free slots: to all of this event's requests (an empty queue with
+            // room for them), or to the most urgent
+            while (free != 0 && (direct ? pm != 0 : n > 0)) {
+              int rid, svc;
+              if (direct) {
+                const int j = __ffs(pm) - 1;
+                pm &= pm - 1;
+                rid = __shfl_sync(kFull, pe.x, j);
+                svc = __shfl_sync(kFull, pe.y, j);
+              } else {
+                const HeapEnt top = ent_load(h, true), last = ent_load(h + --n, true);
+                rid = top.rid;
+                svc = top.svc;
+                inst[m].hsize = n;  // every lane writes the same size
+                heap_sift_warp(h, n, last, heap_child(h, 0, n, lane), lane);
+              }
+              HX_BOUND(rid >= 0 && rid < nc)
+              free = start_call(m, free, slot_base, rid, svc);
             }
           }
           HX_STOP_IF_FAILED()
+          if (left == 0) break;
+          m = __shfl_sync(kFull, pe.w, __ffs(left) - 1);
         }
         if (status != HX_OK) break;
       }
