@@ -86,24 +86,20 @@ int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 // the record says.
 constexpr int kMaxDevices = 64;
 std::mutex g_smem_mu;
-constexpr int kSimKernels = 6;
-int g_smem_limit[kMaxDevices][kSimKernels] = {};  // [device][instantiation]
+int g_smem_limit[kMaxDevices][hx::kSimKernels] = {};  // [device][kernel]
 
-using SimKernel = void (*)(hx::SimArgs, hx::ClusterK);
-constexpr SimKernel kSimKernel[kSimKernels] = {hx::hx_sim_kernel_lean,   hx::hx_sim_kernel,   hx::hx_sim_kernel_faults,
-                                               hx::hx_sim_kernel_lean32, hx::hx_sim_kernel32, hx::hx_sim_kernel_faults32};
-
-// The instantiation of the simulation kernel a cluster runs on.
-int sim_kernel_of(bool generic, const hx::ClusterK& ck) {
-  return (!generic ? 0 : ck.n_faults == 0 ? 1 : 2) + (ck.n_inst <= 32 ? 3 : 0);
+// The instantiation of the simulation kernel for a cluster; few: a run of few
+// warps.  That one fetches a query's records into L1 as it arrives (an event
+// reads two sectors of them that would come from L2 otherwise, about a fifth of
+// its latency) and may use twice the registers.
+int sim_kernel_of(bool generic, const hx::ClusterK& ck, bool few) {
+  return 4 * (!generic ? 0 : ck.n_faults == 0 ? 1 : 2) + (few ? 2 : 0) + (ck.n_inst <= 32 ? 1 : 0);
 }
 
-// Whether a simulation fetches a query's records into L1 as it arrives: an event
-// reads two sectors of them that would come from L2 otherwise, about a fifth of
-// an event's latency.  It pays while the running warps' active queries fit L1
-// (512 warps: 10.9 -> 7.9 ms on 8 traces x 2000 queries x 64 points; 1536 warps
+// Few warps: up to 12 per SM, whose active queries fit L1 (the fetch alone: 512
+// warps 10.9 -> 7.9 ms on 8 traces x 2000 queries x 64 points; 1536 warps
 // 19.3 -> 18.3 ms; 2560 warps +4 %, a full GPU +1-3 %).
-int prefetch_records(int64_t resident_warps, int sms) { return resident_warps <= 12 * (int64_t)sms ? 1 : 0; }
+bool few_warps(int64_t warps, int sms) { return warps <= 12 * (int64_t)sms; }
 
 int ensure_dyn_smem(int kernel, int bytes) {
   int dev = 0;
@@ -112,7 +108,7 @@ int ensure_dyn_smem(int kernel, int bytes) {
   std::lock_guard<std::mutex> lock(g_smem_mu);
   int& cur = g_smem_limit[dev][kernel];
   const int want = std::max(cur, bytes);
-  if (cudaFuncSetAttribute((const void*)kSimKernel[kernel], cudaFuncAttributeMaxDynamicSharedMemorySize, want) != cudaSuccess) {
+  if (cudaFuncSetAttribute((const void*)hx::kSimKernel[kernel], cudaFuncAttributeMaxDynamicSharedMemorySize, want) != cudaSuccess) {
     cudaGetLastError();
     return fail(HX_ERR_CUDA, "cannot reserve " + std::to_string(want) +
                                  " bytes of shared memory for the simulation kernel");
@@ -194,8 +190,7 @@ struct hx_sim {
   // launch shape
   int blocks = 0, resident_warps = 0, smem_per_block = 0;
   bool generic = true;
-  int prefetch = 0;
-  int kernel = 1;  // which instantiation of the simulation kernel runs (kSimKernel)
+  int kernel = 1;  // which instantiation of the simulation kernel runs (hx::kSimKernel)
   int64_t scratch_bytes = 0, device_bytes = 0;
   cudaStream_t last_stream = nullptr;
   bool ran = false;
@@ -501,6 +496,24 @@ int per_warp_smem(const hx::ClusterK& ck) {
                        slot * ck.slot_entries, 16);
 }
 
+// The kernel for a cluster and up to *blocks blocks of it, and the blocks that
+// are resident at once.
+int launch_shape(bool generic, const hx::ClusterK& ck, const cudaDeviceProp& prop, int smem_per_block, int64_t* blocks,
+                 int* kernel) {
+  const int64_t want = std::max<int64_t>(*blocks, 1);
+  *kernel = sim_kernel_of(generic, ck, few_warps(want * hx::kWarpsPerBlock, prop.multiProcessorCount));
+  if (int rc = ensure_dyn_smem(*kernel, smem_per_block)) return rc;
+  int bps = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, (const void*)hx::kSimKernel[*kernel], hx::kWarpsPerBlock * 32,
+                                                    smem_per_block) != cudaSuccess ||
+      bps < 1) {
+    cudaGetLastError();
+    return fail(HX_ERR_CUDA, "simulation kernel does not fit on an SM");
+  }
+  *blocks = std::min<int64_t>(want, (int64_t)bps * prop.multiProcessorCount);
+  return HX_OK;
+}
+
 // Kernel-parameter copy of a validated cluster.
 void fill_cluster(const hx_cluster* cluster, hx::ClusterK& ck) {
   ck = hx::ClusterK{};
@@ -712,25 +725,14 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
     return bail(rc);
 
   h->generic = needs_generic(grid, ck, opt && opt->n_record > 0, opt && opt->force_generic, h->checked);
-  h->kernel = sim_kernel_of(h->generic, ck);
-  const void* kfn = (const void*)kSimKernel[h->kernel];
   // launch shape of the simulation kernel and its per-warp scratch
   h->smem_per_block = hx::kWarpsPerBlock * ck.smem_per_warp;
-  if ((rc = ensure_dyn_smem(h->kernel, h->smem_per_block))) return bail(rc);
-  int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kfn, hx::kWarpsPerBlock * 32, h->smem_per_block) !=
-          cudaSuccess ||
-      bps < 1) {
-    cudaGetLastError();
-    return bail(fail(HX_ERR_CUDA, "simulation kernel does not fit on an SM"));
-  }
-  int64_t blocks = (int64_t)bps * prop.multiProcessorCount;
+  int64_t blocks = (h->n_sims + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock;
   if (opt && opt->max_resident_warps > 0)
     blocks = std::min<int64_t>(blocks, std::max<int64_t>(1, opt->max_resident_warps / hx::kWarpsPerBlock));
-  blocks = std::min<int64_t>(blocks, (h->n_sims + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock);
-  h->blocks = (int)std::max<int64_t>(blocks, 1);
+  if ((rc = launch_shape(h->generic, ck, prop, h->smem_per_block, &blocks, &h->kernel))) return bail(rc);
+  h->blocks = (int)blocks;
   h->resident_warps = h->blocks * hx::kWarpsPerBlock;
-  h->prefetch = prefetch_records(h->resident_warps, prop.multiProcessorCount);
   // the simulations' order: the caller's subset, else possibly the costliest first
   h->work_order = subset.empty()
                       ? costliest_first(grid, n_traces, h->n_c, (int64_t)prop.l2CacheSize, h->resident_warps, &subset)
@@ -877,7 +879,6 @@ static int hx_sim_run_impl(hx_sim* h, void* stream) {
   for (int t = 0; t < HX_MAX_TENANTS; ++t) sa.tenant_topk_off[t] = h->tenant_topk_off[t];
   sa.subset = h->d_subset;
   sa.n_work = h->n_work;
-  sa.prefetch = h->prefetch;
   sa.checked = h->checked ? 1 : 0;
 
   hx::BestArgs ba;
@@ -896,7 +897,7 @@ static int hx_sim_run_impl(hx_sim* h, void* stream) {
   hx::hx_prep_kernel<<<prep_blocks, 256, 0, s>>>(pa, h->ck);
   HX_CUDA(cudaGetLastError());
   if (ev) HX_CUDA(cudaEventRecord(ev[1], s));
-  kSimKernel[h->kernel]<<<h->blocks, hx::kWarpsPerBlock * 32, h->smem_per_block, s>>>(sa, h->ck);
+  hx::kSimKernel[h->kernel]<<<h->blocks, hx::kWarpsPerBlock * 32, h->smem_per_block, s>>>(sa, h->ck);
   HX_CUDA(cudaGetLastError());
   if (ev) HX_CUDA(cudaEventRecord(ev[2], s));
   hx::hx_best_kernel<<<h->n_traces + 1, 256, 0, s>>>(ba);
@@ -1251,14 +1252,9 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
   HX_CUDA(cudaGetDeviceProperties(&prop, dev));
   const int smem_per_block = hx::kWarpsPerBlock * ck.smem_per_warp;
   const bool generic = needs_generic(grid, ck, false, false, false);
-  const int kernel = sim_kernel_of(generic, ck);
-  const void* kfn = (const void*)kSimKernel[kernel];
-  if ((rc = ensure_dyn_smem(kernel, smem_per_block))) return rc;
-  int bps = 0;
-  HX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kfn, hx::kWarpsPerBlock * 32, smem_per_block));
-  if (bps < 1) return fail(HX_ERR_CUDA, "simulation kernel does not fit on an SM");
-  int64_t blocks = std::min<int64_t>((int64_t)bps * prop.multiProcessorCount, fit_warps / hx::kWarpsPerBlock);
-  blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, (P + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock));
+  int64_t blocks = std::min<int64_t>(fit_warps / hx::kWarpsPerBlock, (P + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock);
+  int kernel = 0;
+  if ((rc = launch_shape(generic, ck, prop, smem_per_block, &blocks, &kernel))) return rc;
   const int64_t warps = blocks * hx::kWarpsPerBlock;
   const int64_t o_arena = fixed;
   const int64_t o_chains = o_arena + warps * align_up(arena_per_warp * (int64_t)sizeof(hx::HeapEnt), 256);
@@ -1345,7 +1341,6 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
   for (int t = 0; t < HX_MAX_TENANTS; ++t) sa.tenant_topk_off[t] = 0;
   sa.subset = nullptr;
   sa.n_work = P;
-  sa.prefetch = prefetch_records(warps, prop.multiProcessorCount);
   sa.checked = 0;
 
   hx::BestArgs ba;
@@ -1359,7 +1354,7 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
 
   hx::hx_prep_kernel<<<(unsigned)std::max<int64_t>(1, (nq + 255) / 256), 256, 0, s>>>(pa, ck);
   HX_CUDA(cudaGetLastError());
-  kSimKernel[kernel]<<<(unsigned)blocks, hx::kWarpsPerBlock * 32, smem_per_block, s>>>(sa, ck);
+  hx::kSimKernel[kernel]<<<(unsigned)blocks, hx::kWarpsPerBlock * 32, smem_per_block, s>>>(sa, ck);
   HX_CUDA(cudaGetLastError());
   hx::hx_best_kernel<<<2, 256, 0, s>>>(ba);
   HX_CUDA(cudaGetLastError());

@@ -135,7 +135,6 @@ struct SimArgs {
   int64_t tenant_topk_off[HX_MAX_TENANTS];  // tenant t's top-K heap within the warp's topk slice
   const int64_t* subset;    // [n_work] sims to run in work order, or NULL: all n_sims
   int64_t n_work;
-  int32_t prefetch;         // fetch a query's records into L1 as it arrives
   int32_t checked;          // check the scheduler's invariants after every event (generic kernel)
 };
 
@@ -215,16 +214,15 @@ struct BestArgs {
 };
 
 __global__ void hx_prep_kernel(PrepArgs a, ClusterK c);
-// hx_sim_kernel_lean: every point workload-balanced with the urgency queue,
-// nothing logged; hx_sim_kernel: any mix of dispatch and local-queue policies,
-// tenants and per-call logs; hx_sim_kernel_faults: those with fault windows.
-// Each for clusters of up to 64 instances, two a lane, and of up to 32, one a lane.
-__global__ void hx_sim_kernel_lean(SimArgs a, ClusterK c);
-__global__ void hx_sim_kernel_lean32(SimArgs a, ClusterK c);
-__global__ void hx_sim_kernel(SimArgs a, ClusterK c);
-__global__ void hx_sim_kernel32(SimArgs a, ClusterK c);
-__global__ void hx_sim_kernel_faults(SimArgs a, ClusterK c);
-__global__ void hx_sim_kernel_faults32(SimArgs a, ClusterK c);
+// The instantiations of the simulation kernel.  hx_sim_kernel_lean: every point
+// workload-balanced with the urgency queue, nothing logged; hx_sim_kernel: any
+// mix of dispatch and local-queue policies, tenants and per-call logs;
+// hx_sim_kernel_faults: those with fault windows.  Each for clusters of up to 64
+// instances, two a lane, and of up to 32, one a lane, and both for a full GPU
+// and for a run of few warps: kernel 4 * family + 2 * few + (one a lane).
+using SimKernel = void (*)(SimArgs, ClusterK);
+constexpr int kSimKernels = 12;
+extern const SimKernel kSimKernel[kSimKernels];
 __global__ void hx_best_kernel(BestArgs a);
 __global__ void hx_selftest_div_kernel(const uint64_t* n, const uint64_t* d, uint64_t* q, uint64_t* q_ref,
                                        int64_t count);

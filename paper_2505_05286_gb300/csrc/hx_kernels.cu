@@ -556,10 +556,12 @@ __device__ __noinline__ void log_dispatch(const SimArgs& a, int recj, int rid, i
 // Resident blocks per SM the register allocation aims for (4 warps each): 8
 // with one instance per lane; with two, 7, whose 72 registers hold a
 // simulation's state without spills (8 spill 48 bytes in the event loop: 8
-// traces x 20000 queries x 1024 points 503 ms against 458 ms).
+// traces x 20000 queries x 1024 points 503 ms against 458 ms).  A run of few
+// warps takes what registers it likes.
 #ifndef HX_SIM_MIN_BLOCKS
 #define HX_SIM_MIN_BLOCKS(J) ((J) == 1 ? 8 : 7)
 #endif
+constexpr int kFewMinBlocks = 5;
 
 // Bounds-checked build (-DHX_CHECKED): before every shared- or global-memory
 // access whose index the simulation forms from its own state (instance,
@@ -597,7 +599,7 @@ __device__ __noinline__ void log_dispatch(const SimArgs& a, int recj, int rid, i
 // warp-instructions per call event (8 traces x 2000 queries x 64 points, 8
 // instances: 14.2 -> 10.9 ms); 32 instances, 19 x 5003 x 512: 127 -> 89 ms; 64
 // instances, 8 x 20000 x 1024: 529 -> 460 ms.
-template <int J, bool kGeneric, bool kFaults>
+template <int J, bool kGeneric, bool kFaults, bool kFew>
 __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
   using T = typename Times<kFaults>::T;
   using Slot = typename Times<kFaults>::Slot;
@@ -967,7 +969,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         rel_first = (int32_t)(a.qcall[qbase + qa] - W->cb);
         HX_BOUND(rel_first >= 0 && rel_first < nc)
         rel_count = 1;
-        if (a.prefetch) {
+        if (kFew) {
           // the query's records into L1, 32 bytes a lane (a copy that nobody reads)
           const char* pa = reinterpret_cast<const char*>(rec + rel_first);
           const char* const pe = reinterpret_cast<const char*>(rec + (a.qcall[qbase + qa + 1] - W->cb));
@@ -1224,17 +1226,21 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
   }
 }
 
-#define HX_SIM_KERNEL(name, J, generic, faults)                                                              \
-  __global__ void __launch_bounds__(kWarpsPerBlock * 32, HX_SIM_MIN_BLOCKS(J)) name(SimArgs a, ClusterK c) { \
-    sim_body<J, generic, faults>(a, c);                                                                      \
+#define HX_SIM_KERNEL(name, generic, faults)                                                                      \
+  template <int J, bool kFew>                                                                                     \
+  __global__ void __launch_bounds__(kWarpsPerBlock * 32, kFew ? kFewMinBlocks : HX_SIM_MIN_BLOCKS(J))             \
+      name(SimArgs a, ClusterK c) {                                                                               \
+    sim_body<J, generic, faults, kFew>(a, c);                                                                     \
   }
-HX_SIM_KERNEL(hx_sim_kernel_lean, 2, false, false)
-HX_SIM_KERNEL(hx_sim_kernel_lean32, 1, false, false)
-HX_SIM_KERNEL(hx_sim_kernel, 2, true, false)
-HX_SIM_KERNEL(hx_sim_kernel32, 1, true, false)
-HX_SIM_KERNEL(hx_sim_kernel_faults, 2, true, true)
-HX_SIM_KERNEL(hx_sim_kernel_faults32, 1, true, true)
+HX_SIM_KERNEL(hx_sim_kernel_lean, false, false)
+HX_SIM_KERNEL(hx_sim_kernel, true, false)
+HX_SIM_KERNEL(hx_sim_kernel_faults, true, true)
 #undef HX_SIM_KERNEL
+
+#define HX_FORMS(name) name<2, false>, name<1, false>, name<2, true>, name<1, true>
+const SimKernel kSimKernel[kSimKernels] = {HX_FORMS(hx_sim_kernel_lean), HX_FORMS(hx_sim_kernel),
+                                           HX_FORMS(hx_sim_kernel_faults)};
+#undef HX_FORMS
 
 // ---------------------------------------------------------- best kernel
 namespace {
