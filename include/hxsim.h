@@ -162,8 +162,7 @@ typedef struct hx_grid {
 } hx_grid;
 
 typedef struct hx_options {
-  int32_t n_record;                 /* >= 0 simulations whose per-call log is kept (runs
-                                       the generic kernel) */
+  int32_t n_record;                 /* >= 0 simulations whose per-call log is kept */
   const int32_t* record_sims;       /* [n_record] distinct sim indices (trace * P + point) */
   int32_t max_resident_warps;       /* 0 = fill the GPU */
   int32_t timing;                   /* 1 = time each kernel with CUDA events */
@@ -360,8 +359,8 @@ typedef struct hx_info {
   int32_t warps_per_block;
   int32_t blocks;
   int32_t smem_per_block;
-  int32_t generic_kernel;       /* 1: the kernel with logging and every policy; 0: the
-                                   PQ + workload-balanced instantiation without logging */
+  int32_t generic_kernel;       /* 0: the PQ + workload-balanced instantiation without
+                                   logging; 1: any other (logging, policies, tenants, faults) */
   int32_t work_order;           /* order the simulations are taken in: 0 trace-major, highest
                                    point first; 1 the caller's subset (likewise ordered);
                                    2 every trace's workload-balanced alpha = 1 points first

@@ -92,8 +92,8 @@ int g_smem_limit[kMaxDevices][hx::kSimKernels] = {};  // [device][kernel]
 // warps.  That one fetches a query's records into L1 as it arrives (an event
 // reads two sectors of them that would come from L2 otherwise, about a fifth of
 // its latency) and may use twice the registers.
-int sim_kernel_of(bool generic, const hx::ClusterK& ck, bool few) {
-  return 4 * (!generic ? 0 : ck.n_faults == 0 ? 1 : 2) + (few ? 2 : 0) + (ck.n_inst <= 32 ? 1 : 0);
+int sim_kernel_of(int family, const hx::ClusterK& ck, bool few) {
+  return 4 * family + (few ? 2 : 0) + (ck.n_inst <= 32 ? 1 : 0);
 }
 
 // Few warps: up to 12 per SM, whose active queries fit L1 (the fetch alone: 512
@@ -117,14 +117,15 @@ int ensure_dyn_smem(int kernel, int bytes) {
   return HX_OK;
 }
 
-// The lean instantiation serves grids that are all workload-balanced dispatch
-// with the urgency queue, log nothing, check nothing, count one tenant and
-// have no fault windows.
-bool needs_generic(const hx_grid* grid, const hx::ClusterK& ck, bool record, bool force, bool checked) {
-  if (record || force || checked || ck.n_tenants > 1 || ck.n_faults > 0) return true;
+// The family of the simulation kernel that serves a run: the lean one serves
+// grids that are all workload-balanced dispatch with the urgency queue, log
+// nothing, check nothing, count one tenant and have no fault windows.
+int sim_family(const hx_grid* grid, const hx::ClusterK& ck, bool record, bool force, bool checked) {
+  if (ck.n_faults > 0) return hx::kSimFaults;
+  bool generic = force || checked || ck.n_tenants > 1;
   for (int p = 0; p < grid->n_points; ++p)
-    if (grid->local_policy[p] != HX_LOCAL_PQ || grid->dispatch_policy[p] != HX_DISPATCH_WB) return true;
-  return false;
+    generic |= grid->local_policy[p] != HX_LOCAL_PQ || grid->dispatch_policy[p] != HX_DISPATCH_WB;
+  return generic ? hx::kSimGeneric : record ? hx::kSimLog : hx::kSimLean;
 }
 
 }  // namespace
@@ -159,7 +160,7 @@ struct hx_sim {
   // device: derived and outputs
   hx::CallRec* d_rec = nullptr;
   hx_result* d_results = nullptr;
-  hx_extra* d_extras = nullptr;  // generic kernel only
+  hx_extra* d_extras = nullptr;  // generic families only
   unsigned long long* d_counter = nullptr;
   hx::BestCand* d_best_trace = nullptr;
   hx::BestCand* d_best_global = nullptr;
@@ -176,6 +177,7 @@ struct hx_sim {
   int32_t n_record = 0;
   int64_t rec_stride = 0;
   int32_t* d_rec_map = nullptr;
+  int32_t* d_rec_sims = nullptr;
   // run only these simulations, in work order (NULL: all of them)
   int64_t* d_subset = nullptr;  // the work order when not the kernel's own (see work_order)
   int64_t n_work = 0;
@@ -189,7 +191,7 @@ struct hx_sim {
   std::vector<int32_t> record_sims;
   // launch shape
   int blocks = 0, resident_warps = 0, smem_per_block = 0;
-  bool generic = true;
+  int family = hx::kSimGeneric;
   int kernel = 1;  // which instantiation of the simulation kernel runs (hx::kSimKernel)
   int64_t scratch_bytes = 0, device_bytes = 0;
   cudaStream_t last_stream = nullptr;
@@ -498,10 +500,10 @@ int per_warp_smem(const hx::ClusterK& ck) {
 
 // The kernel for a cluster and up to *blocks blocks of it, and the blocks that
 // are resident at once.
-int launch_shape(bool generic, const hx::ClusterK& ck, const cudaDeviceProp& prop, int smem_per_block, int64_t* blocks,
+int launch_shape(int family, const hx::ClusterK& ck, const cudaDeviceProp& prop, int smem_per_block, int64_t* blocks,
                  int* kernel) {
   const int64_t want = std::max<int64_t>(*blocks, 1);
-  *kernel = sim_kernel_of(generic, ck, few_warps(want * hx::kWarpsPerBlock, prop.multiProcessorCount));
+  *kernel = sim_kernel_of(family, ck, few_warps(want * hx::kWarpsPerBlock, prop.multiProcessorCount));
   if (int rc = ensure_dyn_smem(*kernel, smem_per_block)) return rc;
   int bps = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, (const void*)hx::kSimKernel[*kernel], hx::kWarpsPerBlock * 32,
@@ -724,13 +726,13 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
       (rc = upload(h->d_dp, grid->dispatch_policy, h->n_points, s0)))
     return bail(rc);
 
-  h->generic = needs_generic(grid, ck, opt && opt->n_record > 0, opt && opt->force_generic, h->checked);
+  h->family = sim_family(grid, ck, opt && opt->n_record > 0, opt && opt->force_generic, h->checked);
   // launch shape of the simulation kernel and its per-warp scratch
   h->smem_per_block = hx::kWarpsPerBlock * ck.smem_per_warp;
   int64_t blocks = (h->n_sims + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock;
   if (opt && opt->max_resident_warps > 0)
     blocks = std::min<int64_t>(blocks, std::max<int64_t>(1, opt->max_resident_warps / hx::kWarpsPerBlock));
-  if ((rc = launch_shape(h->generic, ck, prop, h->smem_per_block, &blocks, &h->kernel))) return bail(rc);
+  if ((rc = launch_shape(h->family, ck, prop, h->smem_per_block, &blocks, &h->kernel))) return bail(rc);
   h->blocks = (int)blocks;
   h->resident_warps = h->blocks * hx::kWarpsPerBlock;
   // the simulations' order: the caller's subset, else possibly the costliest first
@@ -746,7 +748,7 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   if (opt && opt->arena_entries > 0) h->arena_per_warp = opt->arena_entries;
   h->chains_per_warp = align_up(std::max(h->max_nq, 1), 256);
   h->topk_per_warp = align_up(h->max_kcap, 32);
-  if (h->generic && ck.n_tenants > 1) {
+  if (ck.n_tenants > 1) {
     // one more heap per tenant after the simulation's own, each sized for a
     // whole trace (a tenant's K never exceeds its trace's), so uploads of new
     // tenant assignments need no reallocation
@@ -761,7 +763,7 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   if ((rc = h->alloc(&h->d_arena, w * h->arena_per_warp)) || (rc = h->alloc(&h->d_chains, w * h->chains_per_warp)) ||
       (rc = h->alloc(&h->d_topk, w * h->topk_per_warp)))
     return bail(rc);
-  if (h->generic && (rc = h->alloc(&h->d_extras, h->n_sims))) return bail(rc);
+  if (h->family >= hx::kSimGeneric && (rc = h->alloc(&h->d_extras, h->n_sims))) return bail(rc);
   h->scratch_bytes = w * (h->arena_per_warp * (int64_t)sizeof(hx::HeapEnt) + h->chains_per_warp +
                           h->topk_per_warp * (int64_t)sizeof(int64_t));
 
@@ -776,10 +778,12 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
       h->record_sims.push_back(sim);
     }
     const int64_t n = (int64_t)h->n_record * h->rec_stride;
-    if ((rc = h->alloc(&h->d_rec_map, h->n_sims)) || (rc = h->alloc(&h->d_rec_inst, n)) ||
+    if ((rc = h->alloc(&h->d_rec_map, h->n_sims)) || (rc = h->alloc(&h->d_rec_sims, h->n_record)) ||
+        (rc = h->alloc(&h->d_rec_inst, n)) ||
         (rc = h->alloc(&h->d_rec_enq, n)) || (rc = h->alloc(&h->d_rec_budget, n)) ||
         (rc = h->alloc(&h->d_rec_start, n)) || (rc = h->alloc(&h->d_rec_end, n)) ||
-        (rc = upload(h->d_rec_map, map.data(), h->n_sims, s0)))
+        (rc = upload(h->d_rec_map, map.data(), h->n_sims, s0)) ||
+        (rc = upload(h->d_rec_sims, opt->record_sims, h->n_record, s0)))
       return bail(rc);
     if (cudaStreamSynchronize(s0) != cudaSuccess) return bail(fail(HX_ERR_CUDA, "record map upload failed"));
   }
@@ -870,7 +874,6 @@ static int hx_sim_run_impl(hx_sim* h, void* stream) {
   sa.rec_map = h->d_rec_map;
   sa.rec_inst = h->d_rec_inst;
   sa.rec_enq = h->d_rec_enq;
-  sa.rec_budget = h->d_rec_budget;
   sa.rec_start = h->d_rec_start;
   sa.rec_end = h->d_rec_end;
   sa.rec_stride = h->rec_stride;
@@ -899,6 +902,21 @@ static int hx_sim_run_impl(hx_sim* h, void* stream) {
   if (ev) HX_CUDA(cudaEventRecord(ev[1], s));
   hx::kSimKernel[h->kernel]<<<h->blocks, hx::kWarpsPerBlock * 32, h->smem_per_block, s>>>(sa, h->ck);
   HX_CUDA(cudaGetLastError());
+  if (h->n_record > 0) {
+    hx::LogArgs la;
+    la.rec = h->d_rec;
+    la.c_off = h->d_c_off;
+    la.rho = h->d_rho;
+    la.record_sims = h->d_rec_sims;
+    la.n_record = h->n_record;
+    la.n_points = h->n_points;
+    la.rec_enq = h->d_rec_enq;
+    la.rec_budget = h->d_rec_budget;
+    la.rec_stride = h->rec_stride;
+    const int64_t log_blocks = (h->rec_stride + 255) / 256 * h->n_record;
+    hx::hx_log_kernel<<<(unsigned)std::min<int64_t>(log_blocks, 1 << 16), 256, 0, s>>>(la, h->ck);
+    HX_CUDA(cudaGetLastError());
+  }
   if (ev) HX_CUDA(cudaEventRecord(ev[2], s));
   hx::hx_best_kernel<<<h->n_traces + 1, 256, 0, s>>>(ba);
   HX_CUDA(cudaGetLastError());
@@ -929,7 +947,7 @@ static int hx_sim_extras_impl(hx_sim* h, hx_extra* host_out, size_t n) {
     HX_CUDA(cudaMemcpy(host_out, h->d_extras, n * sizeof(hx_extra), cudaMemcpyDeviceToHost));
     return HX_OK;
   }
-  // the lean kernel serves one tenant without faults: everything is tenant 0
+  // the lean and logging families serve one tenant without faults: everything is tenant 0
   std::vector<hx_result> res(n);
   HX_CUDA(cudaMemcpy(res.data(), h->d_results, n * sizeof(hx_result), cudaMemcpyDeviceToHost));
   for (size_t i = 0; i < n; ++i) {
@@ -1128,7 +1146,7 @@ int hx_sim_info(hx_sim* h, hx_info* out) {
   out->warps_per_block = hx::kWarpsPerBlock;
   out->blocks = h->blocks;
   out->smem_per_block = h->smem_per_block;
-  out->generic_kernel = h->generic ? 1 : 0;
+  out->generic_kernel = h->family != hx::kSimLean ? 1 : 0;
   out->work_order = h->work_order;
   return HX_OK;
 }
@@ -1251,10 +1269,10 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
   HX_CUDA(cudaGetDevice(&dev));
   HX_CUDA(cudaGetDeviceProperties(&prop, dev));
   const int smem_per_block = hx::kWarpsPerBlock * ck.smem_per_warp;
-  const bool generic = needs_generic(grid, ck, false, false, false);
+  const int family = sim_family(grid, ck, false, false, false);
   int64_t blocks = std::min<int64_t>(fit_warps / hx::kWarpsPerBlock, (P + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock);
   int kernel = 0;
-  if ((rc = launch_shape(generic, ck, prop, smem_per_block, &blocks, &kernel))) return rc;
+  if ((rc = launch_shape(family, ck, prop, smem_per_block, &blocks, &kernel))) return rc;
   const int64_t warps = blocks * hx::kWarpsPerBlock;
   const int64_t o_arena = fixed;
   const int64_t o_chains = o_arena + warps * align_up(arena_per_warp * (int64_t)sizeof(hx::HeapEnt), 256);
@@ -1332,7 +1350,6 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
   sa.rec_map = nullptr;
   sa.rec_inst = nullptr;
   sa.rec_enq = nullptr;
-  sa.rec_budget = nullptr;
   sa.rec_start = nullptr;
   sa.rec_end = nullptr;
   sa.rec_stride = 0;

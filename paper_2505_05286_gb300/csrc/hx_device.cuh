@@ -125,7 +125,6 @@ struct SimArgs {
   const int32_t* rec_map;   // [n_sims] record slot or -1; NULL when not recording
   int32_t* rec_inst;
   int64_t* rec_enq;
-  int64_t* rec_budget;
   int64_t* rec_start;
   int64_t* rec_end;
   int64_t rec_stride;
@@ -203,6 +202,17 @@ struct BestCand {
   int32_t flags;  // bit0 valid, bit1 feasible
 };
 
+struct LogArgs {
+  const CallRec* rec;
+  const int64_t* c_off;
+  const int32_t* rho;
+  const int32_t* record_sims;  // [n_record]
+  int32_t n_record, n_points;
+  const int64_t* rec_enq;
+  int64_t* rec_budget;
+  int64_t rec_stride;
+};
+
 struct BestArgs {
   const hx_result* results;
   const int64_t* q_off;
@@ -215,14 +225,17 @@ struct BestArgs {
 
 __global__ void hx_prep_kernel(PrepArgs a, ClusterK c);
 // The instantiations of the simulation kernel.  hx_sim_kernel_lean: every point
-// workload-balanced with the urgency queue, nothing logged; hx_sim_kernel: any
-// mix of dispatch and local-queue policies, tenants and per-call logs;
-// hx_sim_kernel_faults: those with fault windows.  Each for clusters of up to 64
-// instances, two a lane, and of up to 32, one a lane, and both for a full GPU
-// and for a run of few warps: kernel 4 * family + 2 * few + (one a lane).
+// workload-balanced with the urgency queue, nothing logged; hx_sim_kernel_log:
+// with per-call logs; hx_sim_kernel: those and any mix of dispatch and
+// local-queue policies, tenants and event checks; hx_sim_kernel_faults: all of
+// it with fault windows.  Each for clusters of up to 64 instances, two a lane,
+// and of up to 32, one a lane, and both for a full GPU and for a run of few
+// warps: kernel 4 * family + 2 * few + (one a lane).
+enum { kSimLean = 0, kSimLog = 1, kSimGeneric = 2, kSimFaults = 3 };
 using SimKernel = void (*)(SimArgs, ClusterK);
-constexpr int kSimKernels = 12;
+constexpr int kSimKernels = 16;
 extern const SimKernel kSimKernel[kSimKernels];
+__global__ void hx_log_kernel(LogArgs a, ClusterK c);
 __global__ void hx_best_kernel(BestArgs a);
 __global__ void hx_selftest_div_kernel(const uint64_t* n, const uint64_t* d, uint64_t* q, uint64_t* q_ref,
                                        int64_t count);

@@ -120,6 +120,24 @@ __device__ __forceinline__ int64_t cost_on_type(const ClusterK& c, int t, int64_
   return ceil_div_pos(prompt * kUsPerS, c.prefill[t]) + out * (int64_t)c.decode[t];
 }
 
+// Rest of a request's own path after it (the budget denominator minus its own
+// mean cost), by CallRec::fcode: stage reference costs, i.e. means over instances
+// of Eq. (comp) at the stage's reference tokens, for G, min(rho, R - u)
+// corrections and E.
+__device__ __forceinline__ int64_t rest_of_path(const ClusterK& c, int64_t rho, int row) {
+  int64_t cref[4];
+  for (int s = 0; s < 4; ++s) {
+    int64_t sum = 0;
+    for (int ty = 0; ty < c.n_types; ++ty) sum += cost_on_type(c, ty, c.ref_prompt[s], c.ref_out[s]) * c.cnt[ty];
+    cref[s] = sum / c.n_inst;
+  }
+  const int64_t rmax = c.rmax;
+  if (row == 0) return cref[HX_STAGE_G] + (rho < rmax ? rho : rmax) * cref[HX_STAGE_C] + cref[HX_STAGE_E];
+  if (row == kFRows - 1) return 0;
+  const int64_t left = rmax - (row - 1);
+  return (rho < left ? rho : left) * cref[HX_STAGE_C] + cref[HX_STAGE_E];
+}
+
 // ------------------------------------------------------------- prep kernel
 // One thread per query: Eq. (comp) per call and type, tbar, chain successor
 // links and the deadline arrival + slo_mult * L0 (L0 = S + slowest
@@ -544,13 +562,6 @@ __device__ __forceinline__ void finish_query(WarpShared* W, int64_t now, int64_t
   if (W->tk < W->kcap || v > W->tkmin) topk_insert_warp(W->topk, &W->tk, W->kcap, &W->tkmin, v, lane);
 }
 
-__device__ __noinline__ void log_dispatch(const SimArgs& a, int recj, int rid, int m, int64_t now, int64_t budget) {
-  const int64_t o = (int64_t)recj * a.rec_stride + rid;
-  a.rec_inst[o] = m;
-  a.rec_enq[o] = now;
-  a.rec_budget[o] = budget;
-}
-
 }  // namespace
 
 // Resident blocks per SM the register allocation aims for (4 warps each): 8
@@ -599,8 +610,9 @@ constexpr int kFewMinBlocks = 5;
 // warp-instructions per call event (8 traces x 2000 queries x 64 points, 8
 // instances: 14.2 -> 10.9 ms); 32 instances, 19 x 5003 x 512: 127 -> 89 ms; 64
 // instances, 8 x 20000 x 1024: 529 -> 460 ms.
-template <int J, bool kGeneric, bool kFaults, bool kFew>
+template <int J, int kFamily, bool kFew>
 __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
+  constexpr bool kLog = kFamily >= kSimLog, kGeneric = kFamily >= kSimGeneric, kFaults = kFamily == kSimFaults;
   using T = typename Times<kFaults>::T;
   using Slot = typename Times<kFaults>::Slot;
   constexpr T kIdle = ~T(0);                      // no running call; no arrival in range
@@ -672,29 +684,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     }
     // no chain of any query has finished
     for (int i = 16 * lane; i < nq; i += 512) *reinterpret_cast<uint4*>(W->chains + i) = make_uint4(0, 0, 0, 0);
-    if (lane < kFRows) {
-      // rest of the request's own path after it (the budget denominator minus
-      // its own mean cost): stage reference costs, i.e. means over instances of
-      // Eq. (comp) at the stage's reference tokens, for G, min(rho, R - u)
-      // corrections and E
-      int64_t cref[4];
-      for (int s = 0; s < 4; ++s) {
-        int64_t sum = 0;
-        for (int ty = 0; ty < c.n_types; ++ty) sum += cost_on_type(c, ty, c.ref_prompt[s], c.ref_out[s]) * c.cnt[ty];
-        cref[s] = sum / N;
-      }
-      const int64_t rho = a.rho[p], rmax = c.rmax;
-      int64_t f;
-      if (lane == 0) {
-        f = cref[HX_STAGE_G] + (rho < rmax ? rho : rmax) * cref[HX_STAGE_C] + cref[HX_STAGE_E];
-      } else if (lane == kFRows - 1) {
-        f = 0;
-      } else {
-        const int64_t left = rmax - (lane - 1);
-        f = (rho < left ? rho : left) * cref[HX_STAGE_C] + cref[HX_STAGE_E];
-      }
-      W->frest[lane] = f;
-    }
+    if (lane < kFRows) W->frest[lane] = rest_of_path(c, a.rho[p], lane);
     if (lane == 0) {
       const int64_t A = a.alpha[p];
       W->A = (int32_t)A;
@@ -749,7 +739,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     }
 
     // the record slot of a logged simulation, or -1; the dispatch policy
-    const int recj = kGeneric && a.rec_map ? a.rec_map[sim] : -1;
+    const int recj = kLog && a.rec_map ? a.rec_map[sim] : -1;
     const bool round_robin = kGeneric && a.dpol[p] == HX_DISPATCH_RR;
 
     // times are relative to base; an arrival 2^32 us or more past it reads as kIdle
@@ -820,7 +810,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         e.tag = tag;
         if constexpr (kFaults) e.fail = fail ? 1u : 0u;
         slots[slot_base + s] = e;
-        if (kGeneric && recj >= 0) {
+        if (kLog && recj >= 0) {
           a.rec_start[(int64_t)recj * a.rec_stride + rid] = absolute(now);
           a.rec_end[(int64_t)recj * a.rec_stride + rid] = absolute(end);
         }
@@ -1039,12 +1029,13 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         const int est = low ? ev[0].x : ev[J - 1].x, svc = low ? ev[0].y : ev[J - 1].y;
 #pragma unroll
         for (int j = 0; j < J; ++j) q[j] += lane + 32 * j == m ? est : 0;
-        if (kGeneric && recj >= 0) {
+        if (kLog && recj >= 0) {
+          // (the budget at send time follows from these: hx_log_kernel)
           HX_BOUND(rid < a.rec_stride)
-          const int4 tail = *reinterpret_cast<const int4*>(&r->tbar);
-          const int64_t t_abs = absolute(now);
-          const int64_t budget = slo_budget(r->deadline - t_abs, tail.x, tail.x + W->frest[(tail.w >> 16) & 0xff]);
-          if (lane == 0) log_dispatch(a, recj, rid, m, t_abs, budget);
+          if (lane == 0) {
+            a.rec_inst[(int64_t)recj * a.rec_stride + rid] = m;
+            a.rec_enq[(int64_t)recj * a.rec_stride + rid] = absolute(now);
+          }
         }
         // nothing of this event waits yet, m's queue is empty and m has a free
         // slot for this request and every one still to be dispatched in this
@@ -1226,21 +1217,45 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
   }
 }
 
-#define HX_SIM_KERNEL(name, generic, faults)                                                                      \
-  template <int J, bool kFew>                                                                                     \
-  __global__ void __launch_bounds__(kWarpsPerBlock * 32, kFew ? kFewMinBlocks : HX_SIM_MIN_BLOCKS(J))             \
-      name(SimArgs a, ClusterK c) {                                                                               \
-    sim_body<J, generic, faults, kFew>(a, c);                                                                     \
+#define HX_SIM_KERNEL(name, family)                                                                   \
+  template <int J, bool kFew>                                                                         \
+  __global__ void __launch_bounds__(kWarpsPerBlock * 32, kFew ? kFewMinBlocks : HX_SIM_MIN_BLOCKS(J)) \
+      name(SimArgs a, ClusterK c) {                                                                   \
+    sim_body<J, family, kFew>(a, c);                                                                  \
   }
-HX_SIM_KERNEL(hx_sim_kernel_lean, false, false)
-HX_SIM_KERNEL(hx_sim_kernel, true, false)
-HX_SIM_KERNEL(hx_sim_kernel_faults, true, true)
+HX_SIM_KERNEL(hx_sim_kernel_lean, kSimLean)
+HX_SIM_KERNEL(hx_sim_kernel_log, kSimLog)
+HX_SIM_KERNEL(hx_sim_kernel, kSimGeneric)
+HX_SIM_KERNEL(hx_sim_kernel_faults, kSimFaults)
 #undef HX_SIM_KERNEL
 
 #define HX_FORMS(name) name<2, false>, name<1, false>, name<2, true>, name<1, true>
-const SimKernel kSimKernel[kSimKernels] = {HX_FORMS(hx_sim_kernel_lean), HX_FORMS(hx_sim_kernel),
-                                           HX_FORMS(hx_sim_kernel_faults)};
+const SimKernel kSimKernel[kSimKernels] = {HX_FORMS(hx_sim_kernel_lean), HX_FORMS(hx_sim_kernel_log),
+                                           HX_FORMS(hx_sim_kernel), HX_FORMS(hx_sim_kernel_faults)};
 #undef HX_FORMS
+
+// ----------------------------------------------------------- log kernel
+// The SLO budget at send time (Sec. 4.2) of every logged dispatch, one thread
+// per call of a logged simulation: its division (a hundred instructions) in the
+// event loop would lengthen the logged simulation's chain, which one window's
+// sweep waits for.
+__global__ void __launch_bounds__(256) hx_log_kernel(LogArgs a, ClusterK c) {
+  __shared__ int64_t rest[kFRows];
+  const int64_t per = (a.rec_stride + 255) / 256;  // blocks of calls per simulation
+  for (int64_t b = blockIdx.x; b < per * a.n_record; b += gridDim.x) {
+    const int64_t j = b / per;
+    const int64_t sim = a.record_sims[j], t = sim / a.n_points;
+    __syncthreads();
+    if (threadIdx.x < kFRows) rest[threadIdx.x] = rest_of_path(c, a.rho[sim - t * a.n_points], threadIdx.x);
+    __syncthreads();
+    const int64_t rid = (b - j * per) * 256 + threadIdx.x;
+    if (rid < a.c_off[t + 1] - a.c_off[t]) {
+      const CallRec* const r = a.rec + a.c_off[t] + rid;
+      const int64_t o = j * a.rec_stride + rid, dd = r->tbar + rest[r->fcode];
+      a.rec_budget[o] = slo_budget(r->deadline - a.rec_enq[o], r->tbar, dd);
+    }
+  }
+}
 
 // ---------------------------------------------------------- best kernel
 namespace {
