@@ -293,6 +293,18 @@ __device__ __forceinline__ bool before(uint64_t e0, uint32_t tag0, uint64_t e1, 
   return (e0 < e1) | ((e0 == e1) & (tag0 < tag1));
 }
 
+// A value that every lane holds alike, broadcast so that the compiler knows it:
+// branches on such values need no reconvergence code, and warp-wide operations
+// behind them no check that the warp is whole.
+// Every branch of the event loop that leads to a warp-wide operation is on a
+// broadcast or voted value: 195 -> 171 warp-instructions per event (no BRA.DIV,
+// a tenth of the BSSY / BSYNC), 8 x 2000 queries x 64 points 7.6 -> 6.8 ms,
+// alpha = 1 on 64 instances 3226 -> 2788 cycles per event.
+template <class T>
+__device__ __forceinline__ T uniform(T v) {
+  return __shfl_sync(kFull, v, 0);
+}
+
 __device__ __forceinline__ uint32_t warp_min(uint32_t v) { return __reduce_min_sync(kFull, v); }
 __device__ __forceinline__ uint64_t warp_min(uint64_t v) { return warp_min_u64(v); }
 
@@ -426,7 +438,8 @@ __device__ __forceinline__ void heap_sift_warp(HeapEnt* h, int m, HeapEnt sink, 
 __device__ __noinline__ void topk_insert_warp(int64_t* h, int32_t* size, int kcap, int64_t* root_out, int64_t v,
                                               int lane) {
   __builtin_assume(__isGlobal(h));
-  const int n = *size;
+  const int n = uniform(*size);
+  kcap = uniform(kcap);
   if (n < kcap) {
     // filling: sift up on lane 0 (few levels)
     if (lane == 0) {
@@ -443,7 +456,7 @@ __device__ __noinline__ void topk_insert_warp(int64_t* h, int32_t* size, int kca
     __syncwarp();
     *size = n + 1;
     if (n + 1 == kcap) *root_out = h[0];
-  } else if (v > *root_out) {
+  } else if (__any_sync(kFull, v > *root_out)) {
     // v replaces the root and sinks; one lane per child (latencies are >= 0)
     int i = 0;
     int64_t root = v;
@@ -453,7 +466,7 @@ __device__ __noinline__ void topk_insert_warp(int64_t* h, int32_t* size, int kca
       const int ch = first + lane;
       const uint64_t cv = ch < n ? (uint64_t)h[ch] : ~0ull;
       const uint64_t mn = warp_min_u64(cv);
-      if (mn >= (uint64_t)v) break;
+      if (__any_sync(kFull, mn >= (uint64_t)v)) break;
       const int b = __ffs(__ballot_sync(kFull, cv == mn)) - 1;
       if (i == 0) root = (int64_t)mn;
       if (lane == 0) h[i] = (int64_t)mn;
@@ -500,12 +513,12 @@ __device__ __forceinline__ int push_pending(WarpShared* W, InstState* I, HeapEnt
                                             int lane) {
   HeapEnt* const arena = W->arena;
   __builtin_assume(__isGlobal(arena));
-  const int size = I->hsize, np = __popc(pm);
-  const uint32_t heap = I->heap;
+  const int size = uniform(I->hsize), np = __popc(pm);
+  const uint32_t heap = uniform(I->heap);
   const int hcl = (int)(heap >> kHeapCodeShift), cap = hcl ? 8 << hcl : 0;
   int hoff = (int)(heap & kHeapOffMask);
   if (size + np > cap) {
-    const int ncap = cap ? 2 * cap : 16, bump = W->bump, off = hoff;
+    const int ncap = cap ? 2 * cap : 16, bump = uniform(W->bump), off = hoff;
     if ((int64_t)bump + ncap > arena_per_warp) return HX_ERR_CAPACITY;
     hoff = bump;
     for (int i = lane; i < size; i += 32) arena[hoff + i] = arena[off + i];
@@ -559,7 +572,7 @@ __device__ __forceinline__ void finish_query(WarpShared* W, int64_t now, int64_t
   W->makespan = now;
   // most latencies of a full heap fall below its root and change nothing
   const int64_t v = now - arrival;
-  if (W->tk < W->kcap || v > W->tkmin) topk_insert_warp(W->topk, &W->tk, W->kcap, &W->tkmin, v, lane);
+  if (__any_sync(kFull, (W->tk < W->kcap) | (v > W->tkmin))) topk_insert_warp(W->topk, &W->tk, W->kcap, &W->tkmin, v, lane);
 }
 
 }  // namespace
@@ -610,6 +623,12 @@ constexpr int kFewMinBlocks = 5;
 // warp-instructions per call event (8 traces x 2000 queries x 64 points, 8
 // instances: 14.2 -> 10.9 ms); 32 instances, 19 x 5003 x 512: 127 -> 89 ms; 64
 // instances, 8 x 20000 x 1024: 529 -> 460 ms.
+// The lane with the lowest tag (a call of its own: it is rare, and inlined it
+// would run predicated at every completion).
+__device__ __noinline__ unsigned lowest_id(uint32_t tag) {
+  return __ballot_sync(kFull, tag == __reduce_min_sync(kFull, tag));
+}
+
 template <int J, int kFamily, bool kFew>
 __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
   constexpr bool kLog = kFamily >= kSimLog, kGeneric = kFamily >= kSimGeneric, kFaults = kFamily == kSimFaults;
@@ -618,7 +637,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
   constexpr T kIdle = ~T(0);                      // no running call; no arrival in range
   constexpr T kFar = kFaults ? kIdle : T(1) << 31;  // an event this far moves the base up first
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5;
+  const int warp = uniform((int)(threadIdx.x >> 5));
   // volatile: read once and kept, not read again wherever it is used
   int lane;
   asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
@@ -643,7 +662,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
   for (;;) {
     unsigned long long work = 0;
     if (lane == 0) work = atomicAdd(a.work_counter, 1ull);
-    const int64_t w = (int64_t)__shfl_sync(kFull, work, 0);
+    const int64_t w = (int64_t)uniform(work);
     if (w >= a.n_work) break;
     // trace-major, so that concurrent simulations share a trace in L2; within a
     // trace the highest point index (highest alpha, the longest queues) first
@@ -660,9 +679,9 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     const int64_t sim = (int64_t)t * a.n_points + p;
     const long long clk0 = clock64();
     const int64_t qb = a.q_off[t];
-    const int32_t nq = (int32_t)(a.q_off[t + 1] - qb);
+    const int32_t nq = uniform((int32_t)(a.q_off[t + 1] - qb));
     const int64_t cb = a.c_off[t];
-    const int32_t nc = (int32_t)(a.c_off[t + 1] - cb);
+    const int32_t nc = uniform((int32_t)(a.c_off[t + 1] - cb));
     const CallRec* const rec = a.rec + cb;
     if (lane == 0) {
       W->qb = qb;
@@ -739,8 +758,21 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     }
 
     // the record slot of a logged simulation, or -1; the dispatch policy
-    const int recj = kLog && a.rec_map ? a.rec_map[sim] : -1;
-    const bool round_robin = kGeneric && a.dpol[p] == HX_DISPATCH_RR;
+    const int recj = kLog && a.rec_map ? uniform(a.rec_map[sim]) : -1;
+    const bool round_robin = kGeneric && uniform((int)a.dpol[p]) == HX_DISPATCH_RR;
+
+    // Eq. (comp) and the service time on this lane's instances of the request
+    // that is dispatched next
+    int2 cost_of[J];
+    auto load_costs = [&](int32_t rid) {
+#pragma unroll
+      for (int j = 0; j < J; ++j)
+        cost_of[j] = *reinterpret_cast<const int2*>(reinterpret_cast<const char*>(rec + rid) + lrec[j]);
+    };
+    // what a run of few warps has registers to keep
+    uint8_t* const chains0 = W->chains;
+    const longlong2 tie0 = W->tie;
+    const float4 fscore0 = W->fscore;
 
     // times are relative to base; an arrival 2^32 us or more past it reads as kIdle
     W->base = 0;
@@ -752,7 +784,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     auto absolute = [&](T t) -> int64_t { return kFaults ? (int64_t)t : W->base + (int64_t)t; };
     W->arrivals = 0;
     W->next_arrival = nq > 0 ? a.arrival[qb] : 0;
-    T arr = nq > 0 ? rel(a.arrival[qb]) : kIdle;
+    T arr = nq > 0 ? uniform(rel(a.arrival[qb])) : kIdle;
     T now = 0;
     int32_t status = HX_OK, npend = 0;
     // event bound; re-issued attempts add events while fault windows last
@@ -835,7 +867,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       if (((mn < arr ? mn : arr) >= kFar) | (steps_left == 0)) {
         // the end, too many events, or nothing within 2^31 us of the base, which
         // then moves to the next event
-        const bool more = W->arrivals < nq;
+        const bool more = uniform(W->arrivals) < nq;
         if (mn == kIdle && !more) break;
         if (steps_left-- == 0) {
           status = HX_ERR_STEP_LIMIT;
@@ -854,13 +886,13 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
           for (int j = lane; j < c.slot_entries; j += 32) slots[j].end -= shift;
           __syncwarp();
           W->base = nb;  // every lane writes the same value
-          arr = more ? rel(at) : kIdle;
+          arr = more ? uniform(rel(at)) : kIdle;
           continue;
         }
       }
       --steps_left;
       npend = 0;
-      int cm = -1, waiting = 0;  // the instance whose slot this event frees, and the requests waiting for it
+      int cm = -1, waiting = 0;  // the instance whose slot this event frees, and whether requests wait for it
       // requests released by this event: rel_first .. rel_first + rel_count - 1
       int32_t rel_first = 0, rel_count = 0;
       if (mn <= arr) {
@@ -881,17 +913,26 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         const InstState I = inst[m];
         const uint32_t slot_base = first_slot(m, I);
         HX_BOUND((int)slot_base + 16 <= c.slot_entries && hole < 16 && ((I.cfg & ~I.free) >> hole & 1u))
+        // what the completion does.  A run of few warps reads the query's finished
+        // chains and the first released request's costs before they are known to
+        // be needed, so that no branch delays the loads.
+        const int32_t qid = tail.z;
+        HX_BOUND(qid >= 0 && qid < nq && tail.y >= 0 && tail.y < nc)
+        const uint32_t tw = uniform((uint32_t)tail.w), what = tw >> kDoneShift;
+        uint8_t* const chains = (kFew ? chains0 : W->chains) + qid;
+        __builtin_assume(__isGlobal(chains));
+        int ended = 0;
+        if (kFew || what == kDoneChain) ended = *chains + 1;
+        if (kFew) load_costs(tail.y);
         // the slot is free; the next completion is the earliest of those still running
         const uint32_t free = I.free | 1u << hole;
-        const bool failed = kFaults && reinterpret_cast<const Slot64*>(slots)[slot_base + hole].fail != 0;
+        const bool failed = kFaults && __any_sync(kFull, reinterpret_cast<const Slot64*>(slots)[slot_base + hole].fail != 0);
         const Slot e = slots[slot_base + l16];
         const bool runs = (I.cfg & ~free & 0xffffu & lbit) != 0;
         const T nmin = warp_min(runs ? e.end : kIdle);
         unsigned nb = __ballot_sync(kFull, runs & (e.end == nmin));
         if (nb & (nb - 1)) {
-          // equal ends: the lowest request id
-          const uint32_t id = runs & (e.end == nmin) ? e.tag : 0xffffffffu;
-          nb = __ballot_sync(kFull, id == __reduce_min_sync(kFull, id));
+          nb = lowest_id(runs & (e.end == nmin) ? e.tag : 0xffffffffu);  // equal ends
         }
         const uint32_t ntag = __shfl_sync(kFull, e.tag, 31 - __clz(nb));
         inst[m].free = free;  // every lane stores the same mask
@@ -902,12 +943,16 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
           next_tag[j] = own ? ntag : next_tag[j];
           q[j] -= own ? est : 0;
         }
-        // the freed slot needs a batch boundary only if requests wait for it
+        // bit 0: the last chain ended, if one did; bit 1: requests wait for the
+        // freed slot (only then does it need a batch boundary)
+        const unsigned flags = __ballot_sync(kFull, lane == 0 ? ended == (int)(tw & 0xff) : I.hsize > 0);
         cm = m;
-        waiting = I.hsize;
-        const uint32_t what = (uint32_t)tail.w >> kDoneShift;
-        const int32_t qid = tail.z;
-        HX_BOUND(qid >= 0 && qid < nq)
+        waiting = flags & 2u;
+        // released: the next calls; at a chain's end the evaluation, if it is the last
+        const bool chain = (what == kDoneChain) & !failed;
+        rel_first = tail.y;
+        rel_count = chain ? flags & 1u : tw & 0xff;
+        if (chain) *chains = (uint8_t)ended;  // every lane writes the same byte
         if (kFaults && failed) {
           // the attempt timed out: the request goes out again, avoiding m
           const int32_t n = W->reissued + 1;
@@ -916,22 +961,11 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
           W->excl = c.n_inst > 1 ? m : -1;
           rel_first = rid;
           rel_count = 1;
-        } else if (what == kDoneRelease) {
-          rel_first = tail.y;
-          rel_count = tail.w & 0xff;
-        } else if (what == kDoneChain) {
-          // a chain of the query ended: the last one releases the evaluation
-          uint8_t* const chains = W->chains + qid;
-          __builtin_assume(__isGlobal(chains));
-          const int ended = *chains + 1;
-          __syncwarp();
-          *chains = (uint8_t)ended;  // every lane writes the same byte
-          rel_first = tail.y;
-          rel_count = ended == (tail.w & 0xff) ? 1 : 0;
-        } else {
+          if (kFew) load_costs(rid);
+        } else if (what == kDoneQuery) {
           const int64_t t_abs = absolute(now), dl = r->deadline, at = r->arrival;
           if (kGeneric) {
-            const int ten = (tail.w >> 8) & 0xff;
+            const int ten = (tw >> 8) & 0xff;
             HX_BOUND(ten < HX_MAX_TENANTS)
             if (lane == 0) {
               W->tdone[ten]++;
@@ -943,7 +977,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
               HX_BOUND(W->trace < a.n_traces && kc <= a.tenant_topk_off[0])
               const int64_t v = t_abs - at;
               __syncwarp();
-              if (W->ttk[ten] < kc || v > W->ttkmin[ten])
+              if (__any_sync(kFull, (W->ttk[ten] < kc) | (v > W->ttkmin[ten])))
                 topk_insert_warp(W->topk + a.tenant_topk_off[ten], &W->ttk[ten], kc, &W->ttkmin[ten], v, lane);
             }
           }
@@ -954,10 +988,11 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       } else {
         now = arr;
         const int64_t qbase = W->qb;
-        const int32_t qa = W->arrivals;
-        HX_BOUND(qa < W->nq)
+        const int32_t qa = uniform(W->arrivals);
+        HX_BOUND(qa < nq)
         rel_first = (int32_t)(a.qcall[qbase + qa] - W->cb);
         HX_BOUND(rel_first >= 0 && rel_first < nc)
+        if (kFew) load_costs(rel_first);
         rel_count = 1;
         if (kFew) {
           // the query's records into L1, 32 bytes a lane (a copy that nobody reads)
@@ -969,9 +1004,9 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         }
         __syncwarp();
         W->arrivals = qa + 1;  // every lane writes the same values
-        const int64_t at = qa + 1 < W->nq ? a.arrival[qbase + qa + 1] : 0;
+        const int64_t at = qa + 1 < nq ? a.arrival[qbase + qa + 1] : 0;
         W->next_arrival = at;
-        arr = qa + 1 < W->nq ? rel(at) : kIdle;
+        arr = qa + 1 < nq ? uniform(rel(at)) : kIdle;
       }
 
       // Sec. 4.1 for each released request, in request-id order: score every
@@ -979,23 +1014,23 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       // batch boundary below, and only if it has to wait).
       for (int32_t rid = rel_first; rel_count > 0; ++rid, --rel_count) {
         HX_BOUND(rid < nc)
-        const CallRec* const r = rec + rid;
-        // Eq. (comp) and the service time on this lane's instances
+        if (!kFew) load_costs(rid);
         int2 ev[J];
 #pragma unroll
-        for (int j = 0; j < J; ++j) ev[j] = *reinterpret_cast<const int2*>(reinterpret_cast<const char*>(r) + lrec[j]);
+        for (int j = 0; j < J; ++j) ev[j] = cost_of[j];
+        if (kFew && rel_count > 1) load_costs(rid + 1);
         int m;
         // a re-issued request avoids the instance it timed out on
-        const int excl = kFaults ? W->excl : -1;
+        const int excl = kFaults ? uniform(W->excl) : -1;
         if (kGeneric && round_robin) {
-          m = W->rr;
+          m = uniform(W->rr);
           if (m == excl) m = (m + 1 == N) ? 0 : m + 1;
           __syncwarp();
           W->rr = (m + 1 == N) ? 0 : m + 1;  // every lane writes the same value
         } else {
           // instances that tie in their reward and beat all others: the least cost wins
           // (the lowest instance at alpha = 0, where costs have no weight)
-          const longlong2 tie = W->tie;
+          const longlong2 tie = kFew ? tie0 : W->tie;
           uint32_t cost[J];
 #pragma unroll
           for (int j = 0; j < J; ++j) cost[j] = q[j] <= tie.x ? (uint32_t)ev[j].x & (uint32_t)tie.y : 0xffffffffu;
@@ -1006,7 +1041,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
             if (J == 2) b1 = __ballot_sync(kFull, cost[J - 1] == least);
             m = J == 1 || b0 ? __ffs(b0) - 1 : __ffs(b1) + 31;
           } else {
-            const float4 f = W->fscore;
+            const float4 f = kFew ? fscore0 : W->fscore;
             ScoreRange s[J];
 #pragma unroll
             for (int j = 0; j < J; ++j) s[j] = score_range(q[j], ev[j].x, f, neg_a[j]);
@@ -1042,7 +1077,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         // event: the batch boundary below would start it now whatever the others
         // do, so it starts at once
         const InstState I = inst[m];
-        if (((npend | I.hsize) == 0) & (__popc(I.free) >= rel_count)) {
+        if (__all_sync(kFull, ((npend | I.hsize) == 0) & (__popc(I.free) >= rel_count))) {
           start_call(m, I.free, first_slot(m, I), rid, svc);
           continue;
         }
@@ -1057,7 +1092,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       // for it, and on every instance this event's requests wait for: its free
       // slots go to the most urgent of the waiting requests and the new ones.
       if (npend | waiting) {
-        const int lpol = kGeneric ? W->lpol : HX_LOCAL_PQ;
+        const int lpol = kGeneric ? uniform(W->lpol) : HX_LOCAL_PQ;
         int m = cm;
         int4 pe = make_int4(0, 0, 0, -1);  // entry j on lane j
         unsigned left = 0, pm = 0;
@@ -1070,9 +1105,9 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         for (;;) {
           HX_BOUND(m >= 0 && m < N)
           const InstState I = inst[m];
-          uint32_t free = I.free;
+          uint32_t free = uniform(I.free);
           const uint32_t slot_base = first_slot(m, I);
-          const int hs = I.hsize;
+          const int hs = uniform(I.hsize);
           HeapEnt* h = queue_of(I.heap);
 #ifdef HX_CHECKED
           {
@@ -1106,7 +1141,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
               e.key = __shfl_sync(kFull, e.key, j);
               e.rid = __shfl_sync(kFull, e.rid, j);
               e.svc = __shfl_sync(kFull, e.svc, j);
-              fresh = ent_better(e, top);
+              fresh = __any_sync(kFull, ent_better(e, top));
             } else {
               e = ent_load(h + --n, true);
               if (lane + 1 >= n) kid.key = 0;  // the last entry is no child any more
