@@ -119,9 +119,10 @@ int ensure_dyn_smem(int kernel, int bytes) {
 
 // The family of the simulation kernel that serves a run: the lean one serves
 // grids that are all workload-balanced dispatch with the urgency queue, log
-// nothing, check nothing, count one tenant and have no fault windows.
+// nothing, check nothing, count one tenant and have no fault windows; the wide
+// one serves fault windows and traces with a call of kLongCall us or more.
 int sim_family(const hx_grid* grid, const hx::ClusterK& ck, bool record, bool force, bool checked) {
-  if (ck.n_faults > 0) return hx::kSimFaults;
+  if (ck.n_faults > 0) return hx::kSimWide;
   bool generic = force || checked || ck.n_tenants > 1;
   for (int p = 0; p < grid->n_points; ++p)
     generic |= grid->local_policy[p] != HX_LOCAL_PQ || grid->dispatch_policy[p] != HX_DISPATCH_WB;
@@ -189,10 +190,13 @@ struct hx_sim {
   int64_t* d_rec_start = nullptr;
   int64_t* d_rec_end = nullptr;
   std::vector<int32_t> record_sims;
-  // launch shape
-  int blocks = 0, resident_warps = 0, smem_per_block = 0;
-  int family = hx::kSimGeneric;
-  int kernel = 1;  // which instantiation of the simulation kernel runs (hx::kSimKernel)
+  // the simulation kernel's family and launch for the traces as they are: [0] with
+  // short calls only, [1] with one of kLongCall us or more
+  struct Launch {
+    int family = hx::kSimWide, kernel = 0, blocks = 0, smem_per_block = 0;
+  } launch[2];
+  bool long_calls = false;
+  const Launch& shape() const { return launch[long_calls ? 1 : 0]; }
   int64_t scratch_bytes = 0, device_bytes = 0;
   cudaStream_t last_stream = nullptr;
   bool ran = false;
@@ -293,7 +297,10 @@ int validate_grid(const hx_grid* g) {
   return HX_OK;
 }
 
-int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_prefill, int64_t max_decode) {
+// *long_call: whether a call may cost kLongCall us or more on some type.
+int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_prefill, int64_t max_decode,
+                   bool* long_call) {
+  bool is_long = false;
   const std::string where = "trace " + std::to_string(ti) + ": ";
   if (tr->n_queries < 0 || tr->n_calls < 0 || tr->n_calls >= (1 << 24))
     return fail(HX_ERR_INVALID, where + "n_queries/n_calls out of range");
@@ -347,10 +354,12 @@ int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_
       const int64_t dec = std::max(o, oe) * max_decode;
       if (dec >= kCostMax || p * 1000000 > (kCostMax - 1 - dec) * min_prefill)
         return fail(HX_ERR_INVALID, where + "a call's cost exceeds 2^28 us");
+      is_long |= dec >= hx::kLongCall || p * 1000000 > (hx::kLongCall - 1 - dec) * min_prefill;
       tok_sum += p;
       dec_sum += dec;
     }
   }
+  *long_call = is_long;
   // fault windows stretch attempts (slow-down or timeout) and delay the rest
   int64_t stretch = HX_SCALE, last = tr->n_queries > 0 ? tr->arrival_us[tr->n_queries - 1] : 0;
   for (int f = 0; f < c->n_faults; ++f) {
@@ -414,15 +423,19 @@ void for_each_trace(const hx_trace* traces, int32_t n_traces, F fn) {
 // validate_trace over every trace, in parallel; the lowest-numbered failing
 // trace's status and message are reported, as a loop in order would.
 int validate_traces(const hx_trace* traces, int32_t n_traces, const hx_cluster* c, int64_t min_prefill,
-                    int64_t max_decode) {
+                    int64_t max_decode, bool* long_calls) {
   std::vector<int> rc((size_t)n_traces, HX_OK);
+  std::atomic<bool> any_long{false};
   std::vector<std::string> msg((size_t)n_traces);
   for_each_trace(traces, n_traces, [&](int32_t t) {
-    rc[t] = validate_trace(&traces[t], t, c, min_prefill, max_decode);
+    bool is_long = false;
+    rc[t] = validate_trace(&traces[t], t, c, min_prefill, max_decode, &is_long);
+    if (is_long) any_long = true;
     if (rc[t] != HX_OK) msg[t] = g_err;  // this thread's message
   });
   for (int32_t t = 0; t < n_traces; ++t)
     if (rc[t] != HX_OK) return fail(rc[t], msg[t]);
+  *long_calls = any_long;
   return HX_OK;
 }
 
@@ -492,27 +505,36 @@ int upload_traces(hx_sim* h, const hx_trace* traces, cudaStream_t s) {
 }
 
 // WarpShared and the instance states and slot entries that follow it.
-int per_warp_smem(const hx::ClusterK& ck) {
-  const int64_t slot = ck.n_faults > 0 ? sizeof(hx::Slot64) : sizeof(hx::Slot32);
+int per_warp_smem(const hx::ClusterK& ck, int family) {
+  const int64_t slot = family == hx::kSimWide ? sizeof(hx::Slot64) : sizeof(hx::Slot32);
   return (int)align_up((int64_t)sizeof(hx::WarpShared) + (ck.n_inst <= 32 ? 32 : 64) * (int64_t)sizeof(hx::InstState) +
                        slot * ck.slot_entries, 16);
 }
 
-// The kernel for a cluster and up to *blocks blocks of it, and the blocks that
-// are resident at once.
-int launch_shape(int family, const hx::ClusterK& ck, const cudaDeviceProp& prop, int smem_per_block, int64_t* blocks,
-                 int* kernel) {
-  const int64_t want = std::max<int64_t>(*blocks, 1);
-  *kernel = sim_kernel_of(family, ck, few_warps(want * hx::kWarpsPerBlock, prop.multiProcessorCount));
-  if (int rc = ensure_dyn_smem(*kernel, smem_per_block)) return rc;
+// The launch of a kernel family for a cluster, of up to `want` blocks: the kernel
+// and the blocks that are resident at once.
+int launch_shape(int family, const hx::ClusterK& ck, const cudaDeviceProp& prop, int64_t want, hx_sim::Launch* out) {
+  want = std::max<int64_t>(want, 1);
+  out->family = family;
+  out->kernel = sim_kernel_of(family, ck, few_warps(want * hx::kWarpsPerBlock, prop.multiProcessorCount));
+  out->smem_per_block = hx::kWarpsPerBlock * per_warp_smem(ck, family);
+  if (int rc = ensure_dyn_smem(out->kernel, out->smem_per_block)) return rc;
   int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, (const void*)hx::kSimKernel[*kernel], hx::kWarpsPerBlock * 32,
-                                                    smem_per_block) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, (const void*)hx::kSimKernel[out->kernel],
+                                                    hx::kWarpsPerBlock * 32, out->smem_per_block) != cudaSuccess ||
       bps < 1) {
     cudaGetLastError();
     return fail(HX_ERR_CUDA, "simulation kernel does not fit on an SM");
   }
-  *blocks = std::min<int64_t>(want, (int64_t)bps * prop.multiProcessorCount);
+  out->blocks = (int)std::min<int64_t>(want, (int64_t)bps * prop.multiProcessorCount);
+  return HX_OK;
+}
+
+int launch_sim(const hx_sim::Launch& l, const hx::SimArgs& sa, hx::ClusterK ck, cudaStream_t s) {
+  ck.smem_per_warp = l.smem_per_block / hx::kWarpsPerBlock;
+  if (int rc = ensure_dyn_smem(l.kernel, l.smem_per_block)) return rc;
+  hx::kSimKernel[l.kernel]<<<(unsigned)l.blocks, hx::kWarpsPerBlock * 32, l.smem_per_block, s>>>(sa, ck);
+  HX_CUDA(cudaGetLastError());
   return HX_OK;
 }
 
@@ -563,7 +585,7 @@ void fill_cluster(const hx_cluster* cluster, hx::ClusterK& ck) {
     ck.faults[f].inst = F.inst;
     ck.faults[f].pad = 0;
   }
-  ck.smem_per_warp = per_warp_smem(ck);
+  ck.smem_per_warp = 0;  // by kernel family, at launch
 }
 
 // The simulations of opt->sim_subset, checked (in range, distinct) and sorted
@@ -648,7 +670,8 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   int rc;
   if ((rc = validate_cluster(cluster, &min_prefill, &max_decode))) return rc;
   if ((rc = validate_grid(grid))) return rc;
-  if ((rc = validate_traces(traces, n_traces, cluster, min_prefill, max_decode))) return rc;
+  bool long_calls = false;
+  if ((rc = validate_traces(traces, n_traces, cluster, min_prefill, max_decode, &long_calls))) return rc;
   if (opt && opt->n_record < 0) return fail(HX_ERR_INVALID, "n_record < 0");
   if (opt && opt->n_record > 0) {
     if (!opt->record_sims) return fail(HX_ERR_INVALID, "record_sims is NULL");
@@ -726,18 +749,19 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
       (rc = upload(h->d_dp, grid->dispatch_policy, h->n_points, s0)))
     return bail(rc);
 
-  h->family = sim_family(grid, ck, opt && opt->n_record > 0, opt && opt->force_generic, h->checked);
-  // launch shape of the simulation kernel and its per-warp scratch
-  h->smem_per_block = hx::kWarpsPerBlock * ck.smem_per_warp;
+  // launch shapes of the simulation kernel; later uploads may bring longer calls
   int64_t blocks = (h->n_sims + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock;
   if (opt && opt->max_resident_warps > 0)
     blocks = std::min<int64_t>(blocks, std::max<int64_t>(1, opt->max_resident_warps / hx::kWarpsPerBlock));
-  if ((rc = launch_shape(h->family, ck, prop, h->smem_per_block, &blocks, &h->kernel))) return bail(rc);
-  h->blocks = (int)blocks;
-  h->resident_warps = h->blocks * hx::kWarpsPerBlock;
+  const int family = sim_family(grid, ck, opt && opt->n_record > 0, opt && opt->force_generic, h->checked);
+  if ((rc = launch_shape(family, ck, prop, blocks, &h->launch[0])) ||
+      (rc = launch_shape(hx::kSimWide, ck, prop, blocks, &h->launch[1])))
+    return bail(rc);
+  h->long_calls = long_calls;
+  const int64_t resident_warps = hx::kWarpsPerBlock * (int64_t)h->shape().blocks;
   // the simulations' order: the caller's subset, else possibly the costliest first
   h->work_order = subset.empty()
-                      ? costliest_first(grid, n_traces, h->n_c, (int64_t)prop.l2CacheSize, h->resident_warps, &subset)
+                      ? costliest_first(grid, n_traces, h->n_c, (int64_t)prop.l2CacheSize, resident_warps, &subset)
                       : 1;
   if (!subset.empty() && ((rc = h->alloc(&h->d_subset, (int64_t)subset.size())) ||
                           (rc = upload(h->d_subset, subset.data(), (int64_t)subset.size(), s0))))
@@ -759,11 +783,11 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
     if ((rc = upload(h->d_tenant_kcap, kcap.data(), (int64_t)kcap.size(), s0))) return bail(rc);
     if (cudaStreamSynchronize(s0) != cudaSuccess) return bail(fail(HX_ERR_CUDA, "tenant upload failed"));
   }
-  const int64_t w = h->resident_warps;
+  const int64_t w = hx::kWarpsPerBlock * (int64_t)std::max(h->launch[0].blocks, h->launch[1].blocks);
   if ((rc = h->alloc(&h->d_arena, w * h->arena_per_warp)) || (rc = h->alloc(&h->d_chains, w * h->chains_per_warp)) ||
       (rc = h->alloc(&h->d_topk, w * h->topk_per_warp)))
     return bail(rc);
-  if (h->family >= hx::kSimGeneric && (rc = h->alloc(&h->d_extras, h->n_sims))) return bail(rc);
+  if (family >= hx::kSimGeneric && (rc = h->alloc(&h->d_extras, h->n_sims))) return bail(rc);
   h->scratch_bytes = w * (h->arena_per_warp * (int64_t)sizeof(hx::HeapEnt) + h->chains_per_warp +
                           h->topk_per_warp * (int64_t)sizeof(int64_t));
 
@@ -818,9 +842,15 @@ static int hx_sim_upload_impl(hx_sim* h, const hx_trace* traces, int32_t n_trace
   c.timeout_mult_fp = h->ck.timeout_mult_fp;
   c.n_faults = (int32_t)h->faults.size();
   c.faults = h->faults.data();
-  int rc = validate_traces(traces, n_traces, &c, min_prefill, max_decode);
+  bool long_calls = false;
+  int rc = validate_traces(traces, n_traces, &c, min_prefill, max_decode, &long_calls);
   if (rc) return rc;
-  return upload_traces(h, traces, static_cast<cudaStream_t>(stream));
+  // set first: a copy that fails half-way may leave long calls behind
+  const bool had_long = h->long_calls;
+  h->long_calls = had_long || long_calls;
+  if ((rc = upload_traces(h, traces, static_cast<cudaStream_t>(stream)))) return rc;
+  h->long_calls = long_calls;
+  return HX_OK;
 }
 
 static int hx_sim_run_impl(hx_sim* h, void* stream) {
@@ -894,14 +924,12 @@ static int hx_sim_run_impl(hx_sim* h, void* stream) {
   ba.point_sums = h->d_point_sums;
 
   const int prep_blocks = (int)std::max<int64_t>(1, (h->n_q + 255) / 256);
-  if (int rc = ensure_dyn_smem(h->kernel, h->smem_per_block)) return rc;
   cudaEvent_t* ev = h->timing ? h->run_ev(h->runs) : nullptr;
   if (ev) HX_CUDA(cudaEventRecord(ev[0], s));
   hx::hx_prep_kernel<<<prep_blocks, 256, 0, s>>>(pa, h->ck);
   HX_CUDA(cudaGetLastError());
   if (ev) HX_CUDA(cudaEventRecord(ev[1], s));
-  hx::kSimKernel[h->kernel]<<<h->blocks, hx::kWarpsPerBlock * 32, h->smem_per_block, s>>>(sa, h->ck);
-  HX_CUDA(cudaGetLastError());
+  if (int rc = launch_sim(h->shape(), sa, h->ck, s)) return rc;
   if (h->n_record > 0) {
     hx::LogArgs la;
     la.rec = h->d_rec;
@@ -1142,11 +1170,11 @@ int hx_sim_info(hx_sim* h, hx_info* out) {
   out->n_queries_total = h->n_q;
   out->scratch_bytes = h->scratch_bytes;
   out->device_bytes = h->device_bytes;
-  out->resident_warps = h->resident_warps;
+  out->resident_warps = hx::kWarpsPerBlock * h->shape().blocks;
   out->warps_per_block = hx::kWarpsPerBlock;
-  out->blocks = h->blocks;
-  out->smem_per_block = h->smem_per_block;
-  out->generic_kernel = h->family != hx::kSimLean ? 1 : 0;
+  out->blocks = h->shape().blocks;
+  out->smem_per_block = h->shape().smem_per_block;
+  out->generic_kernel = h->shape().family != hx::kSimLean ? 1 : 0;
   out->work_order = h->work_order;
   return HX_OK;
 }
@@ -1231,7 +1259,8 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
   int rc;
   if ((rc = validate_cluster(cluster, &min_prefill, &max_decode))) return rc;
   if ((rc = validate_grid(grid))) return rc;
-  if ((rc = validate_trace(trace, 0, cluster, min_prefill, max_decode))) return rc;
+  bool long_calls = false;
+  if ((rc = validate_trace(trace, 0, cluster, min_prefill, max_decode, &long_calls))) return rc;
   const int64_t nq = trace->n_queries, nc = trace->n_calls, P = grid->n_points;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
 
@@ -1268,11 +1297,11 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
   cudaDeviceProp prop;
   HX_CUDA(cudaGetDevice(&dev));
   HX_CUDA(cudaGetDeviceProperties(&prop, dev));
-  const int smem_per_block = hx::kWarpsPerBlock * ck.smem_per_warp;
-  const int family = sim_family(grid, ck, false, false, false);
-  int64_t blocks = std::min<int64_t>(fit_warps / hx::kWarpsPerBlock, (P + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock);
-  int kernel = 0;
-  if ((rc = launch_shape(family, ck, prop, smem_per_block, &blocks, &kernel))) return rc;
+  const int family = long_calls ? hx::kSimWide : sim_family(grid, ck, false, false, false);
+  hx_sim::Launch launch;
+  if ((rc = launch_shape(family, ck, prop, std::min<int64_t>(fit_warps / hx::kWarpsPerBlock, (P + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock), &launch)))
+    return rc;
+  const int64_t blocks = launch.blocks;
   const int64_t warps = blocks * hx::kWarpsPerBlock;
   const int64_t o_arena = fixed;
   const int64_t o_chains = o_arena + warps * align_up(arena_per_warp * (int64_t)sizeof(hx::HeapEnt), 256);
@@ -1371,8 +1400,7 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
 
   hx::hx_prep_kernel<<<(unsigned)std::max<int64_t>(1, (nq + 255) / 256), 256, 0, s>>>(pa, ck);
   HX_CUDA(cudaGetLastError());
-  hx::kSimKernel[kernel]<<<(unsigned)blocks, hx::kWarpsPerBlock * 32, smem_per_block, s>>>(sa, ck);
-  HX_CUDA(cudaGetLastError());
+  if ((rc = launch_sim(launch, sa, ck, s))) return rc;
   hx::hx_best_kernel<<<2, 256, 0, s>>>(ba);
   HX_CUDA(cudaGetLastError());
   HX_CUDA(cudaMemcpyAsync(results, at(o_res), (size_t)P * sizeof(hx_result), cudaMemcpyDeviceToHost, s));

@@ -21,6 +21,7 @@ namespace hx {
 constexpr int64_t kScale = 1000000;       // fixed point of alpha, gamma, slo_mult
 constexpr int64_t kUsPerS = 1000000;      // prefill throughput is per second
 constexpr int64_t kRewardCap = (int64_t(1) << 43) - 1;
+constexpr int64_t kLongCall = int64_t(1) << 25;  // us; from here on event times are 64-bit
 constexpr int kWarpsPerBlock = 4;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kFRows = 18;                // S, G/C with 0..15 corrections done, E
@@ -70,7 +71,7 @@ struct ClusterK {
   uint8_t inst_type[HX_MAX_INST];
   uint8_t inst_slots[HX_MAX_INST];
   uint16_t slot_base[HX_MAX_INST];
-  // tenants and faults (only hx_sim_kernel_faults handles faults)
+  // tenants and faults (only hx_sim_kernel_wide handles faults)
   int32_t n_tenants, n_faults;
   int64_t tenant_mult[HX_MAX_TENANTS];
   int64_t timeout_mult_fp;
@@ -227,11 +228,11 @@ __global__ void hx_prep_kernel(PrepArgs a, ClusterK c);
 // The instantiations of the simulation kernel.  hx_sim_kernel_lean: every point
 // workload-balanced with the urgency queue, nothing logged; hx_sim_kernel_log:
 // with per-call logs; hx_sim_kernel: those and any mix of dispatch and
-// local-queue policies, tenants and event checks; hx_sim_kernel_faults: all of
-// it with fault windows.  Each for clusters of up to 64 instances, two a lane,
+// local-queue policies, tenants and event checks; hx_sim_kernel_wide: all of
+// it with fault windows or calls of kLongCall us and more (64-bit times).  Each for clusters of up to 64 instances, two a lane,
 // and of up to 32, one a lane, and both for a full GPU and for a run of few
 // warps: kernel 4 * family + 2 * few + (one a lane).
-enum { kSimLean = 0, kSimLog = 1, kSimGeneric = 2, kSimFaults = 3 };
+enum { kSimLean = 0, kSimLog = 1, kSimGeneric = 2, kSimWide = 3 };
 using SimKernel = void (*)(SimArgs, ClusterK);
 constexpr int kSimKernels = 16;
 extern const SimKernel kSimKernel[kSimKernels];

@@ -270,10 +270,15 @@ __global__ void __launch_bounds__(256) hx_prep_kernel(PrepArgs a, ClusterK c) {
 // -------------------------------------------------------- simulation kernel
 namespace {
 
-// Event times of one simulation.  Without fault windows an attempt runs less
-// than 2^28 us, so 32 bits relative to a base (moved up every 2^31 us) order
-// the running calls and one 32-bit warp minimum finds the next completion;
-// with fault windows an attempt can outlast that and times are 64-bit, base 0.
+// Event times of one simulation are relative to a base.  While every call costs
+// less than 2^25 us on every type and there are no fault windows, they are
+// 32-bit, the base moves up every 2^25 us, and an instance's next completion is
+// time << 6 | instance: one 32-bit warp minimum gives the next event's time and
+// instance (a dispatch's least cost << 6 | instance likewise), without the ballot
+// and the bit search that lengthened the event's chain (8 x 2000 queries x 64
+// points 6.80 -> 6.29 ms, 8 x 20000 x 1024 on 64 instances 431 -> 399 ms).
+// Longer calls and fault windows, whose attempts can outlast that,
+// have 64-bit times, base 0.
 template <bool kWide>
 struct Times {
   using T = uint32_t;
@@ -284,6 +289,8 @@ struct Times<true> {
   using T = uint64_t;
   using Slot = Slot64;
 };
+constexpr int kInstBits = 6;                          // of a key: HX_MAX_INST instances
+constexpr uint64_t kInstMask = (1 << kInstBits) - 1;
 
 // Running calls complete by (end, request id); a tag is request id << 8 | slot.
 __device__ __forceinline__ bool before(uint32_t e0, uint32_t tag0, uint32_t e1, uint32_t tag1) {
@@ -631,11 +638,12 @@ __device__ __noinline__ unsigned lowest_id(uint32_t tag) {
 
 template <int J, int kFamily, bool kFew>
 __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
-  constexpr bool kLog = kFamily >= kSimLog, kGeneric = kFamily >= kSimGeneric, kFaults = kFamily == kSimFaults;
-  using T = typename Times<kFaults>::T;
-  using Slot = typename Times<kFaults>::Slot;
-  constexpr T kIdle = ~T(0);                      // no running call; no arrival in range
-  constexpr T kFar = kFaults ? kIdle : T(1) << 31;  // an event this far moves the base up first
+  constexpr bool kLog = kFamily >= kSimLog, kGeneric = kFamily >= kSimGeneric, kWide = kFamily == kSimWide;
+  using T = typename Times<kWide>::T;
+  using Slot = typename Times<kWide>::Slot;
+  constexpr T kIdle = ~T(0);                        // no time
+  constexpr T kNone = kIdle & ~T(kInstMask);        // keys from here on: no running call, no arrival in range
+  constexpr T kFar = kWide ? kNone : T(1) << 31;  // an event with such a key moves the base up first
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = uniform((int)(threadIdx.x >> 5));
   // volatile: read once and kept, not read again wherever it is used
@@ -740,19 +748,19 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     }
     __syncwarp();
 
-    // What this lane keeps of its instances, in registers: t_queue, the end of
-    // the next completion (kIdle: nothing runs) and its tag (request id << 8 |
+    // What this lane keeps of its instances, in registers: t_queue, the next
+    // completion's key (kNone up: nothing runs) and its tag (request id << 8 |
     // slot).  An instance past N has t_queue INT64_MAX and cost weight -inf in the
     // score filter, and never wins.
     int64_t q[J];
-    T next_end[J];
+    T next_key[J];
     uint32_t next_tag[J];
     float neg_a[J];
 #pragma unroll
     for (int j = 0; j < J; ++j) {
       const bool on = lane + 32 * j < N;
       q[j] = on ? 0 : INT64_MAX;
-      next_end[j] = kIdle;
+      next_key[j] = kIdle;
       next_tag[j] = 0;
       neg_a[j] = on ? -(float)W->A : -INFINITY;
     }
@@ -774,21 +782,22 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     const longlong2 tie0 = W->tie;
     const float4 fscore0 = W->fscore;
 
-    // times are relative to base; an arrival 2^32 us or more past it reads as kIdle
+    // the key of an arrival, after every completion at its time; kNone up: 2^26 us
+    // or more past the base
     W->base = 0;
-    auto rel = [&](int64_t t_abs) -> T {
-      if (kFaults) return (T)t_abs;
+    auto arrival_key = [&](int64_t t_abs) -> T {
+      if (kWide) return (T)t_abs << kInstBits | kInstMask;
       const uint64_t d = (uint64_t)(t_abs - W->base);
-      return (d >> 32) ? kIdle : (T)d;
+      return (d >> (32 - kInstBits)) ? kIdle : (T)d << kInstBits | kInstMask;
     };
-    auto absolute = [&](T t) -> int64_t { return kFaults ? (int64_t)t : W->base + (int64_t)t; };
+    auto absolute = [&](T t) -> int64_t { return kWide ? (int64_t)t : W->base + (int64_t)t; };
     W->arrivals = 0;
     W->next_arrival = nq > 0 ? a.arrival[qb] : 0;
-    T arr = nq > 0 ? uniform(rel(a.arrival[qb])) : kIdle;
+    T arr = nq > 0 ? uniform(arrival_key(a.arrival[qb])) : kIdle;
     T now = 0;
     int32_t status = HX_OK, npend = 0;
     // event bound; re-issued attempts add events while fault windows last
-    int32_t steps_left = nc + nq + 8 + (kFaults ? 16 * nc + 4096 : 0);
+    int32_t steps_left = nc + nq + 8 + (kWide ? 16 * nc + 4096 : 0);
 #ifdef HX_CHECKED
     // the warp's scratch slices must hold this trace's chain counters and top-K
     if (!(nq <= a.chains_per_warp && W->kcap <= a.topk_per_warp && (a.tenant_kcap == nullptr ||
@@ -811,7 +820,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     auto start_call = [&](int m, uint32_t free, uint32_t slot_base, int rid, int svc) -> uint32_t {
       T run = (T)svc;
       bool fail = false;
-      if (kFaults) {
+      if (kWide) {
         // the first fault window of m that covers now, and the timeout (Sec. 3.3)
         int64_t r64 = svc;
         bool in_window = false, down = false;
@@ -835,12 +844,12 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       }
       const int s = 31 - __clz(free);
       const uint32_t tag = (uint32_t)rid << 8 | (uint32_t)s;
-      const T end = now + run;
+      const T end = now + run, key = end << kInstBits | (T)m;
       if (lane == (m & 31)) {
         Slot e;
         e.end = end;
         e.tag = tag;
-        if constexpr (kFaults) e.fail = fail ? 1u : 0u;
+        if constexpr (kWide) e.fail = fail ? 1u : 0u;
         slots[slot_base + s] = e;
         if (kLog && recj >= 0) {
           a.rec_start[(int64_t)recj * a.rec_stride + rid] = absolute(now);
@@ -850,43 +859,43 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
 #pragma unroll
       for (int j = 0; j < J; ++j) {
         // the lowest request id completes first among equal ends
-        const bool first = (lane + 32 * j == m) & before(end, tag, next_end[j], next_tag[j]);
-        next_end[j] = first ? end : next_end[j];
+        const bool first = (lane + 32 * j == m) & before(key, tag, next_key[j], next_tag[j]);
+        next_key[j] = first ? key : next_key[j];
         next_tag[j] = first ? tag : next_tag[j];
       }
       free ^= 1u << s;
       inst[m].free = free;  // every lane stores the same mask
-      digest_push<kFaults>(W, dn, now, call_tag(rid, m), lane);
+      digest_push<kWide>(W, dn, now, call_tag(rid, m), lane);
       return free;
     };
 
     for (;;) {
       HX_STOP_IF_FAILED()
       __syncwarp();
-      const T mn = warp_min(J == 2 && next_end[J - 1] < next_end[0] ? next_end[J - 1] : next_end[0]);
+      const T mn = warp_min(J == 2 && next_key[J - 1] < next_key[0] ? next_key[J - 1] : next_key[0]);
       if (((mn < arr ? mn : arr) >= kFar) | (steps_left == 0)) {
-        // the end, too many events, or nothing within 2^31 us of the base, which
+        // the end, too many events, or nothing within 2^25 us of the base, which
         // then moves to the next event
         const bool more = uniform(W->arrivals) < nq;
-        if (mn == kIdle && !more) break;
+        if (mn >= kNone && !more) break;
         if (steps_left-- == 0) {
           status = HX_ERR_STEP_LIMIT;
           break;
         }
         ++steps_left;
-        if (!kFaults) {
-          digest_flush<kFaults>(W, dn, lane);
+        if (!kWide) {
+          digest_flush<kWide>(W, dn, lane);
           dn = 0;
           const int64_t base = W->base, at = W->next_arrival;
-          int64_t nb = mn == kIdle ? at : base + (int64_t)mn;
+          int64_t nb = mn >= kNone ? at : base + (int64_t)(mn >> kInstBits);
           if (more && at < nb) nb = at;
           const T shift = (T)(nb - base);
 #pragma unroll
-          for (int j = 0; j < J; ++j) next_end[j] = next_end[j] == kIdle ? kIdle : next_end[j] - shift;
+          for (int j = 0; j < J; ++j) next_key[j] = next_key[j] >= kNone ? kIdle : next_key[j] - (shift << kInstBits);
           for (int j = lane; j < c.slot_entries; j += 32) slots[j].end -= shift;
           __syncwarp();
           W->base = nb;  // every lane writes the same value
-          arr = more ? uniform(rel(at)) : kIdle;
+          arr = more ? uniform(arrival_key(at)) : kIdle;
           continue;
         }
       }
@@ -897,13 +906,11 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       int32_t rel_first = 0, rel_count = 0;
       if (mn <= arr) {
         // completion on the lowest instance that has one at mn
-        now = mn;
-        const unsigned b0 = __ballot_sync(kFull, next_end[0] == mn);
-        const unsigned b1 = J == 2 ? __ballot_sync(kFull, next_end[J - 1] == mn) : 0u;
-        const bool low = J == 1 || b0 != 0;
-        const int ml = __ffs(low ? b0 : b1) - 1, m = low ? ml : ml + 32;
-        HX_BOUND(ml >= 0 && m < N)
-        const uint32_t tag = __shfl_sync(kFull, low ? next_tag[0] : next_tag[J - 1], ml);
+        now = mn >> kInstBits;
+        const int m = (int)(mn & kInstMask);
+        const bool low = J == 1 || m < 32;
+        HX_BOUND(m < N)
+        const uint32_t tag = __shfl_sync(kFull, low ? next_tag[0] : next_tag[J - 1], m & 31);
         const int32_t rid = (int32_t)(tag >> 8);
         const int hole = (int)(tag & 0xffu);
         HX_BOUND(rid < nc)
@@ -926,7 +933,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         if (kFew) load_costs(tail.y);
         // the slot is free; the next completion is the earliest of those still running
         const uint32_t free = I.free | 1u << hole;
-        const bool failed = kFaults && __any_sync(kFull, reinterpret_cast<const Slot64*>(slots)[slot_base + hole].fail != 0);
+        const bool failed = kWide && __any_sync(kFull, reinterpret_cast<const Slot64*>(slots)[slot_base + hole].fail != 0);
         const Slot e = slots[slot_base + l16];
         const bool runs = (I.cfg & ~free & 0xffffu & lbit) != 0;
         const T nmin = warp_min(runs ? e.end : kIdle);
@@ -939,7 +946,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
 #pragma unroll
         for (int j = 0; j < J; ++j) {
           const bool own = lane + 32 * j == m;
-          next_end[j] = own ? nmin : next_end[j];
+          next_key[j] = own ? nmin << kInstBits | (T)m : next_key[j];
           next_tag[j] = own ? ntag : next_tag[j];
           q[j] -= own ? est : 0;
         }
@@ -953,7 +960,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         rel_first = tail.y;
         rel_count = chain ? flags & 1u : tw & 0xff;
         if (chain) *chains = (uint8_t)ended;  // every lane writes the same byte
-        if (kFaults && failed) {
+        if (kWide && failed) {
           // the attempt timed out: the request goes out again, avoiding m
           const int32_t n = W->reissued + 1;
           __syncwarp();
@@ -981,12 +988,12 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
                 topk_insert_warp(W->topk + a.tenant_topk_off[ten], &W->ttk[ten], kc, &W->ttkmin[ten], v, lane);
             }
           }
-          digest_push<kFaults>(W, dn, now, query_tag(qid), lane);
+          digest_push<kWide>(W, dn, now, query_tag(qid), lane);
           finish_query(W, t_abs, at, dl, lane);
         }
         HX_BOUND(rel_first >= 0 && rel_count <= HX_MAX_K && rel_first + rel_count <= nc)
       } else {
-        now = arr;
+        now = arr >> kInstBits;
         const int64_t qbase = W->qb;
         const int32_t qa = uniform(W->arrivals);
         HX_BOUND(qa < nq)
@@ -1006,7 +1013,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         W->arrivals = qa + 1;  // every lane writes the same values
         const int64_t at = qa + 1 < nq ? a.arrival[qbase + qa + 1] : 0;
         W->next_arrival = at;
-        arr = qa + 1 < nq ? uniform(rel(at)) : kIdle;
+        arr = qa + 1 < nq ? uniform(arrival_key(at)) : kIdle;
       }
 
       // Sec. 4.1 for each released request, in request-id order: score every
@@ -1021,7 +1028,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         if (kFew && rel_count > 1) load_costs(rid + 1);
         int m;
         // a re-issued request avoids the instance it timed out on
-        const int excl = kFaults ? uniform(W->excl) : -1;
+        const int excl = kWide ? uniform(W->excl) : -1;
         if (kGeneric && round_robin) {
           m = uniform(W->rr);
           if (m == excl) m = (m + 1 == N) ? 0 : m + 1;
@@ -1031,23 +1038,21 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
           // instances that tie in their reward and beat all others: the least cost wins
           // (the lowest instance at alpha = 0, where costs have no weight)
           const longlong2 tie = kFew ? tie0 : W->tie;
-          uint32_t cost[J];
+          T cost[J];  // << 6 | instance
 #pragma unroll
-          for (int j = 0; j < J; ++j) cost[j] = q[j] <= tie.x ? (uint32_t)ev[j].x & (uint32_t)tie.y : 0xffffffffu;
-          const uint32_t least = __reduce_min_sync(kFull, J == 2 && cost[J - 1] < cost[0] ? cost[J - 1] : cost[0]);
-          unsigned b0, b1 = 0;
-          if ((least != 0xffffffffu) & (excl < 0)) {
-            b0 = __ballot_sync(kFull, cost[0] == least);
-            if (J == 2) b1 = __ballot_sync(kFull, cost[J - 1] == least);
-            m = J == 1 || b0 ? __ffs(b0) - 1 : __ffs(b1) + 31;
+          for (int j = 0; j < J; ++j)
+            cost[j] = q[j] <= tie.x ? (T)((uint32_t)ev[j].x & (uint32_t)tie.y) << kInstBits | (T)(lane + 32 * j) : kIdle;
+          const T least = warp_min(J == 2 && cost[J - 1] < cost[0] ? cost[J - 1] : cost[0]);
+          if ((least != kIdle) & (excl < 0)) {
+            m = (int)(least & kInstMask);
           } else {
             const float4 f = kFew ? fscore0 : W->fscore;
             ScoreRange s[J];
 #pragma unroll
             for (int j = 0; j < J; ++j) s[j] = score_range(q[j], ev[j].x, f, neg_a[j]);
             const float lo = warp_max_f32(J == 2 ? fmaxf(s[0].lo, s[J - 1].lo) : s[0].lo);
-            b0 = __ballot_sync(kFull, s[0].hi >= lo);
-            if (J == 2) b1 = __ballot_sync(kFull, s[J - 1].hi >= lo);
+            const unsigned b0 = __ballot_sync(kFull, s[0].hi >= lo);
+            const unsigned b1 = J == 2 ? __ballot_sync(kFull, s[J - 1].hi >= lo) : 0u;
             // one instance's score can reach the best lower bound: it wins
             if ((((b0 & (b0 - 1)) | (b1 & (b1 - 1))) == 0) & ((b0 == 0) != (b1 == 0)) & (excl < 0)) {
               m = J == 1 || b0 ? __ffs(b0) - 1 : __ffs(b1) + 31;
@@ -1057,7 +1062,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
             }
           }
         }
-        if (kFaults) W->excl = -1;
+        if (kWide) W->excl = -1;
         HX_BOUND(m >= 0 && m < N)
         const bool low = J == 1 || m < 32;
         // the winner's costs, on its lane
@@ -1206,7 +1211,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       }
     }
 
-    digest_flush<kFaults>(W, dn, lane);
+    digest_flush<kWide>(W, dn, lane);
     // conservation at the end: every dispatched request finished (t_queue back
     // to zero, no running call, no waiting request)
     bool left = false;
@@ -1219,8 +1224,8 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     if (lane == 0) {
       int st = status;
       const int32_t n_done = W->n_done;
-      const int32_t steps0 = W->nc + nq + 8 + (kFaults ? 16 * W->nc + 4096 : 0);
-      const int64_t events = (steps0 - steps_left) - W->arrivals - (kFaults ? W->reissued : 0);
+      const int32_t steps0 = W->nc + nq + 8 + (kWide ? 16 * W->nc + 4096 : 0);
+      const int64_t events = (steps0 - steps_left) - W->arrivals - (kWide ? W->reissued : 0);
       // every query and every call completed exactly once
       if (st == HX_OK && (leftover || n_done != nq || events != W->nc)) st = HX_ERR_INVARIANT;
       hx_result res;
@@ -1261,12 +1266,12 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
 HX_SIM_KERNEL(hx_sim_kernel_lean, kSimLean)
 HX_SIM_KERNEL(hx_sim_kernel_log, kSimLog)
 HX_SIM_KERNEL(hx_sim_kernel, kSimGeneric)
-HX_SIM_KERNEL(hx_sim_kernel_faults, kSimFaults)
+HX_SIM_KERNEL(hx_sim_kernel_wide, kSimWide)
 #undef HX_SIM_KERNEL
 
 #define HX_FORMS(name) name<2, false>, name<1, false>, name<2, true>, name<1, true>
 const SimKernel kSimKernel[kSimKernels] = {HX_FORMS(hx_sim_kernel_lean), HX_FORMS(hx_sim_kernel_log),
-                                           HX_FORMS(hx_sim_kernel), HX_FORMS(hx_sim_kernel_faults)};
+                                           HX_FORMS(hx_sim_kernel), HX_FORMS(hx_sim_kernel_wide)};
 #undef HX_FORMS
 
 // ----------------------------------------------------------- log kernel

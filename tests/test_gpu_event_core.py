@@ -1,7 +1,8 @@
 """The simulation kernel's event loop at the edges of its representation, against
-the oracle: times around and past 2^31 and 2^32 us (event times are 32-bit,
-relative to a base that moves), calls that end at the same time in one and in
-many slots, queries of more call records than one sweep of the warp fetches."""
+the oracle: times past 2^25, 2^31 and 2^32 us (with short calls event times are
+32-bit, relative to a base that moves every 2^25 us), calls next to 2^25 us, calls
+that end at the same time in one and in many slots, queries of more call records
+than one sweep of the warp fetches."""
 import numpy as np
 import pytest
 
@@ -14,7 +15,7 @@ FIELDS = ["p95_us", "makespan_us", "events", "digest", "slo_met", "n_done", "sta
 INST = [1, 16, 32, 33, 64]
 
 
-def _check(tr, cl, generic):
+def _workload(tr, cl, generic):
     B.build()
     n = 6
     lpol = (np.arange(n) % 3).astype(np.uint8) if generic else np.zeros(n, np.uint8)
@@ -22,14 +23,22 @@ def _check(tr, cl, generic):
                   np.array([W.SCALE, 0, 2 * W.SCALE, W.SCALE, W.SCALE // 4, 4 * W.SCALE], np.int64),
                   np.array([0, 1, 2, 3, 15, 0], np.int32), np.full(n, 300_000 ** 2, np.int64), lpol,
                   np.zeros(n, np.uint8))
-    wl = W.Workload("core", [tr], cl, grid, W.OBJ_P95)
-    sim = H.Sim(wl.traces, wl.cluster, wl.grid)
-    assert sim.info()["generic_kernel"] == int(generic or cl.faults is not None)
+    return W.Workload("core", [tr], cl, grid, W.OBJ_P95)
+
+
+def _same(sim, wl, family):
+    assert sim.info()["generic_kernel"] == int(family)
     sim.run()
     got, want = sim.results(), oracle.run(wl)
-    sim.close()
     for f in FIELDS:
         assert np.array_equal(got[f], want[f]), f
+
+
+def _check(tr, cl, generic, family=None):
+    wl = _workload(tr, cl, generic)
+    sim = H.Sim(wl.traces, wl.cluster, wl.grid)
+    _same(sim, wl, generic or cl.faults is not None if family is None else family)
+    sim.close()
 
 
 def _cluster(n_inst, slots=(1, 3, 16), rmax=2):
@@ -41,23 +50,55 @@ def _cluster(n_inst, slots=(1, 3, 16), rmax=2):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("long_calls", [False, True])
 @pytest.mark.parametrize("kind", ["lean", "generic", "faults"])
 @pytest.mark.parametrize("n_inst", INST)
-def test_times_past_32_bits(n_inst, kind):
+def test_times_past_32_bits(n_inst, kind, long_calls):
     tr = W.make_trace(W.RECIPES[1], 1, 40 + n_inst, n_queries=160)
-    # bursts at the edges of 31 and 32 bits and gaps of more than 2^32 us between them,
-    # with calls of up to 100 s running across
-    at = np.array([0, 2 ** 31 - 10_000_000, 2 ** 31 - 1, 2 ** 31, 2 ** 32 - 3, 2 ** 32 + 2 ** 31 - 1,
+    # bursts at the edges of 25, 26, 31 and 32 bits and gaps of more than 2^32 us between
+    # them, with calls of up to 20 s or 100 s running across
+    at = np.array([0, 2 ** 25 - 1, 2 ** 25, 2 ** 26 - 1, 2 ** 26, 2 ** 31 - 10_000_000, 2 ** 31 - 1, 2 ** 31, 2 ** 32 - 3, 2 ** 32 + 2 ** 31 - 1,
                    3 * 2 ** 32 + 5, 9 * 2 ** 32 - 1], np.int64)
-    tr.arrival_us = np.sort(np.concatenate([at + (i * 997) * (i % 5) for i in range(20)]))
-    tr.prompt[::17] = 1_000_000
+    tr.arrival_us = np.sort(np.concatenate([at + (i * 997) * (i % 5) for i in range(20)]))[:160]
+    tr.prompt[::17] = 1_000_000 if long_calls else 100_000
     cl = _cluster(n_inst)
     if kind == "faults":
         cl.timeout_mult_fp = 2 * W.SCALE
         cl.faults = np.zeros(2, W.FAULT_DTYPE)
         cl.faults[0] = (0, 0, 2 ** 31 - 20_000_000, 2 ** 31 + 20_000_000, 0)
         cl.faults[1] = (n_inst - 1, 0, 2 ** 32 - 5, 2 ** 32 + 60_000_000, 4 * W.SCALE)
-    _check(tr, cl, kind == "generic")
+    _check(tr, cl, kind == "generic", long_calls or kind != "lean")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_inst", [32, 33])
+def test_calls_next_to_the_short_limit(n_inst):
+    """Calls of 2^25 - 1 us keep 32-bit times, 2^25 us take 64-bit ones; a handle
+    follows the traces it is given, in either direction."""
+    cl = _cluster(n_inst)
+    cl.prefill_tok_s[:] = 1_000_000
+    cl.decode_us_tok[:] = 32
+    short = W.make_trace(W.RECIPES[1], 1, 9, n_queries=100)
+    short.prompt[:] = 1 + short.prompt % 900_000
+    short.prompt[::3], short.out[::3], short.out_est[::3] = 31, (2 ** 20 - 1), (2 ** 20 - 1)
+    assert int((short.prompt.astype(np.int64) + 32 * np.maximum(short.out, short.out_est)).max()) == 2 ** 25 - 1
+    longer = W.Trace(short.arrival_us, short.k, short.call_base, short.prompt.copy(), short.out, short.out_est,
+                     short.stage, short.cand, short.retry)
+    longer.prompt[::3] = 32
+    a, b = _workload(short, cl, False), _workload(longer, cl, False)
+    sim = H.Sim(a.traces, cl, a.grid)
+    _same(sim, a, 0)
+    sim.upload(b.traces)
+    _same(sim, b, 1)
+    sim.upload(a.traces)
+    _same(sim, a, 0)
+    sim.close()
+    sim = H.Sim(b.traces, cl, b.grid)
+    _same(sim, b, 1)
+    sim.close()
+    for wl in (a, b):
+        got, _ = H.run_static(wl.traces[0], cl, wl.grid)
+        assert np.array_equal(got["digest"], oracle.run(wl)["digest"])
 
 
 @pytest.mark.gpu
