@@ -139,6 +139,7 @@ struct hx_sim {
   int32_t n_tenants = 0;          // as given in hx_cluster (validation of later uploads)
   std::vector<hx_fault> faults;
   std::vector<int32_t> h_nq, h_nc;
+  std::vector<int64_t> q_off, c_off;  // [n_traces + 1]
   // device: inputs
   int64_t* d_arrival = nullptr;
   int64_t* d_qcall = nullptr;
@@ -176,7 +177,8 @@ struct hx_sim {
   int64_t arena_per_warp = 0, chains_per_warp = 0, topk_per_warp = 0;
   // device: records
   int32_t n_record = 0;
-  int64_t rec_stride = 0;
+  int64_t rec_calls = 0, rec_stride = 0;  // calls and int64 units per logged simulation
+  int64_t* d_rec_log = nullptr;
   int32_t* d_rec_map = nullptr;
   int32_t* d_rec_sims = nullptr;
   // run only these simulations, in work order (NULL: all of them)
@@ -184,11 +186,6 @@ struct hx_sim {
   int64_t n_work = 0;
   int32_t work_order = 0;       // hx_info.work_order
   bool checked = false;
-  int32_t* d_rec_inst = nullptr;
-  int64_t* d_rec_enq = nullptr;
-  int64_t* d_rec_budget = nullptr;
-  int64_t* d_rec_start = nullptr;
-  int64_t* d_rec_end = nullptr;
   std::vector<int32_t> record_sims;
   // the simulation kernel's family and launch for the traces as they are: [0] with
   // short calls only, [1] with one of kLongCall us or more
@@ -207,25 +204,44 @@ struct hx_sim {
   std::vector<cudaEvent_t> ev;
   int64_t runs = 0;
   cudaEvent_t* run_ev(int64_t r) { return ev.data() + 4 * (r % kTimedRuns); }
-  std::vector<void*> allocs;
+  // Everything the handle holds on the device is one block, laid out by place()
+  // and allocated by commit() (28 allocations and as many frees took 260 us of a
+  // fresh 2.8 ms window sweep; one of each takes 65).
+  unsigned char* block = nullptr;
+  std::vector<std::pair<void**, int64_t>> placed;
+  // The inputs lead it: the per-query arrays, the constants of cluster and grid and
+  // the per-call arrays.  `stage` is the same on the host, so that an upload is one
+  // copy (64 traces' 384 copies took 2.5 ms); more than kStageMost bytes of inputs
+  // keep no stage, and their per-call arrays are copied from the caller's.
+  static constexpr int64_t kStageMost = int64_t(64) << 20;
+  std::unique_ptr<unsigned char[]> stage;
+  int64_t query_bytes = 0, const_bytes = 0, input_bytes = 0;  // ends of the three parts
+  bool keep_stage() const { return input_bytes <= kStageMost; }
 
   template <class T>
-  int alloc(T** p, int64_t count) {
-    size_t bytes = (size_t)std::max<int64_t>(count, 1) * sizeof(T);
+  void place(T** p, int64_t count) {
+    placed.emplace_back(reinterpret_cast<void**>(p), device_bytes);
+    device_bytes += align_up(std::max<int64_t>(count, 1) * (int64_t)sizeof(T), 256);
+  }
+  int commit() {
     void* q = nullptr;
-    cudaError_t e = cudaMalloc(&q, bytes);
+    cudaError_t e = cudaMalloc(&q, (size_t)device_bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
-      return fail(HX_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes: " + cudaGetErrorString(e));
+      return fail(HX_ERR_OOM, "cudaMalloc of " + std::to_string(device_bytes) + " bytes: " + cudaGetErrorString(e));
     }
-    allocs.push_back(q);
-    device_bytes += (int64_t)bytes;
-    *p = static_cast<T*>(q);
+    block = static_cast<unsigned char*>(q);
+    for (const auto& p : placed) *p.first = block + p.second;
     return HX_OK;
+  }
+  // where the host copy of a device input is
+  template <class T>
+  T* staged(T* d) const {
+    return reinterpret_cast<T*>(stage.get() + (reinterpret_cast<unsigned char*>(d) - block));
   }
 
   ~hx_sim() {
-    for (void* p : allocs) cudaFree(p);
+    cudaFree(block);
     for (auto e : ev)
       if (e) cudaEventDestroy(e);
   }
@@ -420,10 +436,12 @@ void for_each_trace(const hx_trace* traces, int32_t n_traces, F fn) {
   if (first) std::rethrow_exception(first);
 }
 
-// validate_trace over every trace, in parallel; the lowest-numbered failing
-// trace's status and message are reported, as a loop in order would.
+// validate_trace over every trace, in parallel, and then pack(t); the
+// lowest-numbered failing trace's status and message are reported, as a loop in
+// order would.
+template <class F>
 int validate_traces(const hx_trace* traces, int32_t n_traces, const hx_cluster* c, int64_t min_prefill,
-                    int64_t max_decode, bool* long_calls) {
+                    int64_t max_decode, bool* long_calls, F pack) {
   std::vector<int> rc((size_t)n_traces, HX_OK);
   std::atomic<bool> any_long{false};
   std::vector<std::string> msg((size_t)n_traces);
@@ -432,6 +450,7 @@ int validate_traces(const hx_trace* traces, int32_t n_traces, const hx_cluster* 
     rc[t] = validate_trace(&traces[t], t, c, min_prefill, max_decode, &is_long);
     if (is_long) any_long = true;
     if (rc[t] != HX_OK) msg[t] = g_err;  // this thread's message
+    else pack(t);
   });
   for (int32_t t = 0; t < n_traces; ++t)
     if (rc[t] != HX_OK) return fail(rc[t], msg[t]);
@@ -446,61 +465,52 @@ int upload(T* dst, const T* src, int64_t count, cudaStream_t s) {
   return HX_OK;
 }
 
-// Top-K size of each (trace, tenant) for the per-tenant P95: n_t - ceil(0.95 n_t) + 1
-// over the tenant's n_t queries (0 without queries); at most the trace's own K.
-std::vector<int32_t> tenant_kcaps(const hx_trace* traces, int32_t n_traces) {
-  std::vector<int32_t> k((size_t)n_traces * HX_MAX_TENANTS, 0);
-  for (int t = 0; t < n_traces; ++t) {
-    int32_t n[HX_MAX_TENANTS] = {0, 0, 0, 0};
-    for (int32_t i = 0; i < traces[t].n_queries; ++i) n[traces[t].tenant ? traces[t].tenant[i] : 0]++;
-    for (int u = 0; u < HX_MAX_TENANTS; ++u)
-      k[(size_t)t * HX_MAX_TENANTS + u] = n[u] ? n[u] - (95 * n[u] + 99) / 100 + 1 : 0;
+// A validated trace's part of the staged inputs.
+void pack_trace(hx_sim* h, const hx_trace& tr, int32_t t) {
+  const int64_t qo = h->q_off[t], co = h->c_off[t], nq = tr.n_queries, nc = tr.n_calls;
+  int64_t* const qcall = h->staged(h->d_qcall) + qo;
+  for (int64_t i = 0; i < nq; ++i) qcall[i] = co + tr.call_base[i];
+  if (t == h->n_traces - 1) qcall[nq] = h->n_c;
+  if (nq > 0) {
+    std::memcpy(h->staged(h->d_arrival) + qo, tr.arrival_us, (size_t)nq * sizeof(int64_t));
+    std::memcpy(h->staged(h->d_k) + qo, tr.k, (size_t)nq);
+    if (tr.tenant) std::memcpy(h->staged(h->d_tenant) + qo, tr.tenant, (size_t)nq);
+    else std::memset(h->staged(h->d_tenant) + qo, 0, (size_t)nq);
   }
-  return k;
+  if (h->d_tenant_kcap) {
+    // top-K size of each tenant for its P95: n_t - ceil(0.95 n_t) + 1 over its n_t
+    // queries (0 without queries); at most the trace's own K
+    int32_t n[HX_MAX_TENANTS] = {0, 0, 0, 0};
+    for (int64_t i = 0; i < nq; ++i) n[tr.tenant ? tr.tenant[i] : 0]++;
+    int32_t* const kcap = h->staged(h->d_tenant_kcap) + (int64_t)t * HX_MAX_TENANTS;
+    for (int u = 0; u < HX_MAX_TENANTS; ++u) kcap[u] = n[u] ? n[u] - (95 * n[u] + 99) / 100 + 1 : 0;
+  }
+  if (h->keep_stage() && nc > 0) {
+    std::memcpy(h->staged(h->d_prompt) + co, tr.prompt, (size_t)nc * sizeof(int32_t));
+    std::memcpy(h->staged(h->d_out) + co, tr.out, (size_t)nc * sizeof(int32_t));
+    std::memcpy(h->staged(h->d_out_est) + co, tr.out_est, (size_t)nc * sizeof(int32_t));
+    std::memcpy(h->staged(h->d_stage) + co, tr.stage, (size_t)nc);
+    std::memcpy(h->staged(h->d_cand) + co, tr.cand, (size_t)nc);
+    std::memcpy(h->staged(h->d_retry) + co, tr.retry, (size_t)nc);
+  }
 }
 
-// Copies the per-call and per-query trace arrays of all traces to the device.
-int upload_traces(hx_sim* h, const hx_trace* traces, cudaStream_t s) {
-  std::vector<int64_t> arrival((size_t)h->n_q), qcall((size_t)h->n_q + 1);
-  std::vector<uint8_t> kq((size_t)h->n_q), tenant((size_t)h->n_q, 0);
-  std::vector<int64_t> q0((size_t)h->n_traces + 1, 0), c0((size_t)h->n_traces + 1, 0);
-  for (int t = 0; t < h->n_traces; ++t) {
-    q0[t + 1] = q0[t] + traces[t].n_queries;
-    c0[t + 1] = c0[t] + traces[t].n_calls;
-  }
-  for_each_trace(traces, h->n_traces, [&](int32_t t) {
-    const hx_trace& tr = traces[t];
-    const int64_t qo = q0[t], co = c0[t];
-    for (int32_t i = 0; i < tr.n_queries; ++i) {
-      arrival[qo + i] = tr.arrival_us[i];
-      kq[qo + i] = tr.k[i];
-      qcall[qo + i] = co + tr.call_base[i];
-      if (tr.tenant) tenant[qo + i] = tr.tenant[i];
-    }
-  });
-  int64_t co = c0[h->n_traces];
-  qcall[h->n_q] = co;
+// Copies the first `bytes` of the staged inputs to the device, and the per-call
+// arrays that are not staged.
+int upload_inputs(hx_sim* h, const hx_trace* traces, int64_t bytes, cudaStream_t s) {
   int rc;
-  if ((rc = upload(h->d_arrival, arrival.data(), h->n_q, s)) || (rc = upload(h->d_k, kq.data(), h->n_q, s)) ||
-      (rc = upload(h->d_tenant, tenant.data(), h->n_q, s)) || (rc = upload(h->d_qcall, qcall.data(), h->n_q + 1, s)))
-    return rc;
-  co = 0;
-  for (int t = 0; t < h->n_traces; ++t) {
+  if ((rc = upload(h->block, h->stage.get(), bytes, s))) return rc;
+  for (int t = 0; t < h->n_traces && !h->keep_stage(); ++t) {
     const hx_trace& tr = traces[t];
+    const int64_t co = h->c_off[t];
     if ((rc = upload(h->d_prompt + co, tr.prompt, tr.n_calls, s)) || (rc = upload(h->d_out + co, tr.out, tr.n_calls, s)) ||
         (rc = upload(h->d_out_est + co, tr.out_est, tr.n_calls, s)) ||
         (rc = upload(h->d_stage + co, tr.stage, tr.n_calls, s)) || (rc = upload(h->d_cand + co, tr.cand, tr.n_calls, s)) ||
         (rc = upload(h->d_retry + co, tr.retry, tr.n_calls, s)))
       return rc;
-    co += tr.n_calls;
   }
-  std::vector<int32_t> kcap;
-  if (h->d_tenant_kcap) {
-    kcap = tenant_kcaps(traces, h->n_traces);
-    if ((rc = upload(h->d_tenant_kcap, kcap.data(), (int64_t)kcap.size(), s))) return rc;
-  }
-  // the host staging vectors die here: the copies must finish first
   HX_CUDA(cudaStreamSynchronize(s));
+  if (!h->keep_stage()) h->stage.reset();
   return HX_OK;
 }
 
@@ -670,23 +680,19 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   int rc;
   if ((rc = validate_cluster(cluster, &min_prefill, &max_decode))) return rc;
   if ((rc = validate_grid(grid))) return rc;
-  bool long_calls = false;
-  if ((rc = validate_traces(traces, n_traces, cluster, min_prefill, max_decode, &long_calls))) return rc;
-  if (opt && opt->n_record < 0) return fail(HX_ERR_INVALID, "n_record < 0");
-  if (opt && opt->n_record > 0) {
-    if (!opt->record_sims) return fail(HX_ERR_INVALID, "record_sims is NULL");
-    std::vector<int32_t> sorted(opt->record_sims, opt->record_sims + opt->n_record);
-    std::sort(sorted.begin(), sorted.end());
-    const int64_t n_sims = (int64_t)n_traces * grid->n_points;
-    for (size_t j = 0; j < sorted.size(); ++j)
-      if (sorted[j] < 0 || sorted[j] >= n_sims || (j > 0 && sorted[j] == sorted[j - 1]))
-        return fail(HX_ERR_INVALID, "record_sims must be distinct valid sim indices");
+  auto validate = [&](bool* long_calls, auto pack) {
+    return validate_traces(traces, n_traces, cluster, min_prefill, max_decode, long_calls, pack);
+  };
+  int64_t n_calls = 0;
+  bool bad_counts = false, long_calls = false;
+  for (int32_t i = 0; i < n_traces; ++i) {
+    bad_counts |= traces[i].n_queries < 0 || traces[i].n_calls < 0 || traces[i].n_calls >= (1 << 24);
+    n_calls += traces[i].n_calls;
   }
-  if (opt && opt->checked != 0 && opt->checked != 1) return fail(HX_ERR_INVALID, "checked must be 0 or 1");
-  if (opt && opt->arena_entries < 0) return fail(HX_ERR_INVALID, "arena_entries < 0");
-  std::vector<int64_t> subset;
-  if ((rc = order_subset(opt, n_traces, grid->n_points, &subset))) return rc;
-
+  if (bad_counts || n_calls >= (int64_t(1) << 31)) {
+    if ((rc = validate(&long_calls, [](int32_t) {}))) return rc;
+    return fail(HX_ERR_INVALID, "more than 2^31 calls in total");
+  }
   // the handle is freed on every early return (and exception) until it is handed out
   std::unique_ptr<hx_sim> owner(new (std::nothrow) hx_sim());
   hx_sim* h = owner.get();
@@ -695,7 +701,9 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   h->n_traces = n_traces;
   h->n_points = grid->n_points;
   h->n_sims = (int64_t)n_traces * grid->n_points;
-  std::vector<int64_t> q_off(n_traces + 1, 0), c_off(n_traces + 1, 0);
+  std::vector<int64_t>&q_off = h->q_off, &c_off = h->c_off;
+  q_off.assign((size_t)n_traces + 1, 0);
+  c_off.assign((size_t)n_traces + 1, 0);
   for (int t = 0; t < n_traces; ++t) {
     const int32_t nq = traces[t].n_queries, nc = traces[t].n_calls;
     h->h_nq.push_back(nq);
@@ -708,46 +716,79 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   }
   h->n_q = q_off[n_traces];
   h->n_c = c_off[n_traces];
-  h->n_work = subset.empty() ? h->n_sims : (int64_t)subset.size();
-  h->checked = opt && opt->checked == 1;
-  if (h->n_c >= (int64_t(1) << 31)) return bail(fail(HX_ERR_INVALID, "more than 2^31 calls in total"));
-
   // cluster constants (kernel parameter)
   hx::ClusterK& ck = h->ck;
   fill_cluster(cluster, ck);
   h->n_tenants = cluster->n_tenants;
   h->faults.assign(cluster->faults, cluster->faults + cluster->n_faults);
 
+  // the inputs: per-query arrays and constants, then the per-call arrays
+  const bool tenants = ck.n_tenants > 1;
+  h->place(&h->d_arrival, h->n_q);
+  h->place(&h->d_qcall, h->n_q + 1);
+  h->place(&h->d_k, h->n_q);
+  h->place(&h->d_tenant, h->n_q);
+  if (tenants) h->place(&h->d_tenant_kcap, (int64_t)n_traces * HX_MAX_TENANTS);
+  h->query_bytes = h->device_bytes;
+  h->place(&h->d_q_off, n_traces + 1);
+  h->place(&h->d_c_off, n_traces + 1);
+  h->place(&h->d_alpha, h->n_points);
+  h->place(&h->d_gamma, h->n_points);
+  h->place(&h->d_beta, h->n_points);
+  h->place(&h->d_rho, h->n_points);
+  h->place(&h->d_lp, h->n_points);
+  h->place(&h->d_dp, h->n_points);
+  h->const_bytes = h->device_bytes;
+  h->place(&h->d_prompt, h->n_c);
+  h->place(&h->d_out, h->n_c);
+  h->place(&h->d_out_est, h->n_c);
+  h->place(&h->d_stage, h->n_c);
+  h->place(&h->d_cand, h->n_c);
+  h->place(&h->d_retry, h->n_c);
+  h->input_bytes = h->device_bytes;
+  const int64_t staged_bytes = h->keep_stage() ? h->input_bytes : h->const_bytes;
+  h->stage.reset(new unsigned char[(size_t)staged_bytes]);
+  // staged() needs the offsets only: the block is allocated when its size is known
+  for (const auto& p : h->placed) *p.first = h->block + p.second;
+  if ((rc = validate(&long_calls, [&](int32_t i) { pack_trace(h, traces[i], i); }))) return bail(rc);
+  if (opt && opt->n_record < 0) return bail(fail(HX_ERR_INVALID, "n_record < 0"));
+  if (opt && opt->n_record > 0) {
+    if (!opt->record_sims) return bail(fail(HX_ERR_INVALID, "record_sims is NULL"));
+    std::vector<int32_t> sorted(opt->record_sims, opt->record_sims + opt->n_record);
+    std::sort(sorted.begin(), sorted.end());
+    const int64_t n_sims = (int64_t)n_traces * grid->n_points;
+    for (size_t j = 0; j < sorted.size(); ++j)
+      if (sorted[j] < 0 || sorted[j] >= n_sims || (j > 0 && sorted[j] == sorted[j - 1]))
+        return bail(fail(HX_ERR_INVALID, "record_sims must be distinct valid sim indices"));
+  }
+  if (opt && opt->checked != 0 && opt->checked != 1) return bail(fail(HX_ERR_INVALID, "checked must be 0 or 1"));
+  if (opt && opt->arena_entries < 0) return bail(fail(HX_ERR_INVALID, "arena_entries < 0"));
+  std::vector<int64_t> subset;
+  if ((rc = order_subset(opt, n_traces, grid->n_points, &subset))) return bail(rc);
+
+  h->n_work = subset.empty() ? h->n_sims : (int64_t)subset.size();
+  h->checked = opt && opt->checked == 1;
+  std::copy(q_off.begin(), q_off.end(), h->staged(h->d_q_off));
+  std::copy(c_off.begin(), c_off.end(), h->staged(h->d_c_off));
+  std::copy_n(grid->alpha_fp, h->n_points, h->staged(h->d_alpha));
+  std::copy_n(grid->gamma_fp, h->n_points, h->staged(h->d_gamma));
+  std::copy_n(grid->beta_us2, h->n_points, h->staged(h->d_beta));
+  std::copy_n(grid->rho, h->n_points, h->staged(h->d_rho));
+  std::copy_n(grid->local_policy, h->n_points, h->staged(h->d_lp));
+  std::copy_n(grid->dispatch_policy, h->n_points, h->staged(h->d_dp));
   int dev = 0;
   cudaDeviceProp prop;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) {
     cudaGetLastError();
     return bail(fail(HX_ERR_CUDA, "no CUDA device"));
   }
-  // device inputs
-  if ((rc = h->alloc(&h->d_arrival, h->n_q)) || (rc = h->alloc(&h->d_k, h->n_q)) ||
-      (rc = h->alloc(&h->d_tenant, h->n_q)) ||
-      (rc = h->alloc(&h->d_qcall, h->n_q + 1)) || (rc = h->alloc(&h->d_q_off, n_traces + 1)) ||
-      (rc = h->alloc(&h->d_c_off, n_traces + 1)) || (rc = h->alloc(&h->d_prompt, h->n_c)) ||
-      (rc = h->alloc(&h->d_out, h->n_c)) || (rc = h->alloc(&h->d_out_est, h->n_c)) ||
-      (rc = h->alloc(&h->d_stage, h->n_c)) || (rc = h->alloc(&h->d_cand, h->n_c)) ||
-      (rc = h->alloc(&h->d_retry, h->n_c)) || (rc = h->alloc(&h->d_alpha, h->n_points)) ||
-      (rc = h->alloc(&h->d_gamma, h->n_points)) || (rc = h->alloc(&h->d_beta, h->n_points)) ||
-      (rc = h->alloc(&h->d_rho, h->n_points)) || (rc = h->alloc(&h->d_lp, h->n_points)) ||
-      (rc = h->alloc(&h->d_dp, h->n_points)) || (rc = h->alloc(&h->d_rec, h->n_c)) ||
-      (rc = h->alloc(&h->d_results, h->n_sims)) || (rc = h->alloc(&h->d_counter, 1)) ||
-      (rc = h->alloc(&h->d_best_trace, 2 * (int64_t)n_traces)) || (rc = h->alloc(&h->d_best_global, 2)) ||
-      (rc = h->alloc(&h->d_point_sums, 3 * (int64_t)h->n_points)))
-    return bail(rc);
-  cudaStream_t s0 = nullptr;
-  if ((rc = upload_traces(h, traces, s0)) || (rc = upload(h->d_q_off, q_off.data(), n_traces + 1, s0)) ||
-      (rc = upload(h->d_c_off, c_off.data(), n_traces + 1, s0)) ||
-      (rc = upload(h->d_alpha, grid->alpha_fp, h->n_points, s0)) ||
-      (rc = upload(h->d_gamma, grid->gamma_fp, h->n_points, s0)) ||
-      (rc = upload(h->d_beta, grid->beta_us2, h->n_points, s0)) || (rc = upload(h->d_rho, grid->rho, h->n_points, s0)) ||
-      (rc = upload(h->d_lp, grid->local_policy, h->n_points, s0)) ||
-      (rc = upload(h->d_dp, grid->dispatch_policy, h->n_points, s0)))
-    return bail(rc);
+  // derived and outputs
+  h->place(&h->d_rec, h->n_c);
+  h->place(&h->d_results, h->n_sims);
+  h->place(&h->d_counter, 1);
+  h->place(&h->d_best_trace, 2 * (int64_t)n_traces);
+  h->place(&h->d_best_global, 2);
+  h->place(&h->d_point_sums, 3 * (int64_t)h->n_points);
 
   // launch shapes of the simulation kernel; later uploads may bring longer calls
   int64_t blocks = (h->n_sims + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock;
@@ -763,54 +804,51 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   h->work_order = subset.empty()
                       ? costliest_first(grid, n_traces, h->n_c, (int64_t)prop.l2CacheSize, resident_warps, &subset)
                       : 1;
-  if (!subset.empty() && ((rc = h->alloc(&h->d_subset, (int64_t)subset.size())) ||
-                          (rc = upload(h->d_subset, subset.data(), (int64_t)subset.size(), s0))))
-    return bail(rc);
+  if (!subset.empty()) h->place(&h->d_subset, (int64_t)subset.size());
   // heap arena: doubling regions of 16, 32, ... entries per instance total at
   // most 4 * (requests ever queued) + 16 * instances
   h->arena_per_warp = 4 * (int64_t)h->max_nc + 16 * HX_MAX_INST;
   if (opt && opt->arena_entries > 0) h->arena_per_warp = opt->arena_entries;
   h->chains_per_warp = align_up(std::max(h->max_nq, 1), 256);
   h->topk_per_warp = align_up(h->max_kcap, 32);
-  if (ck.n_tenants > 1) {
+  if (tenants) {
     // one more heap per tenant after the simulation's own, each sized for a
     // whole trace (a tenant's K never exceeds its trace's), so uploads of new
     // tenant assignments need no reallocation
     for (int t = 0; t < HX_MAX_TENANTS; ++t) h->tenant_topk_off[t] = h->topk_per_warp * (1 + t);
     h->topk_per_warp *= 1 + HX_MAX_TENANTS;
-    if ((rc = h->alloc(&h->d_tenant_kcap, (int64_t)n_traces * HX_MAX_TENANTS))) return bail(rc);
-    const std::vector<int32_t> kcap = tenant_kcaps(traces, n_traces);
-    if ((rc = upload(h->d_tenant_kcap, kcap.data(), (int64_t)kcap.size(), s0))) return bail(rc);
-    if (cudaStreamSynchronize(s0) != cudaSuccess) return bail(fail(HX_ERR_CUDA, "tenant upload failed"));
   }
   const int64_t w = hx::kWarpsPerBlock * (int64_t)std::max(h->launch[0].blocks, h->launch[1].blocks);
-  if ((rc = h->alloc(&h->d_arena, w * h->arena_per_warp)) || (rc = h->alloc(&h->d_chains, w * h->chains_per_warp)) ||
-      (rc = h->alloc(&h->d_topk, w * h->topk_per_warp)))
-    return bail(rc);
-  if (family >= hx::kSimGeneric && (rc = h->alloc(&h->d_extras, h->n_sims))) return bail(rc);
+  h->place(&h->d_arena, w * h->arena_per_warp);
+  h->place(&h->d_chains, w * h->chains_per_warp);
+  h->place(&h->d_topk, w * h->topk_per_warp);
+  if (family >= hx::kSimGeneric) h->place(&h->d_extras, h->n_sims);
   h->scratch_bytes = w * (h->arena_per_warp * (int64_t)sizeof(hx::HeapEnt) + h->chains_per_warp +
                           h->topk_per_warp * (int64_t)sizeof(int64_t));
 
-  // per-call logs of selected simulations
+  // per-call logs of selected simulations: enq, budget, start, end (int64) and inst
+  // (int32) of one simulation side by side, so that they are read back in one copy
+  std::vector<int32_t> map;
   if (opt && opt->n_record > 0) {
     h->n_record = opt->n_record;
-    h->rec_stride = std::max(h->max_nc, 1);
-    std::vector<int32_t> map((size_t)h->n_sims, -1);
+    h->rec_calls = std::max(h->max_nc, 1);
+    h->rec_stride = 4 * h->rec_calls + (h->rec_calls + 1) / 2;
+    map.assign((size_t)h->n_sims, -1);
     for (int j = 0; j < opt->n_record; ++j) {
       const int32_t sim = opt->record_sims[j];  // checked above: distinct, in range
       map[sim] = j;
       h->record_sims.push_back(sim);
     }
-    const int64_t n = (int64_t)h->n_record * h->rec_stride;
-    if ((rc = h->alloc(&h->d_rec_map, h->n_sims)) || (rc = h->alloc(&h->d_rec_sims, h->n_record)) ||
-        (rc = h->alloc(&h->d_rec_inst, n)) ||
-        (rc = h->alloc(&h->d_rec_enq, n)) || (rc = h->alloc(&h->d_rec_budget, n)) ||
-        (rc = h->alloc(&h->d_rec_start, n)) || (rc = h->alloc(&h->d_rec_end, n)) ||
-        (rc = upload(h->d_rec_map, map.data(), h->n_sims, s0)) ||
-        (rc = upload(h->d_rec_sims, opt->record_sims, h->n_record, s0)))
-      return bail(rc);
-    if (cudaStreamSynchronize(s0) != cudaSuccess) return bail(fail(HX_ERR_CUDA, "record map upload failed"));
+    h->place(&h->d_rec_map, h->n_sims);
+    h->place(&h->d_rec_sims, h->n_record);
+    h->place(&h->d_rec_log, h->n_record * h->rec_stride);
   }
+  if ((rc = h->commit())) return bail(rc);
+  cudaStream_t s0 = nullptr;
+  if ((rc = upload_inputs(h, traces, staged_bytes, s0)) || (rc = upload(h->d_subset, subset.data(), (int64_t)subset.size(), s0)) ||
+      (rc = upload(h->d_rec_map, map.data(), (int64_t)map.size(), s0)) ||
+      (rc = upload(h->d_rec_sims, h->record_sims.data(), h->n_record, s0)))
+    return bail(rc);
   if (opt && opt->timing) {
     h->timing = true;
     h->ev.assign(4 * hx_sim::kTimedRuns, nullptr);
@@ -843,12 +881,16 @@ static int hx_sim_upload_impl(hx_sim* h, const hx_trace* traces, int32_t n_trace
   c.n_faults = (int32_t)h->faults.size();
   c.faults = h->faults.data();
   bool long_calls = false;
-  int rc = validate_traces(traces, n_traces, &c, min_prefill, max_decode, &long_calls);
+  if (!h->stage) h->stage.reset(new unsigned char[(size_t)h->query_bytes]);
+  int rc = validate_traces(traces, n_traces, &c, min_prefill, max_decode, &long_calls,
+                           [&](int32_t t) { pack_trace(h, traces[t], t); });
   if (rc) return rc;
   // set first: a copy that fails half-way may leave long calls behind
   const bool had_long = h->long_calls;
   h->long_calls = had_long || long_calls;
-  if ((rc = upload_traces(h, traces, static_cast<cudaStream_t>(stream)))) return rc;
+  if ((rc = upload_inputs(h, traces, h->keep_stage() ? h->input_bytes : h->query_bytes,
+                          static_cast<cudaStream_t>(stream))))
+    return rc;
   h->long_calls = long_calls;
   return HX_OK;
 }
@@ -902,10 +944,11 @@ static int hx_sim_run_impl(hx_sim* h, void* stream) {
   sa.topk = h->d_topk;
   sa.topk_per_warp = h->topk_per_warp;
   sa.rec_map = h->d_rec_map;
-  sa.rec_inst = h->d_rec_inst;
-  sa.rec_enq = h->d_rec_enq;
-  sa.rec_start = h->d_rec_start;
-  sa.rec_end = h->d_rec_end;
+  sa.rec_inst = reinterpret_cast<int32_t*>(h->d_rec_log + 4 * h->rec_calls);
+  sa.rec_enq = h->d_rec_log;
+  sa.rec_start = h->d_rec_log + 2 * h->rec_calls;
+  sa.rec_end = h->d_rec_log + 3 * h->rec_calls;
+  sa.rec_calls = h->rec_calls;
   sa.rec_stride = h->rec_stride;
   sa.extras = h->d_extras;
   sa.tenant_kcap = h->d_tenant_kcap;
@@ -938,10 +981,11 @@ static int hx_sim_run_impl(hx_sim* h, void* stream) {
     la.record_sims = h->d_rec_sims;
     la.n_record = h->n_record;
     la.n_points = h->n_points;
-    la.rec_enq = h->d_rec_enq;
-    la.rec_budget = h->d_rec_budget;
+    la.rec_enq = h->d_rec_log;
+    la.rec_budget = h->d_rec_log + h->rec_calls;
+    la.rec_calls = h->rec_calls;
     la.rec_stride = h->rec_stride;
-    const int64_t log_blocks = (h->rec_stride + 255) / 256 * h->n_record;
+    const int64_t log_blocks = (h->rec_calls + 255) / 256 * h->n_record;
     hx::hx_log_kernel<<<(unsigned)std::min<int64_t>(log_blocks, 1 << 16), 256, 0, s>>>(la, h->ck);
     HX_CUDA(cudaGetLastError());
   }
@@ -1085,13 +1129,15 @@ static int hx_sim_records_impl(hx_sim* h, int32_t rec_index, int32_t* inst, int6
   const int t = (int)(h->record_sims[rec_index] / h->n_points);
   if ((int64_t)n_calls != h->h_nc[t]) return fail(HX_ERR_INVALID, "n_calls differs from the trace's");
   HX_CUDA(cudaStreamSynchronize(h->last_stream));
-  const int64_t o = (int64_t)rec_index * h->rec_stride;
   if (n_calls == 0) return HX_OK;
-  if (inst) HX_CUDA(cudaMemcpy(inst, h->d_rec_inst + o, n_calls * sizeof(int32_t), cudaMemcpyDeviceToHost));
-  if (enq_us) HX_CUDA(cudaMemcpy(enq_us, h->d_rec_enq + o, n_calls * sizeof(int64_t), cudaMemcpyDeviceToHost));
-  if (budget_us) HX_CUDA(cudaMemcpy(budget_us, h->d_rec_budget + o, n_calls * sizeof(int64_t), cudaMemcpyDeviceToHost));
-  if (start_us) HX_CUDA(cudaMemcpy(start_us, h->d_rec_start + o, n_calls * sizeof(int64_t), cudaMemcpyDeviceToHost));
-  if (end_us) HX_CUDA(cudaMemcpy(end_us, h->d_rec_end + o, n_calls * sizeof(int64_t), cudaMemcpyDeviceToHost));
+  // one copy of the simulation's log, then its columns
+  const int64_t* const d = h->d_rec_log + (int64_t)rec_index * h->rec_stride;
+  std::unique_ptr<int64_t[]> log(new int64_t[(size_t)h->rec_stride]);
+  HX_CUDA(cudaMemcpy(log.get(), d, (size_t)h->rec_stride * sizeof(int64_t), cudaMemcpyDeviceToHost));
+  int64_t* const cols[4] = {enq_us, budget_us, start_us, end_us};
+  for (int i = 0; i < 4; ++i)
+    if (cols[i]) std::memcpy(cols[i], log.get() + i * h->rec_calls, n_calls * sizeof(int64_t));
+  if (inst) std::memcpy(inst, log.get() + 4 * h->rec_calls, n_calls * sizeof(int32_t));
   return HX_OK;
 }
 
@@ -1381,6 +1427,7 @@ static int hx_sim_run_static_impl(const hx_trace* trace, const hx_cluster* clust
   sa.rec_enq = nullptr;
   sa.rec_start = nullptr;
   sa.rec_end = nullptr;
+  sa.rec_calls = 0;
   sa.rec_stride = 0;
   sa.extras = nullptr;
   sa.tenant_kcap = nullptr;

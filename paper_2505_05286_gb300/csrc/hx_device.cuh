@@ -128,7 +128,7 @@ struct SimArgs {
   int64_t* rec_enq;
   int64_t* rec_start;
   int64_t* rec_end;
-  int64_t rec_stride;
+  int64_t rec_calls, rec_stride;  // calls and int64 units per logged simulation
   hx_extra* extras;         // [n_sims] per-tenant counts and re-issues (generic kernel), or NULL
   const int32_t* tenant_kcap;  // [n_traces * 4] top-K size per (trace, tenant) (0: no queries), or
                                // NULL: one tenant
@@ -211,7 +211,7 @@ struct LogArgs {
   int32_t n_record, n_points;
   const int64_t* rec_enq;
   int64_t* rec_budget;
-  int64_t rec_stride;
+  int64_t rec_calls, rec_stride;
 };
 
 struct BestArgs {

@@ -1071,9 +1071,9 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         for (int j = 0; j < J; ++j) q[j] += lane + 32 * j == m ? est : 0;
         if (kLog && recj >= 0) {
           // (the budget at send time follows from these: hx_log_kernel)
-          HX_BOUND(rid < a.rec_stride)
+          HX_BOUND(rid < a.rec_calls)
           if (lane == 0) {
-            a.rec_inst[(int64_t)recj * a.rec_stride + rid] = m;
+            a.rec_inst[2 * (int64_t)recj * a.rec_stride + rid] = m;
             a.rec_enq[(int64_t)recj * a.rec_stride + rid] = absolute(now);
           }
         }
@@ -1281,7 +1281,7 @@ const SimKernel kSimKernel[kSimKernels] = {HX_FORMS(hx_sim_kernel_lean), HX_FORM
 // sweep waits for.
 __global__ void __launch_bounds__(256) hx_log_kernel(LogArgs a, ClusterK c) {
   __shared__ int64_t rest[kFRows];
-  const int64_t per = (a.rec_stride + 255) / 256;  // blocks of calls per simulation
+  const int64_t per = (a.rec_calls + 255) / 256;  // blocks of calls per simulation
   for (int64_t b = blockIdx.x; b < per * a.n_record; b += gridDim.x) {
     const int64_t j = b / per;
     const int64_t sim = a.record_sims[j], t = sim / a.n_points;

@@ -1,0 +1,47 @@
+"""New traces on a kept handle: inputs that are staged on the host and copied at
+once, and inputs past the stage's size, whose per-call arrays are copied from the
+caller's; with and without tenants, and after a rejected upload."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2505_05286_gb300 import build as B
+from paper_2505_05286_gb300 import hxsim as H
+from paper_2505_05286_gb300 import workloads as W
+
+FIELDS = ["p95_us", "makespan_us", "events", "digest", "slo_met", "n_done", "status"]
+
+
+def _traces(recipe, n, nq, seed):
+    # no corrections: every seed gives the same shapes
+    r = W.Recipe(**{**recipe.__dict__, "p_err": 0.0})
+    return [W.make_trace(r, 1, seed * 100 + t, n_queries=nq) for t in range(n)], W.make_cluster(r)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("tenants", [False, True])
+@pytest.mark.parametrize("n,nq", [(3, 50), (38, 20000)])  # 13 KB, and 68 MB of calls (the stage holds 64)
+def test_upload_replaces_every_input(n, nq, tenants):
+    B.build()
+    recipe = W.EXTRA["two-tenant"] if tenants else W.RECIPES[1]
+    a, cl = _traces(recipe, n, nq, 1)
+    b, _ = _traces(recipe, n, nq, 2)
+    grid = W.subset_grid(W.make_grid(recipe), [0, 40])
+    sims = [1, 2 * n - 2]  # first and last trace
+    sim = H.Sim(a, cl, grid, subset=sims)
+    bad = list(b)
+    bad[-1] = W.Trace(**{**b[-1].__dict__, "prompt": b[-1].prompt * 0})
+    for step, traces in enumerate((a, b, b, a)):
+        if step == 2:  # refused: the handle keeps what it has
+            with pytest.raises(H.HxError):
+                sim.upload(bad)
+        elif step:
+            sim.upload(traces)
+        sim.run()
+        got = sim.results()[sims]
+        want, extra = oracle.run(W.Workload("upload", traces, cl, grid, 0), sims, extra=True)
+        for f in FIELDS:
+            assert np.array_equal(got[f], want[f]), f
+        if tenants:
+            assert np.array_equal(sim.extras()[sims]["p95_us"], extra["p95_us"])
+    sim.close()
