@@ -58,15 +58,18 @@ __device__ __forceinline__ int warp_argmax_s64(int64_t s, int idx) {
 // conversions, the approximate reciprocal, one product), so below 2^30 the
 // remainder's quotient is below 2^9 and the refined estimate within one of n/d.
 // Quotients of 2^30 or more take the exact integer path.
-__device__ __forceinline__ uint64_t udiv_trial(uint64_t n, uint64_t d) {
-  float rd;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"((float)d));
-  const float qf = (float)n * rd;
-  if (qf >= 1073741824.0f) return n / d;
+__device__ __forceinline__ uint64_t udiv_refine(uint64_t n, uint64_t d, float rd, float qf) {
   uint64_t q = (uint32_t)qf;
   q += (int64_t)(int32_t)((float)(int64_t)(n - q * d) * rd);
   const int64_t r = (int64_t)(n - q * d);
   return q - (r < 0 ? 1 : 0) + (r >= (int64_t)d ? 1 : 0);
+}
+
+__device__ __forceinline__ uint64_t udiv_trial(uint64_t n, uint64_t d) {
+  float rd;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"((float)d));
+  const float qf = (float)n * rd;
+  return qf >= 1073741824.0f ? n / d : udiv_refine(n, d, rd, qf);
 }
 
 // Workload-balanced reward term of Eq. (score): beta / max(t_queue, 1), capped.
@@ -355,16 +358,26 @@ __device__ __forceinline__ bool ent_better(const HeapEnt& a, const HeapEnt& b) {
   return (a.key > b.key) | ((a.key == b.key) & (a.rid < b.rid));
 }
 
-// A heap entry in one 16-byte access, under a predicate and not a branch;
-// without it the load leaves an entry that goes after every other.
+// A heap entry in one 16-byte access.
+__device__ __forceinline__ HeapEnt ent_load(const HeapEnt* p) {
+  HeapEnt e;
+  uint32_t lo, hi;
+  asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(lo), "=r"(hi), "=r"(e.rid), "=r"(e.svc)
+               : "l"(p)
+               : "memory");
+  e.key = (unsigned long long)hi << 32 | lo;
+  return e;
+}
+
+// The same under a predicate and not a branch; without it the key is 0, below
+// every key (rid and svc are whatever they were).
 __device__ __forceinline__ HeapEnt ent_load(const HeapEnt* p, bool on) {
   HeapEnt e;
   uint32_t lo = 0, hi = 0;
-  e.rid = INT_MAX;
-  e.svc = 0;
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.s32 p, %5, 0;\n @p ld.global.v4.b32 {%0, %1, %2, %3}, [%4];\n}"
-      : "+r"(lo), "+r"(hi), "+r"(e.rid), "+r"(e.svc)
+      : "+r"(lo), "+r"(hi), "=r"(e.rid), "=r"(e.svc)
       : "l"(p), "r"((int)on)
       : "memory");
   e.key = (unsigned long long)hi << 32 | lo;
@@ -391,7 +404,7 @@ __device__ __forceinline__ void heap_push(HeapEnt* h, int n, HeapEnt e) {
   int i = n;
   while (i > 0) {
     const int par = (i - 1) >> 5;
-    const HeapEnt pe = ent_load(h + par, true);
+    const HeapEnt pe = ent_load(h + par);
     if (!ent_better(e, pe)) break;
     ent_store(h + i, pe, true);
     i = par;
@@ -497,18 +510,38 @@ __device__ __forceinline__ int64_t slo_budget(int64_t num, int64_t tb, int64_t d
   return budget_wide(num, tb, dd);
 }
 
+__device__ __noinline__ int64_t budget_exact(int64_t num, int64_t tb, int64_t dd) { return slo_budget(num, tb, dd); }
+
 // Local-queue key, higher first, of a request dispatched now: Eq. (priority)
 // with the budget at send time (now) and the common now dropped; FCFS: earliest
 // enqueue; LLF: least deadline - now - remaining work, again with the common
-// now dropped.  est is its Eq. (comp) on the instance.
+// now dropped.  est is its Eq. (comp) on the instance.  All lanes call, those
+// without a request with some other, so that its branches are uniform.
 __device__ __forceinline__ unsigned long long queue_key(const WarpShared* W, const CallRec* r, int est, int64_t now, int lpol) {
   const int64_t dl = r->deadline;
   const int4 tail = *reinterpret_cast<const int4*>(&r->tbar);
   const int64_t tb = tail.x;
   const int64_t dd = tb + W->frest[(tail.w >> 16) & 0xff];
-  const int64_t key = lpol == HX_LOCAL_PQ     ? kScale * ((int64_t)est - slo_budget(dl - now, tb, dd)) - W->G * now
-                      : lpol == HX_LOCAL_FCFS ? -now
-                                              : dd - dl;
+  int64_t key;
+  if (lpol == HX_LOCAL_PQ) {
+    // slo_budget with one uniform branch: |num| * tbar below 2^62 and a quotient
+    // below 2^30 on every lane, or all lanes take the exact divisions
+    const int64_t num = dl - now;
+    const uint64_t n = (uint64_t)(num < 0 ? -num : num);
+    float rd;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"((float)dd));
+    const float qf = (float)(n * (uint64_t)tb) * rd;
+    int64_t budget;
+    if (__all_sync(kFull, ((n >> 34) == 0) & (qf < 1073741824.0f))) {
+      const uint64_t res = udiv_refine(n * (uint64_t)tb, (uint64_t)dd, rd, qf);
+      budget = num < 0 ? -(int64_t)res : (int64_t)res;
+    } else {
+      budget = budget_exact(num, tb, dd);
+    }
+    key = kScale * ((int64_t)est - budget) - W->G * now;
+  } else {
+    key = lpol == HX_LOCAL_FCFS ? -now : dd - dl;
+  }
   return (unsigned long long)key ^ 1ull << 63;
 }
 
@@ -1128,8 +1161,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
           }
           HeapEnt e;
           if (pm) {
-            e.key = (hs > 0 || __popc(pm) > __popc(free)) && ((pm >> lane) & 1u)
-                        ? queue_key(W, rec + pe.x, pe.z, absolute(now), lpol) : 0;
+            e.key = hs > 0 || __popc(pm) > __popc(free) ? queue_key(W, rec + pe.x, pe.z, absolute(now), lpol) : 0;
             e.rid = pe.x;
             e.svc = pe.y;
           }
@@ -1138,7 +1170,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
             // the queue's top, or to the new request if that is more urgent; the
             // queue's last entry or the new one sinks from the top.
             HeapEnt kid = heap_child(h, 0, hs, lane);
-            const HeapEnt top = ent_load(h, true);
+            const HeapEnt top = ent_load(h);
             int n = hs;
             bool fresh = false;
             if (pm) {
@@ -1148,7 +1180,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
               e.svc = __shfl_sync(kFull, e.svc, j);
               fresh = __any_sync(kFull, ent_better(e, top));
             } else {
-              e = ent_load(h + --n, true);
+              e = ent_load(h + --n);
               if (lane + 1 >= n) kid.key = 0;  // the last entry is no child any more
               inst[m].hsize = n;  // every lane writes the same size
             }
@@ -1175,7 +1207,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
                 rid = __shfl_sync(kFull, pe.x, j);
                 svc = __shfl_sync(kFull, pe.y, j);
               } else {
-                const HeapEnt top = ent_load(h, true), last = ent_load(h + --n, true);
+                const HeapEnt top = ent_load(h), last = ent_load(h + --n);
                 rid = top.rid;
                 svc = top.svc;
                 inst[m].hsize = n;  // every lane writes the same size
