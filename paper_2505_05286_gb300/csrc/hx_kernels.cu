@@ -626,6 +626,7 @@ __device__ __forceinline__ void finish_query(WarpShared* W, int64_t now, int64_t
 #define HX_SIM_MIN_BLOCKS(J) ((J) == 1 ? 8 : 7)
 #endif
 constexpr int kFewMinBlocks = 5;
+constexpr int kLongQueue = 128;  // entries (512: 27.0 ms)
 
 // Bounds-checked build (-DHX_CHECKED): before every shared- or global-memory
 // access whose index the simulation forms from its own state (instance,
@@ -840,6 +841,17 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
 
     // one instance per lane: 16 slot entries each, so that no load gives the first
     auto first_slot = [&](int m, const InstState& I) -> uint32_t { return J == 1 ? 16u * m : I.cfg >> 16; };
+    // A request starts that waited in a long queue: its record's second half and
+    // the records that follow have left L1 since its query arrived (3000 queries on
+    // 64 instances, whose alpha = 1 queue grows past 1000: 29.0 -> 26.4 ms).  Left
+    // out with one instance per lane, where it cost the sweeps 1 to 2 %: their
+    // queues stayed short.
+    auto fetch_after = [&](int32_t rid) {
+      const int64_t off = (int64_t)rid * 64 + 32 + 32 * lane;
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&W->sink);
+      const char* const from = reinterpret_cast<const char*>(rec) + off;
+      if (off < (int64_t)nc * 64) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(from) : "memory");
+    };
     auto queue_of = [&](uint32_t heap) -> HeapEnt* {
       HeapEnt* const arena = W->arena;
       __builtin_assume(__isGlobal(arena));
@@ -1196,6 +1208,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
             }
             const int rid = fresh ? e.rid : top.rid, svc = fresh ? e.svc : top.svc;
             HX_BOUND(rid >= 0 && rid < nc)
+            if (kFew && J == 2 && n >= kLongQueue) fetch_after(rid);
             start_call(m, free, slot_base, rid, svc);
             if (!fresh) heap_sift_warp(h, n, e, kid, lane);
           } else {
