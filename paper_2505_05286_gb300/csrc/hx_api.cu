@@ -96,10 +96,12 @@ int sim_kernel_of(int family, const hx::ClusterK& ck, bool few) {
   return 4 * family + (few ? 2 : 0) + (ck.n_inst <= 32 ? 1 : 0);
 }
 
-// Few warps: up to 12 per SM, whose active queries fit L1 (the fetch alone: 512
-// warps 10.9 -> 7.9 ms on 8 traces x 2000 queries x 64 points; 1536 warps
-// 19.3 -> 18.3 ms; 2560 warps +4 %, a full GPU +1-3 %).
-bool few_warps(int64_t warps, int sms) { return warps <= 12 * (int64_t)sms; }
+// Few warps: up to the 20 per SM that those kernels' registers let reside.  Against
+// the full GPU's form: 1216 to 3040 warps 6 to 22 % faster (36 traces x 2000
+// queries x 64 points 11.5 -> 8.9 ms, 2560 warps on 64 instances 80 -> 75 ms); runs
+// of several waves are faster in the full form (8192 simulations on 16 instances
+// 119 ms against 137).
+bool few_warps(int64_t warps, int sms) { return warps <= 20 * (int64_t)sms; }
 
 int ensure_dyn_smem(int kernel, int bytes) {
   int dev = 0;
