@@ -121,10 +121,10 @@ int ensure_dyn_smem(int kernel, int bytes) {
 
 // The family of the simulation kernel that serves a run: the lean one serves
 // grids that are all workload-balanced dispatch with the urgency queue, log
-// nothing, check nothing, count one tenant and have no fault windows; the wide
-// one serves fault windows and traces with a call of kLongCall us or more.
+// nothing, check nothing, count one tenant and have no fault windows.  (The wide
+// one serves any run of traces with an attempt of kLongCall us or more.)
 int sim_family(const hx_grid* grid, const hx::ClusterK& ck, bool record, bool force, bool checked) {
-  if (ck.n_faults > 0) return hx::kSimWide;
+  if (ck.n_faults > 0) return hx::kSimFaults;
   bool generic = force || checked || ck.n_tenants > 1;
   for (int p = 0; p < grid->n_points; ++p)
     generic |= grid->local_policy[p] != HX_LOCAL_PQ || grid->dispatch_policy[p] != HX_DISPATCH_WB;
@@ -190,7 +190,7 @@ struct hx_sim {
   bool checked = false;
   std::vector<int32_t> record_sims;
   // the simulation kernel's family and launch for the traces as they are: [0] with
-  // short calls only, [1] with one of kLongCall us or more
+  // short calls only, [1] with an attempt of kLongCall us or more
   struct Launch {
     int family = hx::kSimWide, kernel = 0, blocks = 0, smem_per_block = 0;
   } launch[2];
@@ -315,10 +315,15 @@ int validate_grid(const hx_grid* g) {
   return HX_OK;
 }
 
-// *long_call: whether a call may cost kLongCall us or more on some type.
+// *long_call: whether an attempt may take kLongCall us or more on some type.
 int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_prefill, int64_t max_decode,
                    bool* long_call) {
   bool is_long = false;
+  // fault windows stretch attempts (slow-down or timeout) and delay the rest
+  int64_t stretch = HX_SCALE;
+  for (int f = 0; f < c->n_faults; ++f)
+    stretch = std::max(stretch, std::max<int64_t>(c->faults[f].slow_fp, c->timeout_mult_fp));
+  const int64_t long_cost = (hx::kLongCall - 1) * HX_SCALE / stretch + 1;  // stretched, kLongCall or more
   const std::string where = "trace " + std::to_string(ti) + ": ";
   if (tr->n_queries < 0 || tr->n_calls < 0 || tr->n_calls >= (1 << 24))
     return fail(HX_ERR_INVALID, where + "n_queries/n_calls out of range");
@@ -372,18 +377,14 @@ int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_
       const int64_t dec = std::max(o, oe) * max_decode;
       if (dec >= kCostMax || p * 1000000 > (kCostMax - 1 - dec) * min_prefill)
         return fail(HX_ERR_INVALID, where + "a call's cost exceeds 2^28 us");
-      is_long |= dec >= hx::kLongCall || p * 1000000 > (hx::kLongCall - 1 - dec) * min_prefill;
+      is_long |= dec >= long_cost || p * 1000000 > (long_cost - 1 - dec) * min_prefill;
       tok_sum += p;
       dec_sum += dec;
     }
   }
   *long_call = is_long;
-  // fault windows stretch attempts (slow-down or timeout) and delay the rest
-  int64_t stretch = HX_SCALE, last = tr->n_queries > 0 ? tr->arrival_us[tr->n_queries - 1] : 0;
-  for (int f = 0; f < c->n_faults; ++f) {
-    stretch = std::max(stretch, std::max<int64_t>(c->faults[f].slow_fp, c->timeout_mult_fp));
-    last = std::max(last, c->faults[f].t1_us);
-  }
+  int64_t last = tr->n_queries > 0 ? tr->arrival_us[tr->n_queries - 1] : 0;
+  for (int f = 0; f < c->n_faults; ++f) last = std::max(last, c->faults[f].t1_us);
   const int64_t widen = 1 + (stretch + HX_SCALE - 1) / HX_SCALE, halve = c->n_faults > 0 ? 1 : 2;
   const __int128 tok_us = (__int128)tok_sum * 1000000;
   const int64_t lower = (int64_t)((tok_us + min_prefill - 1) / min_prefill) + dec_sum;

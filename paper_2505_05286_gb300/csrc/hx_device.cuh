@@ -71,7 +71,7 @@ struct ClusterK {
   uint8_t inst_type[HX_MAX_INST];
   uint8_t inst_slots[HX_MAX_INST];
   uint16_t slot_base[HX_MAX_INST];
-  // tenants and faults (only hx_sim_kernel_wide handles faults)
+  // tenants and faults (only the last two kernel families handle faults)
   int32_t n_tenants, n_faults;
   int64_t tenant_mult[HX_MAX_TENANTS];
   int64_t timeout_mult_fp;
@@ -138,13 +138,15 @@ struct SimArgs {
   int32_t checked;          // check the scheduler's invariants after every event (generic kernel)
 };
 
-// A running call in its batch slot: end time and request id << 8 | slot.
+// A running call in its batch slot: end time and request id << 8 | kFailBit if the
+// attempt times out at its end | slot.
+constexpr uint32_t kFailBit = 0x80;
 struct __align__(8) Slot32 {
   uint32_t end, tag;
 };
 struct __align__(16) Slot64 {
   uint64_t end;
-  uint32_t tag, fail;           // fail: the attempt times out at `end`
+  uint32_t tag, pad;
 };
 
 // One instance as every lane reads it (one 16-byte load).  Its t_queue and next
@@ -228,13 +230,14 @@ __global__ void hx_prep_kernel(PrepArgs a, ClusterK c);
 // The instantiations of the simulation kernel.  hx_sim_kernel_lean: every point
 // workload-balanced with the urgency queue, nothing logged; hx_sim_kernel_log:
 // with per-call logs; hx_sim_kernel: those and any mix of dispatch and
-// local-queue policies, tenants and event checks; hx_sim_kernel_wide: all of
-// it with fault windows or calls of kLongCall us and more (64-bit times).  Each for clusters of up to 64 instances, two a lane,
+// local-queue policies, tenants and event checks; hx_sim_kernel_faults: all of
+// it with fault windows; hx_sim_kernel_wide: all of it with attempts of kLongCall
+// us and more (64-bit times).  Each for clusters of up to 64 instances, two a lane,
 // and of up to 32, one a lane, and both for a full GPU and for a run of few
 // warps: kernel 4 * family + 2 * few + (one a lane).
-enum { kSimLean = 0, kSimLog = 1, kSimGeneric = 2, kSimWide = 3 };
+enum { kSimLean = 0, kSimLog = 1, kSimGeneric = 2, kSimFaults = 3, kSimWide = 4 };
 using SimKernel = void (*)(SimArgs, ClusterK);
-constexpr int kSimKernels = 16;
+constexpr int kSimKernels = 20;
 extern const SimKernel kSimKernel[kSimKernels];
 __global__ void hx_log_kernel(LogArgs a, ClusterK c);
 __global__ void hx_best_kernel(BestArgs a);

@@ -273,15 +273,13 @@ __global__ void __launch_bounds__(256) hx_prep_kernel(PrepArgs a, ClusterK c) {
 // -------------------------------------------------------- simulation kernel
 namespace {
 
-// Event times of one simulation are relative to a base.  While every call costs
-// less than 2^25 us on every type and there are no fault windows, they are
-// 32-bit, the base moves up every 2^25 us, and an instance's next completion is
+// Event times of one simulation are relative to a base.  While no attempt can take
+// 2^25 us (on any type, stretched by fault windows and timeouts), they are 32-bit, the base moves up every 2^25 us, and an instance's next completion is
 // time << 6 | instance: one 32-bit warp minimum gives the next event's time and
 // instance (a dispatch's least cost << 6 | instance likewise), without the ballot
 // and the bit search that lengthened the event's chain (8 x 2000 queries x 64
 // points 6.80 -> 6.29 ms, 8 x 20000 x 1024 on 64 instances 431 -> 399 ms).
-// Longer calls and fault windows, whose attempts can outlast that,
-// have 64-bit times, base 0.
+// Longer attempts have 64-bit times, base 0.
 template <bool kWide>
 struct Times {
   using T = uint32_t;
@@ -295,7 +293,8 @@ struct Times<true> {
 constexpr int kInstBits = 6;                          // of a key: HX_MAX_INST instances
 constexpr uint64_t kInstMask = (1 << kInstBits) - 1;
 
-// Running calls complete by (end, request id); a tag is request id << 8 | slot.
+// Running calls complete by (end, request id); a tag is request id << 8 |
+// kFailBit if the attempt times out | slot.
 __device__ __forceinline__ bool before(uint32_t e0, uint32_t tag0, uint32_t e1, uint32_t tag1) {
   return ((uint64_t)e0 << 32 | tag0) < ((uint64_t)e1 << 32 | tag1);
 }
@@ -672,7 +671,8 @@ __device__ __noinline__ unsigned lowest_id(uint32_t tag) {
 
 template <int J, int kFamily, bool kFew>
 __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
-  constexpr bool kLog = kFamily >= kSimLog, kGeneric = kFamily >= kSimGeneric, kWide = kFamily == kSimWide;
+  constexpr bool kLog = kFamily >= kSimLog, kGeneric = kFamily >= kSimGeneric;
+  constexpr bool kFaults = kFamily >= kSimFaults, kWide = kFamily == kSimWide;
   using T = typename Times<kWide>::T;
   using Slot = typename Times<kWide>::Slot;
   constexpr T kIdle = ~T(0);                        // no time
@@ -831,7 +831,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     T now = 0;
     int32_t status = HX_OK, npend = 0;
     // event bound; re-issued attempts add events while fault windows last
-    int32_t steps_left = nc + nq + 8 + (kWide ? 16 * nc + 4096 : 0);
+    int32_t steps_left = nc + nq + 8 + (kFaults ? 16 * nc + 4096 : 0);
 #ifdef HX_CHECKED
     // the warp's scratch slices must hold this trace's chain counters and top-K
     if (!(nq <= a.chains_per_warp && W->kcap <= a.topk_per_warp && (a.tenant_kcap == nullptr ||
@@ -865,13 +865,14 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     auto start_call = [&](int m, uint32_t free, uint32_t slot_base, int rid, int svc) -> uint32_t {
       T run = (T)svc;
       bool fail = false;
-      if (kWide) {
+      if (kFaults) {
         // the first fault window of m that covers now, and the timeout (Sec. 3.3)
+        const int64_t t_abs = absolute(now);
         int64_t r64 = svc;
         bool in_window = false, down = false;
         for (int f = 0; f < c.n_faults; ++f) {
           const FaultK& F = c.faults[f];
-          if (F.inst == m && (int64_t)now >= F.t0 && (int64_t)now < F.t1) {
+          if (F.inst == m && t_abs >= F.t0 && t_abs < F.t1) {
             in_window = true;
             if (F.slow == 0) down = true;
             else r64 = (r64 * F.slow + kScale - 1) / kScale;
@@ -888,13 +889,13 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         run = (T)r64;
       }
       const int s = 31 - __clz(free);
-      const uint32_t tag = (uint32_t)rid << 8 | (uint32_t)s;
+      const uint32_t tag = (uint32_t)rid << 8 | (kFaults && fail ? kFailBit : 0u) | (uint32_t)s;
       const T end = now + run, key = end << kInstBits | (T)m;
       if (lane == (m & 31)) {
         Slot e;
         e.end = end;
         e.tag = tag;
-        if constexpr (kWide) e.fail = fail ? 1u : 0u;
+        if constexpr (kWide) e.pad = 0;
         slots[slot_base + s] = e;
         if (kLog && recj >= 0) {
           a.rec_start[(int64_t)recj * a.rec_stride + rid] = absolute(now);
@@ -957,7 +958,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         HX_BOUND(m < N)
         const uint32_t tag = __shfl_sync(kFull, low ? next_tag[0] : next_tag[J - 1], m & 31);
         const int32_t rid = (int32_t)(tag >> 8);
-        const int hole = (int)(tag & 0xffu);
+        const int hole = (int)(tag & 15u);
         HX_BOUND(rid < nc)
         const CallRec* const r = rec + rid;
         const int4 tail = *reinterpret_cast<const int4*>(&r->tbar);
@@ -978,7 +979,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         if (kFew) load_costs(tail.y);
         // the slot is free; the next completion is the earliest of those still running
         const uint32_t free = I.free | 1u << (tag & 31u);
-        const bool failed = kWide && __any_sync(kFull, reinterpret_cast<const Slot64*>(slots)[slot_base + hole].fail != 0);
+        const bool failed = kFaults && (tag & kFailBit) != 0;
         const Slot e = slots[slot_base + l16];
         const bool runs = (I.cfg & ~free & lbit) != 0;
         const T nmin = warp_min(runs ? e.end : kIdle);
@@ -1015,7 +1016,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         rel_first = tail.y;
         rel_count = chain ? (int)last : (int)(tw & 0xff);
         if (chain) *chains = (uint8_t)ended;  // every lane writes the same byte
-        if (kWide && failed) {
+        if (kFaults && failed) {
           // the attempt timed out: the request goes out again, avoiding m
           const int32_t n = W->reissued + 1;
           __syncwarp();
@@ -1083,7 +1084,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
         if (kFew && rel_count > 1) load_costs(rid + 1);
         int m;
         // a re-issued request avoids the instance it timed out on
-        const int excl = kWide ? uniform(W->excl) : -1;
+        const int excl = kFaults ? uniform(W->excl) : -1;
         if (kGeneric && round_robin) {
           m = uniform(W->rr);
           if (m == excl) m = (m + 1 == N) ? 0 : m + 1;
@@ -1117,7 +1118,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
             }
           }
         }
-        if (kWide) W->excl = -1;
+        if (kFaults) W->excl = -1;
         HX_BOUND(m >= 0 && m < N)
         const bool low = J == 1 || m < 32;
         // the winner's costs, on its lane
@@ -1279,8 +1280,8 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     if (lane == 0) {
       int st = status;
       const int32_t n_done = W->n_done;
-      const int32_t steps0 = W->nc + nq + 8 + (kWide ? 16 * W->nc + 4096 : 0);
-      const int64_t events = (steps0 - steps_left) - W->arrivals - (kWide ? W->reissued : 0);
+      const int32_t steps0 = W->nc + nq + 8 + (kFaults ? 16 * W->nc + 4096 : 0);
+      const int64_t events = (steps0 - steps_left) - W->arrivals - (kFaults ? W->reissued : 0);
       // every query and every call completed exactly once
       if (st == HX_OK && (leftover || n_done != nq || events != W->nc)) st = HX_ERR_INVARIANT;
       hx_result res;
@@ -1321,12 +1322,14 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
 HX_SIM_KERNEL(hx_sim_kernel_lean, kSimLean)
 HX_SIM_KERNEL(hx_sim_kernel_log, kSimLog)
 HX_SIM_KERNEL(hx_sim_kernel, kSimGeneric)
+HX_SIM_KERNEL(hx_sim_kernel_faults, kSimFaults)
 HX_SIM_KERNEL(hx_sim_kernel_wide, kSimWide)
 #undef HX_SIM_KERNEL
 
 #define HX_FORMS(name) name<2, false>, name<1, false>, name<2, true>, name<1, true>
 const SimKernel kSimKernel[kSimKernels] = {HX_FORMS(hx_sim_kernel_lean), HX_FORMS(hx_sim_kernel_log),
-                                           HX_FORMS(hx_sim_kernel), HX_FORMS(hx_sim_kernel_wide)};
+                                           HX_FORMS(hx_sim_kernel), HX_FORMS(hx_sim_kernel_faults),
+                                           HX_FORMS(hx_sim_kernel_wide)};
 #undef HX_FORMS
 
 // ----------------------------------------------------------- log kernel

@@ -102,6 +102,28 @@ def test_calls_next_to_the_short_limit(n_inst):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("n_inst", [3, 40])
+@pytest.mark.parametrize("slow,timeout", [(2, 0), (2, 2), (0.5, 1), (0, 2), (100, 0)])
+def test_attempts_next_to_the_short_limit(n_inst, slow, timeout):
+    """Fault windows whose slow-down or timeout takes a call to 2^25 - 1, 2^25 and
+    past it: the same results with 32-bit and with 64-bit times."""
+    cl = _cluster(n_inst)
+    cl.prefill_tok_s[:] = 1_000_000
+    cl.decode_us_tok[:] = 32
+    cl.timeout_mult_fp = timeout * W.SCALE
+    cl.faults = np.zeros(2, W.FAULT_DTYPE)
+    cl.faults[0] = (0, 0, 0, 400_000_000, int(slow * W.SCALE))
+    cl.faults[1] = (n_inst - 1, 0, 100_000_000, 600_000_000, W.SCALE)
+    stretch = max(slow, timeout, 1)
+    for cost in (2 ** 25 // stretch - 1, 2 ** 25 // stretch, 2 ** 25 // stretch + 2):
+        tr = W.make_trace(W.RECIPES[1], 1, 21, n_queries=60)
+        tr.arrival_us = tr.arrival_us * 20
+        tr.out[::2] = tr.out_est[::2] = int(cost) // 32 - 1
+        tr.prompt[::2] = int(cost) - 32 * (int(cost) // 32 - 1)
+        _check(tr, cl, True, 1)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("generic", [False, True])
 @pytest.mark.parametrize("slots", [(1, 1, 1), (16, 16, 16), (2, 15, 16)])
 @pytest.mark.parametrize("n_inst", INST)
