@@ -9,6 +9,7 @@
 //                     event simulation of the workload-balanced dispatcher
 //                     (Sec. 4.1) and the urgency queues (Sec. 4.2), and
 //                     reduces it to P95 / SLO count / digest (Sec. 4.3).
+//   hx_log_kernel   : the SLO budgets (Sec. 4.2) of logged simulations' calls.
 //   hx_best_kernel  : argmin of the P95 objective per trace and over the grid.
 #pragma once
 
@@ -21,7 +22,7 @@ namespace hx {
 constexpr int64_t kScale = 1000000;       // fixed point of alpha, gamma, slo_mult
 constexpr int64_t kUsPerS = 1000000;      // prefill throughput is per second
 constexpr int64_t kRewardCap = (int64_t(1) << 43) - 1;
-constexpr int64_t kLongCall = int64_t(1) << 25;  // us; from here on event times are 64-bit
+constexpr int64_t kLongCall = int64_t(1) << 25;  // us; attempts this long need 64-bit event times
 constexpr int kWarpsPerBlock = 4;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kFRows = 18;                // S, G/C with 0..15 corrections done, E

@@ -1,10 +1,12 @@
-// hx_kernels.cu -- the three kernels of the batched HexGen-Flow scheduler
-// simulation (arXiv 2505.05286, Sec. 4.1-4.3) for sm_103a.
+// hx_kernels.cu -- the kernels of the batched HexGen-Flow scheduler simulation
+// (arXiv 2505.05286, Sec. 4.1-4.3) for sm_103a.
 //
-// Integer-only: every time is int64 microseconds, every score and key int64
-// fixed point; every division is the compiler's truncating `/`.  Nothing here
-// is a dense contraction, so there are no tensor-core paths; the simulation
-// kernel is bound by the SM issue rate, the preparation kernel by HBM.
+// Every result is integer arithmetic: times are int64 microseconds, scores and
+// keys int64 fixed point, divisions truncate.  Single precision only bounds a
+// score or estimates a quotient, and what it leaves open is decided exactly.
+// Nothing here is a dense contraction, so there are no tensor-core paths; the
+// simulation kernel is bound by its chain of dependent instructions and, on a
+// full GPU, by the integer pipe, the preparation kernel by HBM.
 #include <climits>
 
 #include "hx_device.cuh"
@@ -273,13 +275,15 @@ __global__ void __launch_bounds__(256) hx_prep_kernel(PrepArgs a, ClusterK c) {
 // -------------------------------------------------------- simulation kernel
 namespace {
 
-// Event times of one simulation are relative to a base.  While no attempt can take
-// 2^25 us (on any type, stretched by fault windows and timeouts), they are 32-bit, the base moves up every 2^25 us, and an instance's next completion is
+// Event times of one simulation are relative to a base.  While no attempt can
+// take 2^25 us (on any type, stretched by fault windows and timeouts), they are
+// 32-bit, the base moves up every 2^25 us, and an instance's next completion is
 // time << 6 | instance: one 32-bit warp minimum gives the next event's time and
 // instance (a dispatch's least cost << 6 | instance likewise), without the ballot
 // and the bit search that lengthened the event's chain (8 x 2000 queries x 64
-// points 6.80 -> 6.29 ms, 8 x 20000 x 1024 on 64 instances 431 -> 399 ms).
-// Longer attempts have 64-bit times, base 0.
+// points 6.80 -> 6.29 ms, 8 x 20000 x 1024 on 64 instances 431 -> 399 ms; fault
+// windows on 24 x 2000 x 64 15.5 -> 13.8 ms).  Longer attempts have 64-bit times,
+// base 0.
 template <bool kWide>
 struct Times {
   using T = uint32_t;
@@ -619,8 +623,9 @@ __device__ __forceinline__ void finish_query(WarpShared* W, int64_t now, int64_t
 // Resident blocks per SM the register allocation aims for (4 warps each): 8
 // with one instance per lane; with two, 7, whose 72 registers hold a
 // simulation's state without spills (8 spill 48 bytes in the event loop: 8
-// traces x 20000 queries x 1024 points 503 ms against 458 ms).  A run of few
-// warps takes what registers it likes.
+// traces x 20000 queries x 1024 points 503 ms against 458 ms).  The form for few
+// warps aims at 5 (96 registers, no spills: 64 x 3001 x 16 25.5 -> 23.5 ms; 4 or 6
+// blocks 1 to 4 % slower).
 #ifndef HX_SIM_MIN_BLOCKS
 #define HX_SIM_MIN_BLOCKS(J) ((J) == 1 ? 8 : 7)
 #endif
@@ -648,27 +653,28 @@ constexpr int kLongQueue = 128;  // entries (512: 27.0 ms)
 #define HX_STOP_IF_FAILED()
 #endif
 
-// One warp, one simulation.  J instances per lane: lane l owns l and, with J = 2,
-// l + 32.
-//
-// An event is a chain of dependent warp instructions, and their number bounds
-// both a lone simulation (5 to 7 cycles per instruction) and a full GPU (issue
-// slots 80 to 85 % busy).  So the state that only scores and the next event need
-// stays in the owner lane's registers, where an update is a select; event times
-// are 32-bit, so one warp reduction finds the next completion; running calls sit
-// unsorted in their slots under a free mask, so a start is one store and one
-// comparison, and a completion one reduction over the instance's slots; and up
-// to 32 instances take one lane each (half the per-lane work).  Against sorted
-// 64-bit slot keys and per-instance arrays in shared memory: 342 -> 178
-// warp-instructions per call event (8 traces x 2000 queries x 64 points, 8
-// instances: 14.2 -> 10.9 ms); 32 instances, 19 x 5003 x 512: 127 -> 89 ms; 64
-// instances, 8 x 20000 x 1024: 529 -> 460 ms.
 // The lane with the lowest tag (a call of its own: it is rare, and inlined it
 // would run predicated at every completion).
 __device__ __noinline__ unsigned lowest_id(uint32_t tag) {
   return __ballot_sync(kFull, tag == __reduce_min_sync(kFull, tag));
 }
 
+// One warp, one simulation.  J instances per lane: lane l owns l and, with J = 2,
+// l + 32.  kFew: the form for runs of few warps.
+//
+// An event is a chain of dependent warp instructions.  A lone simulation waits on
+// it (171 instructions, 820 cycles per call event with one instance per lane); a
+// full GPU, 7 or 8 warps per scheduler, spends 165 instructions, 1730 cycles per
+// event and warp, on its half-rate integer pipe (68 % busy) and issue slots (67 %).
+// So the state that only scores and the next event need stays in the owner lane's
+// registers, where an update is a select; event times are 32-bit, so one warp
+// reduction finds the next completion; running calls sit unsorted in their slots
+// under a free mask, so a start is one store and one comparison, and a completion
+// one reduction over the instance's slots; and up to 32 instances take one lane
+// each (half the per-lane work).  Against sorted 64-bit slot keys and per-instance
+// arrays in shared memory, when this layout came: 342 -> 178 instructions, 8 x 2000
+// queries x 64 points on 8 instances 14.2 -> 10.9 ms, 19 x 5003 x 512 on 32
+// instances 127 -> 89 ms, 8 x 20000 x 1024 on 64 instances 529 -> 460 ms.
 template <int J, int kFamily, bool kFew>
 __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
   constexpr bool kLog = kFamily >= kSimLog, kGeneric = kFamily >= kSimGeneric;
