@@ -187,13 +187,13 @@ struct __align__(16) WarpShared {
   int64_t sim, clk0;            // result index and start clock of the simulation
   int64_t base;                 // what the 32-bit event times are relative to (written alike by every lane)
   int64_t next_arrival;         // time of the next arrival (likewise)
-  int32_t arrivals, trace;      // arrivals taken so far (likewise); the simulation's trace
+  int32_t arrivals;             // arrivals taken so far (likewise)
   uint64_t digest;
   int64_t makespan;
   int32_t n_done, slo_met, sink, tk;  // sink: where prefetched records are copied to
   int64_t tkmin;                // root of the full top-K heap (written alike by every lane)
-  int32_t tslo[HX_MAX_TENANTS], tdone[HX_MAX_TENANTS];  // per-tenant counts (generic kernel)
-  int32_t ttk[HX_MAX_TENANTS];  // per-tenant top-K heaps: entries (generic kernel with tenants)
+  int2 tcount[HX_MAX_TENANTS];  // per tenant: completed queries, SLO hits (generic kernel)
+  int32_t tkcap[HX_MAX_TENANTS], ttk[HX_MAX_TENANTS];  // per-tenant top-K heaps: capacities, entries
   int64_t ttkmin[HX_MAX_TENANTS];  //                 and roots once full
   int32_t reissued, excl;       // timed-out attempts; the instance a re-issue avoids (-1: none)
 };
