@@ -157,8 +157,9 @@ struct __align__(16) InstState {
   int32_t hsize;                // local queue: heap size
   uint32_t heap;                // local queue: heap offset in the arena, capacity code << 27
                                 // (8 << code entries; 0: none yet)
-  uint32_t cfg;                 // its slots' mask, first slot << 16
+  uint32_t cfg;                 // its slots' mask, first slot << 16, kWindowsBit: it has fault windows
 };
+constexpr uint32_t kWindowsBit = 1u << 31;
 constexpr int kHeapCodeShift = 27;  // the arena holds at most 4 * 2^24 + 1024 entries
 constexpr uint32_t kHeapOffMask = (1u << kHeapCodeShift) - 1;
 

@@ -124,6 +124,21 @@ def test_attempts_next_to_the_short_limit(n_inst, slow, timeout):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("n_inst,on", [(1, [0]), (32, [31]), (32, list(range(16))), (33, [32]), (64, [0, 31, 32, 63]), (64, [])])
+def test_windows_of_some_instances(n_inst, on):
+    """Instances without fault windows beside ones that have some (at the edges of
+    a lane's first and second), and windows that no call meets."""
+    cl = _cluster(n_inst)
+    cl.timeout_mult_fp = 2 * W.SCALE
+    cl.faults = np.zeros(len(on) or 1, W.FAULT_DTYPE)
+    cl.faults[0] = (0, 0, 2 ** 37, 2 ** 38, W.SCALE)
+    for i, m in enumerate(on):
+        cl.faults[i] = (m, 0, 5_000_000 * i, 40_000_000 + 5_000_000 * i, (3 * W.SCALE, 0)[i % 2])
+    tr = W.make_trace(W.RECIPES[1], 1, 80 + n_inst, n_queries=120)
+    _check(tr, cl, True, 1)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("generic", [False, True])
 @pytest.mark.parametrize("slots", [(1, 1, 1), (16, 16, 16), (2, 15, 16)])
 @pytest.mark.parametrize("n_inst", INST)
