@@ -422,32 +422,39 @@ __device__ __forceinline__ HeapEnt heap_child(const HeapEnt* h, int i, int m, in
   return ent_load(h + child, child < m);
 }
 
-// All lanes call with the same arguments but c, their child of the root.  The
-// top entry has left the heap and `sink` takes its place, sinking to its level;
-// the heap then holds m entries (m = n - 1 and sink = the last entry: a pop;
-// m = n and sink = a new entry: a replace).
-__device__ __forceinline__ void heap_sift_warp(HeapEnt* h, int m, HeapEnt sink, HeapEnt c, int lane) {
+// One level of a sift: all lanes call with the same arguments but c, their child
+// of node i.  Unless `sink` goes before every child, the best one moves up to
+// node i, which becomes the node it came from, c its children there; else false.
+__device__ __forceinline__ bool heap_step(HeapEnt* h, int m, const HeapEnt& sink, int& i, HeapEnt& c, int lane) {
+  if (32 * i + 1 >= m) return false;
   const uint32_t sink_hi = (uint32_t)(sink.key >> 32);
-  int i = 0;
-  while (32 * i + 1 < m) {
-    // the first child by (key desc, rid asc): the keys' high words decide, the
-    // low words and the rids among equals only
-    const uint32_t hi = (uint32_t)(c.key >> 32);
-    const uint32_t mh = __reduce_max_sync(kFull, hi);
-    if (mh < sink_hi) break;
-    unsigned best = __ballot_sync(kFull, hi == mh);
-    if (((best & (best - 1)) != 0) | (mh == sink_hi)) {
-      const uint32_t lo = (uint32_t)c.key, ml = __reduce_max_sync(kFull, hi == mh ? lo : 0u);
-      best = __ballot_sync(kFull, (hi == mh) & (lo == ml));
-      const bool tie = (best >> lane) & 1u;
-      const uint32_t mr = __reduce_min_sync(kFull, tie ? (uint32_t)c.rid : 0xffffffffu);
-      best = __ballot_sync(kFull, tie & ((uint32_t)c.rid == mr));
-      if (__ballot_sync(kFull, ent_better(c, sink)) == 0) break;
-    }
-    const int b = 31 - __clz(best);
-    ent_store(h + i, c, lane == b);  // the best child moves up
-    i = 32 * i + 1 + b;
-    c = heap_child(h, i, m, lane);
+  // the first child by (key desc, rid asc): the keys' high words decide, the
+  // low words and the rids among equals only
+  const uint32_t hi = (uint32_t)(c.key >> 32);
+  const uint32_t mh = __reduce_max_sync(kFull, hi);
+  if (mh < sink_hi) return false;
+  unsigned best = __ballot_sync(kFull, hi == mh);
+  if (((best & (best - 1)) != 0) | (mh == sink_hi)) {
+    const uint32_t lo = (uint32_t)c.key, ml = __reduce_max_sync(kFull, hi == mh ? lo : 0u);
+    best = __ballot_sync(kFull, (hi == mh) & (lo == ml));
+    const bool tie = (best >> lane) & 1u;
+    const uint32_t mr = __reduce_min_sync(kFull, tie ? (uint32_t)c.rid : 0xffffffffu);
+    best = __ballot_sync(kFull, tie & ((uint32_t)c.rid == mr));
+    if (__ballot_sync(kFull, ent_better(c, sink)) == 0) return false;
+  }
+  const int b = 31 - __clz(best);
+  ent_store(h + i, c, lane == b);  // the best child moves up
+  i = 32 * i + 1 + b;
+  c = heap_child(h, i, m, lane);
+  return true;
+}
+
+// All lanes call with the same arguments but c, their child of node i, whose entry
+// has left.  `sink` takes its place, sinking to its level; the heap then holds m
+// entries (m = n - 1 and sink = the last entry: a pop; m = n and sink = a new
+// entry: a replace).
+__device__ __forceinline__ void heap_sift_warp(HeapEnt* h, int m, HeapEnt sink, int i, HeapEnt c, int lane) {
+  while (heap_step(h, m, sink, i, c, lane)) {
   }
   ent_store(h + i, sink, (lane == 0) & (m > 0));
   __syncwarp();
@@ -1198,18 +1205,34 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
             pm = __ballot_sync(kFull, pe.w == m);
             left &= ~pm;
           }
-          HeapEnt e;
+          // kEarly: where requests wait and one slot is free, the queue's top and its
+          // root's children are loaded before the new request's key is formed, and
+          // the first level of the sift is done before the start, so that the next
+          // level's load passes meanwhile (32 x 5000 queries x 256 points on 16
+          // instances 119.5 -> 116.1 ms, 19 x 5003 x 512 on 32 81.7 -> 79.4, a lone
+          // 3000 queries on 64 26.6 -> 25.95).  The other two forms lose more where
+          // no request waits: 8 x 2000 x 64 on 8 instances 6.24 -> 6.32, 8 x 20000 x
+          // 1024 on 64 378 -> 385.
+          constexpr bool kEarly = kFew == (J == 2);
+          const bool single = hs > 0 && m == cm && __popc(pm) < 2;
+          HeapEnt kid, top, e;
+          if (kEarly && single) {
+            kid = heap_child(h, 0, hs, lane);
+            top = ent_load(h);
+          }
           if (pm) {
             e.key = hs > 0 || __popc(pm) > __popc(free) ? queue_key(W, rec + pe.x, pe.z, absolute(now), lpol) : 0;
             e.rid = pe.x;
             e.svc = pe.y;
           }
-          if (hs > 0 && m == cm && __popc(pm) < 2) {
+          if (kEarly ? single : hs > 0 && m == cm && __popc(pm) < 2) {
+            if (!kEarly) {
+              kid = heap_child(h, 0, hs, lane);
+              top = ent_load(h);
+            }
             // requests wait, so this event freed m's only free slot.  It goes to
             // the queue's top, or to the new request if that is more urgent; the
             // queue's last entry or the new one sinks from the top.
-            HeapEnt kid = heap_child(h, 0, hs, lane);
-            const HeapEnt top = ent_load(h);
             int n = hs;
             bool fresh = false;
             if (pm) {
@@ -1226,8 +1249,15 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
             const int rid = fresh ? e.rid : top.rid, svc = fresh ? e.svc : top.svc;
             HX_BOUND(rid >= 0 && rid < nc)
             if (kFew && J == 2 && n >= kLongQueue) fetch_after(rid);
+            int at = 0;
+            bool more = false;
+            if (kEarly && !fresh) more = heap_step(h, n, e, at, kid, lane);
             start_call(m, free, slot_base, windows_on(I), rid, svc);
-            if (!fresh) heap_sift_warp(h, n, e, kid, lane);
+            if (!fresh) {
+              if (!kEarly || more) while (heap_step(h, n, e, at, kid, lane)) {}
+              ent_store(h + at, e, (lane == 0) & (n > 0));
+              __syncwarp();
+            }
           } else {
             const bool direct = hs == 0 && __popc(pm) <= __popc(free);
             int n = 0;
@@ -1251,7 +1281,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
                 rid = top.rid;
                 svc = top.svc;
                 inst[m].hsize = n;  // every lane writes the same size
-                heap_sift_warp(h, n, last, heap_child(h, 0, n, lane), lane);
+                heap_sift_warp(h, n, last, 0, heap_child(h, 0, n, lane), lane);
               }
               HX_BOUND(rid >= 0 && rid < nc)
               free = start_call(m, free, slot_base, windows_on(I), rid, svc);

@@ -71,6 +71,26 @@ def test_queue_sizes(n_inst, slots, n, equal, generic):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("equal", [False, True])
+@pytest.mark.parametrize("n", [1, 2, 16, 31, 32, 33, 34, 1057, 1058])
+@pytest.mark.parametrize("n_inst", [1, 33])
+def test_queue_sizes_on_a_full_gpu(n_inst, n, equal):
+    """The same with more than 20 warps per SM: every copy of a trace as the oracle."""
+    B.build()
+    cl = W.make_cluster(W.RECIPES[1])
+    cl.inst_type = np.zeros(n_inst, np.uint8)
+    cl.slots = np.array([1] * 3, np.int32)
+    tr, grid, copies = _burst(n, equal, n), _grid([0]), 1600
+    sim = H.Sim([tr] * copies, cl, grid)
+    sim.run()
+    got, want = sim.results(), oracle.run(W.Workload("queue", [tr], cl, grid, W.OBJ_P95))
+    assert sim.info()["resident_warps"] > 20 * 152
+    sim.close()
+    for f in FIELDS:
+        assert np.array_equal(got[f].reshape(copies, 2), np.tile(np.asarray(want[f]).reshape(1, 2), (copies, 1))), f
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("kind", ["lean", "policies", "tenants", "faults"])
 @pytest.mark.parametrize("n_inst", [8, 40])
 def test_logged_budgets(n_inst, kind):
