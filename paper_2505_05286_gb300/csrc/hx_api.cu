@@ -195,6 +195,7 @@ struct hx_sim {
     int family = hx::kSimWide, kernel = 0, blocks = 0, smem_per_block = 0;
   } launch[2];
   bool long_calls = false;
+  int32_t* d_long = nullptr;    // the same on the device, for captured runs
   const Launch& shape() const { return launch[long_calls ? 1 : 0]; }
   int64_t scratch_bytes = 0, device_bytes = 0;
   cudaStream_t last_stream = nullptr;
@@ -543,6 +544,22 @@ int launch_shape(int family, const hx::ClusterK& ck, const cudaDeviceProp& prop,
   return HX_OK;
 }
 
+// Whether s is being captured (if that cannot be told, the launches say so).
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cap != cudaStreamCaptureStatusNone;
+}
+
+// Gives the simulation kernel that follows all of the work, or none of it.
+__global__ void hx_gate_kernel(const int32_t* long_calls, int32_t want, unsigned long long n_work,
+                               unsigned long long* work_counter) {
+  *work_counter = (*long_calls != 0) == (want != 0) ? 0ull : n_work;
+}
+
 int launch_sim(const hx_sim::Launch& l, const hx::SimArgs& sa, hx::ClusterK ck, cudaStream_t s) {
   ck.smem_per_warp = l.smem_per_block / hx::kWarpsPerBlock;
   if (int rc = ensure_dyn_smem(l.kernel, l.smem_per_block)) return rc;
@@ -732,6 +749,7 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   h->place(&h->d_k, h->n_q);
   h->place(&h->d_tenant, h->n_q);
   if (tenants) h->place(&h->d_tenant_kcap, (int64_t)n_traces * HX_MAX_TENANTS);
+  h->place(&h->d_long, 1);
   h->query_bytes = h->device_bytes;
   h->place(&h->d_q_off, n_traces + 1);
   h->place(&h->d_c_off, n_traces + 1);
@@ -754,6 +772,7 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   // staged() needs the offsets only: the block is allocated when its size is known
   for (const auto& p : h->placed) *p.first = h->block + p.second;
   if ((rc = validate(&long_calls, [&](int32_t i) { pack_trace(h, traces[i], i); }))) return bail(rc);
+  *h->staged(h->d_long) = long_calls;
   if (opt && opt->n_record < 0) return bail(fail(HX_ERR_INVALID, "n_record < 0"));
   if (opt && opt->n_record > 0) {
     if (!opt->record_sims) return bail(fail(HX_ERR_INVALID, "record_sims is NULL"));
@@ -891,6 +910,7 @@ static int hx_sim_upload_impl(hx_sim* h, const hx_trace* traces, int32_t n_trace
   // set first: a copy that fails half-way may leave long calls behind
   const bool had_long = h->long_calls;
   h->long_calls = had_long || long_calls;
+  *h->staged(h->d_long) = long_calls;
   if ((rc = upload_inputs(h, traces, h->keep_stage() ? h->input_bytes : h->query_bytes,
                           static_cast<cudaStream_t>(stream))))
     return rc;
@@ -975,7 +995,17 @@ static int hx_sim_run_impl(hx_sim* h, void* stream) {
   hx::hx_prep_kernel<<<prep_blocks, 256, 0, s>>>(pa, h->ck);
   HX_CUDA(cudaGetLastError());
   if (ev) HX_CUDA(cudaEventRecord(ev[1], s));
-  if (int rc = launch_sim(h->shape(), sa, h->ck, s)) return rc;
+  if (capturing(s)) {
+    // traces uploaded before a replay may need the other family: both are
+    // captured, and the one that does not serve them finds no work left
+    for (int f = 0; f < 2; ++f) {
+      hx_gate_kernel<<<1, 1, 0, s>>>(h->d_long, f, (unsigned long long)h->n_work, h->d_counter);
+      HX_CUDA(cudaGetLastError());
+      if (int rc = launch_sim(h->launch[f], sa, h->ck, s)) return rc;
+    }
+  } else if (int rc = launch_sim(h->shape(), sa, h->ck, s)) {
+    return rc;
+  }
   if (h->n_record > 0) {
     hx::LogArgs la;
     la.rec = h->d_rec;

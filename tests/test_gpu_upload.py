@@ -45,3 +45,38 @@ def test_upload_replaces_every_input(n, nq, tenants):
         if tenants:
             assert np.array_equal(sim.extras()[sims]["p95_us"], extra["p95_us"])
     sim.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("force_generic", [False, True])
+@pytest.mark.parametrize("record", [(), (1,)])
+def test_captured_run_follows_uploads(force_generic, record):
+    """A captured run serves whatever traces are uploaded before a replay, also ones
+    whose calls need 64-bit times where those at the capture did not, and back."""
+    import torch
+    B.build()
+    recipe = W.RECIPES[1]
+    a, cl = _traces(recipe, 2, 60, 1)
+    b, _ = _traces(recipe, 2, 60, 2)
+    b[1].prompt[::3] = 1_000_000  # past 2^25 us on the slower types
+    grid = W.subset_grid(W.make_grid(recipe), [0, 40, 63])
+    for first, second in ((a, b), (b, a)):
+        sim = H.Sim(first, cl, grid, record_sims=record, force_generic=force_generic)
+        sim.run()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            sim.run(torch.cuda.current_stream())
+        for traces in (first, second, first):
+            sim.upload(traces)
+            graph.replay()
+            torch.cuda.synchronize()
+            got, wl = sim.results(), W.Workload("captured", traces, cl, grid, 0)
+            want = oracle.run(wl)
+            for f in FIELDS:
+                assert np.array_equal(got[f], want[f]), f
+            for j, s in enumerate(record):
+                _, log = oracle.simulate(traces[s // 3], cl, oracle.point_of(grid, s % 3), log=True)
+                for f in ("budget", "start", "end"):
+                    assert np.array_equal(sim.records(j)[f], log[f]), f
+        sim.close()
