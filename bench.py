@@ -43,7 +43,10 @@ L2_BYTES = 129 * 2 ** 20
 SM_COUNT_FALLBACK = 152
 
 
-WARP_INST_PER_EVENT = 300
+# Unit of work of the roofline: about what one simulated call event takes on up
+# to 32 instances (counted with ncu: 178 on 8 with few warps, 169 on 32 with a
+# full GPU).  More instances, long queues and the other families execute more.
+WARP_INST_PER_EVENT = 180
 KERNEL_SRC = os.path.join(ROOT, "paper_2505_05286_gb300", "csrc", "hx_kernels.cu")
 # ncu figures of the simulation kernel, each file keyed to the kernel source's
 # SHA-256: DRAM traffic of one full ceiling launch (a one-pass capture of the
@@ -461,10 +464,10 @@ def run_gpu(args):
     peaks, peak_kind = _peaks()
     clocks = clk.summary()
     # Roofline of the dominant kernel (the simulation kernel): the SM issue
-    # rate.  Algorithmic work per simulated call event: ~300 warp-instructions
-    # (N = 64 instances over 32 lanes, one int64 division, score, argmax,
-    # next-event minimum, queue and bookkeeping); peak: every scheduler of
-    # every SM issuing one warp-instruction per cycle at the maximum SM clock.
+    # rate.  Work per simulated call event: ~180 warp-instructions (next-event
+    # minimum, score and argmax over the lanes' instances, queue costs, starts
+    # and bookkeeping); peak: every scheduler of every SM issuing one
+    # warp-instruction per cycle at the maximum SM clock.
     sm_count = torch.cuda.get_device_properties(0).multi_processor_count
     sm_mhz = float(peaks.get("sm_max_mhz", 2070.0))
     peak = sm_count * 4 * sm_mhz * 1e6
