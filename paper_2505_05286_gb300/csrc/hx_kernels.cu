@@ -706,6 +706,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     W->chains = a.chains + gw * a.chains_per_warp;
     W->topk = a.topk + gw * a.topk_per_warp;
   }
+  __syncwarp();  // every lane clears its part of W->chains before a simulation's first barrier
   const int N = c.n_inst;
   // an instance's slots are read one per lane of the lower half warp
   const int l16 = lane & 15;
