@@ -1358,6 +1358,8 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
     }
     __syncwarp();
   }
+  // the last prefetches' copies land before the block's shared memory is given back
+  if (kFew) asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 #define HX_SIM_KERNEL(name, family)                                                                   \

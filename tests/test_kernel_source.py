@@ -19,3 +19,10 @@ def test_scratch_slices_reach_every_lane_before_their_first_use():
     other lane reads one."""
     after = _sim_body().split("W->topk = a.topk + gw * a.topk_per_warp;")[1]
     assert "__syncwarp();" in after[:re.search(r"W->(arena|chains|topk)\b", after).start()]
+
+
+def test_prefetches_end_before_the_kernel_does():
+    """cp.async copies that nobody reads are waited for before the block exits."""
+    body = _sim_body()
+    assert "cp.async.ca" in body
+    assert "cp.async.wait_all;" in body[body.rindex("__syncwarp();"):]
