@@ -830,7 +830,9 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   // heap arena: doubling regions of 16, 32, ... entries per instance total at
   // most 4 * (requests ever queued) + 16 * instances
   h->arena_per_warp = 4 * (int64_t)h->max_nc + 16 * HX_MAX_INST;
-  if (opt && opt->arena_entries > 0) h->arena_per_warp = opt->arena_entries;
+  // (no more than a queue's offset can reach: a queue past it is HX_ERR_CAPACITY)
+  if (opt && opt->arena_entries > 0)
+    h->arena_per_warp = std::min<int64_t>(opt->arena_entries, int64_t(hx::kHeapOffMask) + 1);
   h->chains_per_warp = align_up(std::max(h->max_nq, 1), 256);
   h->topk_per_warp = align_up(h->max_kcap, 32);
   if (tenants) {
