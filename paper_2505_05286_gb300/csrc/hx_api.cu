@@ -316,6 +316,12 @@ int validate_grid(const hx_grid* g) {
   return HX_OK;
 }
 
+// Counts that no valid trace has (a query has at least one call): nothing may be
+// read or sized by them.
+bool bad_counts(const hx_trace& tr) {
+  return tr.n_queries < 0 || tr.n_calls < 0 || tr.n_calls >= (1 << 24) || tr.n_queries > tr.n_calls;
+}
+
 // *long_call: whether an attempt may take kLongCall us or more on some type.
 int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_prefill, int64_t max_decode,
                    bool* long_call) {
@@ -326,8 +332,7 @@ int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_
     stretch = std::max(stretch, std::max<int64_t>(c->faults[f].slow_fp, c->timeout_mult_fp));
   const int64_t long_cost = (hx::kLongCall - 1) * HX_SCALE / stretch + 1;  // stretched, kLongCall or more
   const std::string where = "trace " + std::to_string(ti) + ": ";
-  if (tr->n_queries < 0 || tr->n_calls < 0 || tr->n_calls >= (1 << 24))
-    return fail(HX_ERR_INVALID, where + "n_queries/n_calls out of range");
+  if (bad_counts(*tr)) return fail(HX_ERR_INVALID, where + "n_queries/n_calls out of range");
   if (tr->n_queries > 0 && (!tr->arrival_us || !tr->k || !tr->prompt || !tr->out || !tr->out_est || !tr->stage ||
                             !tr->cand || !tr->retry))
     return fail(HX_ERR_INVALID, where + "array is NULL");
@@ -704,12 +709,12 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
     return validate_traces(traces, n_traces, cluster, min_prefill, max_decode, long_calls, pack);
   };
   int64_t n_calls = 0;
-  bool bad_counts = false, long_calls = false;
+  bool refuse = false, long_calls = false;
   for (int32_t i = 0; i < n_traces; ++i) {
-    bad_counts |= traces[i].n_queries < 0 || traces[i].n_calls < 0 || traces[i].n_calls >= (1 << 24);
+    refuse |= bad_counts(traces[i]);
     n_calls += traces[i].n_calls;
   }
-  if (bad_counts || n_calls >= (int64_t(1) << 31)) {
+  if (refuse || n_calls >= (int64_t(1) << 31)) {
     if ((rc = validate(&long_calls, [](int32_t) {}))) return rc;
     return fail(HX_ERR_INVALID, "more than 2^31 calls in total");
   }

@@ -229,6 +229,23 @@ def test_rejects_bad_options(lib):
         assert not h.value
 
 
+def test_rejects_more_queries_than_calls_before_sizing_anything(lib):
+    """Every query has at least one call.  Counts that say otherwise are refused as
+    they are, without a look at arrays of that length or memory for them (here
+    1.5 TB of staged queries, which would be HX_ERR_OOM)."""
+    wl = W.make_workload(0, n_queries=20)
+    tr = H._Traces([wl.traces[0]] * 40)
+    for t in tr.arr:
+        t.n_queries = 2 ** 31 - 1
+    hc, keep_c = H._cluster_struct(wl.cluster)
+    hg, keep_g = H._grid_struct(wl.grid)
+    h = ctypes.c_void_p()
+    rc = lib.hx_sim_create(tr.arr, 40, ctypes.byref(hc), ctypes.byref(hg), None, ctypes.byref(h))
+    err = lib.hx_last_error().decode()
+    assert rc == H.HX_ERR_INVALID and err.startswith("trace 0: n_queries"), (rc, err)
+    assert not h.value
+
+
 def test_null_safety(lib):
     assert lib.hx_sim_destroy(None) == H.HX_OK
     assert lib.hx_sim_run(None, None) == H.HX_ERR_INVALID
