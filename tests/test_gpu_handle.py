@@ -1,4 +1,7 @@
 """What a handle reserves on the device and the host, and which kernels it runs."""
+import ctypes
+import time
+
 import numpy as np
 import pytest
 
@@ -30,3 +33,52 @@ def test_arena_holds_no_more_than_a_queue_offset_reaches():
         for f in FIELDS:
             assert np.array_equal(got[f], want[f]), f
     assert scratch[0] == scratch[1] > 4 * 16 * 2 ** 27
+
+
+def _logged(queries):
+    """A run of two traces of these queries and of half as many with every call of both logged."""
+    wl = W.make_workload(4, n_traces=1, n_queries=queries)
+    wl.traces.append(W.make_workload(4, n_traces=2, n_queries=queries // 2).traces[1])
+    wl.grid = W.subset_grid(wl.grid, [0])
+    sim = H.Sim(wl.traces, wl.cluster, wl.grid, record_sims=[1, 0])
+    sim.run()
+    return wl, sim
+
+
+@pytest.mark.parametrize("queries", [40, 380, 420, 1580, 1620, 5000])  # 300 to 38000 calls
+def test_records_by_column(queries):
+    """Any choice of the log's columns, read in one copy (short logs) or by column."""
+    wl, sim = _logged(queries)
+    names = ("inst", "enq", "budget", "start", "end")
+    for j, t in enumerate((1, 0)):
+        _, want = oracle.simulate(wl.traces[t], wl.cluster, oracle.point_of(wl.grid, 0), log=True)
+        n = len(wl.traces[t].prompt)
+        for pick in (names, ("end",), ("inst",), ("enq", "budget"), ("inst", "start", "end")):
+            out = {f: np.full(n, -7, np.int32 if f == "inst" else np.int64) for f in names}
+            assert sim.lib.hx_sim_records(sim.h, j, *[H._p(out[f]) if f in pick else None for f in names], n) == H.HX_OK
+            for f in names:
+                assert np.array_equal(out[f], want[f]) if f in pick else (out[f] == -7).all(), (pick, f)
+    sim.close()
+
+
+def test_one_column_of_a_long_log_costs_one_copy():
+    """Reading one column of 150k calls takes about as long as a copy of its bytes
+    (five times that when the whole log went through a buffer)."""
+    import torch
+    wl, sim = _logged(20000)
+    n = len(wl.traces[0].prompt)
+    host, dev = torch.zeros(n, dtype=torch.int64), torch.zeros(n, dtype=torch.int64, device="cuda")
+    at = ctypes.c_void_p(host.data_ptr())
+
+    def median_us(read):
+        t = []
+        for _ in range(41):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            read()
+            t.append(1e6 * (time.perf_counter() - t0))
+        return sorted(t)[20]
+    column = median_us(lambda: sim.lib.hx_sim_records(sim.h, 1, None, None, None, None, at, n))
+    copy = median_us(lambda: host.copy_(dev))
+    sim.close()
+    assert column < 2.5 * copy + 10, (column, copy)
