@@ -214,12 +214,12 @@ struct hx_sim {
   std::vector<std::pair<void**, int64_t>> placed;
   // The inputs lead it: the per-query arrays, the constants of cluster and grid and
   // the per-call arrays.  `stage` is the same on the host, so that an upload is one
-  // copy (64 traces' 384 copies took 2.5 ms); more than kStageMost bytes of inputs
-  // keep no stage, and their per-call arrays are copied from the caller's.
-  static constexpr int64_t kStageMost = int64_t(64) << 20;
+  // copy (64 traces' 384 copies took 2.5 ms).  The per-call arrays are staged while
+  // that is cheaper than six copies a trace from the caller's (see stage_calls_of);
+  // otherwise they are copied from there and no stage is kept.
   std::unique_ptr<unsigned char[]> stage;
   int64_t query_bytes = 0, const_bytes = 0, input_bytes = 0;  // ends of the three parts
-  bool keep_stage() const { return input_bytes <= kStageMost; }
+  bool stage_calls = false;
 
   template <class T>
   void place(T** p, int64_t count) {
@@ -407,14 +407,30 @@ int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_
   return HX_OK;
 }
 
-// fn(t) for t = 0 .. n_traces - 1 on up to 16 host threads, one trace at a
-// time each, when the traces hold enough calls to pay for the threads.
+// Host threads that work on so many traces and calls: up to 16, when the calls pay
+// for them.
+int host_threads(int32_t n_traces, int64_t calls) {
+  const int64_t hw = std::max<int64_t>(1, std::thread::hardware_concurrency());
+  return (int)std::min<int64_t>({16, hw, (int64_t)n_traces, calls / 200000 + 1});
+}
+
+// Whether to stage the per-call arrays of so many traces: up to 64 MiB of inputs,
+// and 1.25 MiB a trace for every thread that stages them.  A thread stages about 19
+// GB/s and a trace's own six copies cost about 66 us, their bytes next to nothing:
+// one trace of 45k calls uploads in 0.25 ms staged and 0.28 not, one of 151k in 0.72
+// and 0.67, one of 756k in 3.3 and 3.0; four of 151k (four threads) in 0.95 and
+// 1.05, 64 of 23k in 2.4 and 4.9.
+constexpr int64_t kStageMost = int64_t(64) << 20, kStagePerThread = int64_t(1280) << 10;
+bool stage_calls_of(int32_t n_traces, int64_t calls, int64_t input_bytes, int64_t call_bytes) {
+  return input_bytes <= kStageMost && call_bytes <= kStagePerThread * n_traces * host_threads(n_traces, calls);
+}
+
+// fn(t) for t = 0 .. n_traces - 1 on host_threads(), one trace at a time each.
 template <class F>
 void for_each_trace(const hx_trace* traces, int32_t n_traces, F fn) {
   int64_t calls = 0;
   for (int32_t t = 0; t < n_traces; ++t) calls += traces[t].n_calls;
-  const int64_t hw = std::max<int64_t>(1, std::thread::hardware_concurrency());
-  const int nt = (int)std::min<int64_t>({16, hw, (int64_t)n_traces, calls / 200000 + 1});
+  const int nt = host_threads(n_traces, calls);
   if (nt <= 1) {
     for (int32_t t = 0; t < n_traces; ++t) fn(t);
     return;
@@ -494,7 +510,7 @@ void pack_trace(hx_sim* h, const hx_trace& tr, int32_t t) {
     int32_t* const kcap = h->staged(h->d_tenant_kcap) + (int64_t)t * HX_MAX_TENANTS;
     for (int u = 0; u < HX_MAX_TENANTS; ++u) kcap[u] = n[u] ? n[u] - (95 * n[u] + 99) / 100 + 1 : 0;
   }
-  if (h->keep_stage() && nc > 0) {
+  if (h->stage_calls && nc > 0) {
     std::memcpy(h->staged(h->d_prompt) + co, tr.prompt, (size_t)nc * sizeof(int32_t));
     std::memcpy(h->staged(h->d_out) + co, tr.out, (size_t)nc * sizeof(int32_t));
     std::memcpy(h->staged(h->d_out_est) + co, tr.out_est, (size_t)nc * sizeof(int32_t));
@@ -509,7 +525,7 @@ void pack_trace(hx_sim* h, const hx_trace& tr, int32_t t) {
 int upload_inputs(hx_sim* h, const hx_trace* traces, int64_t bytes, cudaStream_t s) {
   int rc;
   if ((rc = upload(h->block, h->stage.get(), bytes, s))) return rc;
-  for (int t = 0; t < h->n_traces && !h->keep_stage(); ++t) {
+  for (int t = 0; t < h->n_traces && !h->stage_calls; ++t) {
     const hx_trace& tr = traces[t];
     const int64_t co = h->c_off[t];
     if ((rc = upload(h->d_prompt + co, tr.prompt, tr.n_calls, s)) || (rc = upload(h->d_out + co, tr.out, tr.n_calls, s)) ||
@@ -519,7 +535,7 @@ int upload_inputs(hx_sim* h, const hx_trace* traces, int64_t bytes, cudaStream_t
       return rc;
   }
   HX_CUDA(cudaStreamSynchronize(s));
-  if (!h->keep_stage()) h->stage.reset();
+  if (!h->stage_calls) h->stage.reset();
   return HX_OK;
 }
 
@@ -772,7 +788,8 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   h->place(&h->d_cand, h->n_c);
   h->place(&h->d_retry, h->n_c);
   h->input_bytes = h->device_bytes;
-  const int64_t staged_bytes = h->keep_stage() ? h->input_bytes : h->const_bytes;
+  h->stage_calls = stage_calls_of(n_traces, h->n_c, h->input_bytes, h->input_bytes - h->const_bytes);
+  const int64_t staged_bytes = h->stage_calls ? h->input_bytes : h->const_bytes;
   h->stage.reset(new unsigned char[(size_t)staged_bytes]);
   // staged() needs the offsets only: the block is allocated when its size is known
   for (const auto& p : h->placed) *p.first = h->block + p.second;
@@ -918,7 +935,7 @@ static int hx_sim_upload_impl(hx_sim* h, const hx_trace* traces, int32_t n_trace
   const bool had_long = h->long_calls;
   h->long_calls = had_long || long_calls;
   *h->staged(h->d_long) = long_calls;
-  if ((rc = upload_inputs(h, traces, h->keep_stage() ? h->input_bytes : h->query_bytes,
+  if ((rc = upload_inputs(h, traces, h->stage_calls ? h->input_bytes : h->query_bytes,
                           static_cast<cudaStream_t>(stream))))
     return rc;
   h->long_calls = long_calls;

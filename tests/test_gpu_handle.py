@@ -82,3 +82,37 @@ def test_one_column_of_a_long_log_costs_one_copy():
     copy = median_us(lambda: host.copy_(dev))
     sim.close()
     assert column < 2.5 * copy + 10, (column, copy)
+
+
+class _MallInfo(ctypes.Structure):
+    _fields_ = [(f, ctypes.c_size_t) for f in ("arena", "ordblks", "smblks", "hblks", "hblkhd", "usmblks", "fsmblks",
+                                               "uordblks", "fordblks", "keepcost")]
+
+
+def _host_bytes():
+    """Bytes that malloc has handed out (main arena and mapped blocks)."""
+    info = ctypes.CDLL(None).mallinfo2
+    info.restype = _MallInfo
+    m = info()
+    return m.uordblks + m.hblkhd
+
+
+@pytest.mark.parametrize("n,queries,staged", [(1, 11000, True), (1, 12000, False), (2, 30000, False), (8, 20000, True)])
+def test_calls_are_staged_where_that_is_cheaper(n, queries, staged):
+    """A handle keeps a host copy of its calls only where one copy of it is cheaper
+    than copies of every trace's arrays: not for a few large traces."""
+    wl = W.make_workload(1, n_traces=n, n_queries=queries)
+    wl.grid = W.subset_grid(wl.grid, [5])
+    H.Sim(wl.traces, wl.cluster, wl.grid, max_resident_warps=4).close()
+    before = _host_bytes()
+    sim = H.Sim(wl.traces, wl.cluster, wl.grid, max_resident_warps=4)
+    kept = _host_bytes() - before
+    per_call = 15 * sum(len(t.prompt) for t in wl.traces)
+    assert (kept > per_call) == staged, (kept, per_call)
+    for step in range(2):  # a new handle's inputs, and an upload's
+        sim.run()
+        got, want = sim.results(), oracle.run(wl)
+        for f in FIELDS:
+            assert np.array_equal(got[f], want[f]), f
+        sim.upload(wl.traces)
+    sim.close()
