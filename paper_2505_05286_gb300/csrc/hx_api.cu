@@ -325,7 +325,6 @@ bool bad_counts(const hx_trace& tr) {
 // *long_call: whether an attempt may take kLongCall us or more on some type.
 int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_prefill, int64_t max_decode,
                    bool* long_call) {
-  bool is_long = false;
   // fault windows stretch attempts (slow-down or timeout) and delay the rest
   int64_t stretch = HX_SCALE;
   for (int f = 0; f < c->n_faults; ++f)
@@ -343,7 +342,7 @@ int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_
   // ceil(prompt * 10^6 / min_prefill) + max(out, out_est) * max_decode;
   // summed here as sum(prompt) and sum(decode part), the sum of the ceilings
   // lying within n_calls above the ceiling of the sum
-  int64_t tok_sum = 0, dec_sum = 0;
+  int64_t tok_sum = 0, dec_sum = 0, most = 0;
   for (int32_t i = 0; i < tr->n_queries; ++i) {
     if (tr->arrival_us[i] < 0 || (i > 0 && tr->arrival_us[i] < tr->arrival_us[i - 1]))
       return fail(HX_ERR_INVALID, where + "arrivals must be non-negative and sorted");
@@ -379,16 +378,18 @@ int validate_trace(const hx_trace* tr, int ti, const hx_cluster* c, int64_t min_
       if (p < 1 || p > kTokMax || o < 0 || o > kTokMax || oe < 0 || oe > kTokMax)
         return fail(HX_ERR_INVALID, where + "token counts out of range");
       // ceil(p * 10^6 / min_prefill) + dec >= 2^28, decided without a division:
-      // ceil(x / d) >= m exactly when x > (m - 1) * d
-      const int64_t dec = std::max(o, oe) * max_decode;
-      if (dec >= kCostMax || p * 1000000 > (kCostMax - 1 - dec) * min_prefill)
+      // ceil(x / d) + y >= m exactly when x + y * d > (m - 1) * d (below 2^60 here);
+      // whether the longest call is a long one, likewise, once for the trace (per call
+      // it was a tenth of the time that a trace of 756k calls takes to upload)
+      const int64_t dec = std::max(o, oe) * max_decode, scaled = p * 1000000 + dec * min_prefill;
+      if (dec >= kCostMax || scaled > (kCostMax - 1) * min_prefill)
         return fail(HX_ERR_INVALID, where + "a call's cost exceeds 2^28 us");
-      is_long |= dec >= long_cost || p * 1000000 > (long_cost - 1 - dec) * min_prefill;
+      most = std::max(most, scaled);
       tok_sum += p;
       dec_sum += dec;
     }
   }
-  *long_call = is_long;
+  *long_call = most > (long_cost - 1) * min_prefill;
   int64_t last = tr->n_queries > 0 ? tr->arrival_us[tr->n_queries - 1] : 0;
   for (int f = 0; f < c->n_faults; ++f) last = std::max(last, c->faults[f].t1_us);
   const int64_t widen = 1 + (stretch + HX_SCALE - 1) / HX_SCALE, halve = c->n_faults > 0 ? 1 : 2;

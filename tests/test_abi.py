@@ -181,6 +181,34 @@ def test_parallel_validation_names_the_first_bad_trace(lib):
     assert rc == H.HX_ERR_INVALID and err.startswith("trace 5:") and "token" in err, err
 
 
+@pytest.mark.parametrize("prefill", [1, 7, 999_983, 1_000_000, 2 ** 31 - 1])
+@pytest.mark.parametrize("decode", [0, 1, 255, 4099, 2 ** 31 - 1])
+def test_call_cost_limit_is_exact(lib, prefill, decode):
+    """ceil(prompt * 10^6 / prefill) + max(out, out_est) * decode: below 2^28 us, at
+    the extremes of the rates too."""
+    wl = W.make_workload(0, n_queries=1)
+    cl = wl.cluster
+    cl.prefill_tok_s[:], cl.decode_us_tok[:] = prefill, decode
+    cl.stage_ref_prompt[:], cl.stage_ref_out[:] = 1, 0
+    top = 2 ** 28 - 1
+    rng = np.random.default_rng(prefill + decode)
+    for _ in range(12):
+        t = _copy_trace(wl.traces[0])
+        t.prompt[:], t.out[:], t.out_est[:] = 1, 0, 0
+        out = int(rng.integers(0, min(2 ** 20, top // decode if decode else 2 ** 20) + 1))
+        for p in {1, 2 ** 20, max(1, (top - out * decode) * prefill // 10 ** 6) + int(rng.integers(0, 2))}:
+            if p > 2 ** 20:
+                continue
+            t.prompt[-1], t.out[-1], t.out_est[-1] = p, out, out // 2
+            costs = [-(-int(x) * 10 ** 6 // prefill) + max(int(a), int(b)) * decode
+                     for x, a, b in zip(t.prompt, t.out, t.out_est)]
+            rc, err, h = _create(lib, [t], cl, wl.grid)
+            if h.value:
+                lib.hx_sim_destroy(h)
+            assert (rc == H.HX_ERR_INVALID) == (max(costs) > top), (p, out, err)
+            assert max(costs) <= top or "2^28" in err, err
+
+
 def test_horizon_limit_is_exact(lib):
     # without fault windows the horizon is the sum over calls of
     # ceil(prompt * 10^6 / min prefill rate) + max(out, out_est) * max decode
