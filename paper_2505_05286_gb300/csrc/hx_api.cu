@@ -835,8 +835,9 @@ static int hx_sim_create_impl(const hx_trace* traces, int32_t n_traces, const hx
   h->place(&h->d_best_global, 2);
   h->place(&h->d_point_sums, 3 * (int64_t)h->n_points);
 
-  // launch shapes of the simulation kernel; later uploads may bring longer calls
-  int64_t blocks = (h->n_sims + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock;
+  // launch shapes of the simulation kernel, for the simulations that run; later
+  // uploads may bring longer calls
+  int64_t blocks = (h->n_work + hx::kWarpsPerBlock - 1) / hx::kWarpsPerBlock;
   if (opt && opt->max_resident_warps > 0)
     blocks = std::min<int64_t>(blocks, std::max<int64_t>(1, opt->max_resident_warps / hx::kWarpsPerBlock));
   const int family = sim_family(grid, ck, opt && opt->n_record > 0, opt && opt->force_generic, h->checked);

@@ -116,3 +116,24 @@ def test_calls_are_staged_where_that_is_cheaper(n, queries, staged):
             assert np.array_equal(got[f], want[f]), f
         sim.upload(wl.traces)
     sim.close()
+
+
+@pytest.mark.parametrize("record", [(), (4097,)])
+@pytest.mark.parametrize("n", [1, 5, 100])
+def test_a_subset_is_sized_by_what_runs(n, record):
+    """A few simulations of a large grid take the warps and the scratch that they
+    need (and with them the kernels for runs of few warps), not the grid's."""
+    wl = W.make_workload(2, n_traces=32, n_queries=60)
+    subset = [4097 + 13 * i for i in range(n)]
+    sim = H.Sim(wl.traces, wl.cluster, wl.grid, subset=subset, record_sims=record)
+    info = sim.info()
+    assert info["blocks"] == -(-n // info["warps_per_block"])
+    few = H.Sim(wl.traces, wl.cluster, W.subset_grid(wl.grid, [0]), max_resident_warps=4)
+    assert info["scratch_bytes"] == info["blocks"] * few.info()["scratch_bytes"]
+    few.close()
+    sim.run()
+    got, want = sim.results(), oracle.run(wl, subset)
+    sim.close()
+    for f in FIELDS:
+        assert np.array_equal(got[f][subset], want[f]), f
+    assert (np.delete(got["status"], subset) == H.HX_SKIPPED).all()
