@@ -192,7 +192,7 @@ struct hx_sim {
   // the simulation kernel's family and launch for the traces as they are: [0] with
   // short calls only, [1] with an attempt of kLongCall us or more
   struct Launch {
-    int family = hx::kSimWide, kernel = 0, blocks = 0, smem_per_block = 0;
+    int family = hx::kSimWide, kernel = 0, blocks = 0, smem_per_block = 0, slot_entries = 0;
   } launch[2];
   bool long_calls = false;
   int32_t* d_long = nullptr;    // the same on the device, for captured runs
@@ -541,10 +541,10 @@ int upload_inputs(hx_sim* h, const hx_trace* traces, int64_t bytes, cudaStream_t
 }
 
 // WarpShared and the instance states and slot entries that follow it.
-int per_warp_smem(const hx::ClusterK& ck, int family) {
+int per_warp_smem(const hx::ClusterK& ck, int family, int slot_entries) {
   const int64_t slot = family == hx::kSimWide ? sizeof(hx::Slot64) : sizeof(hx::Slot32);
   return (int)align_up((int64_t)sizeof(hx::WarpShared) + (ck.n_inst <= 32 ? 32 : 64) * (int64_t)sizeof(hx::InstState) +
-                       slot * ck.slot_entries, 16);
+                       slot * slot_entries, 16);
 }
 
 // The launch of a kernel family for a cluster, of up to `want` blocks: the kernel
@@ -552,8 +552,10 @@ int per_warp_smem(const hx::ClusterK& ck, int family) {
 int launch_shape(int family, const hx::ClusterK& ck, const cudaDeviceProp& prop, int64_t want, hx_sim::Launch* out) {
   want = std::max<int64_t>(want, 1);
   out->family = family;
-  out->kernel = sim_kernel_of(family, ck, few_warps(want * hx::kWarpsPerBlock, prop.multiProcessorCount));
-  out->smem_per_block = hx::kWarpsPerBlock * per_warp_smem(ck, family);
+  const bool few = few_warps(want * hx::kWarpsPerBlock, prop.multiProcessorCount);
+  out->kernel = sim_kernel_of(family, ck, few);
+  out->slot_entries = ck.n_inst <= 32 && hx::spaced_slots(1, family == hx::kSimWide, few) ? 16 * 32 : ck.slot_entries;
+  out->smem_per_block = hx::kWarpsPerBlock * per_warp_smem(ck, family, out->slot_entries);
   if (int rc = ensure_dyn_smem(out->kernel, out->smem_per_block)) return rc;
   int bps = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, (const void*)hx::kSimKernel[out->kernel],
@@ -584,6 +586,7 @@ __global__ void hx_gate_kernel(const int32_t* long_calls, int32_t want, unsigned
 
 int launch_sim(const hx_sim::Launch& l, const hx::SimArgs& sa, hx::ClusterK ck, cudaStream_t s) {
   ck.smem_per_warp = l.smem_per_block / hx::kWarpsPerBlock;
+  ck.slot_entries = l.slot_entries;
   if (int rc = ensure_dyn_smem(l.kernel, l.smem_per_block)) return rc;
   hx::kSimKernel[l.kernel]<<<(unsigned)l.blocks, hx::kWarpsPerBlock * 32, l.smem_per_block, s>>>(sa, ck);
   HX_CUDA(cudaGetLastError());
@@ -621,7 +624,7 @@ void fill_cluster(const hx_cluster* cluster, hx::ClusterK& ck) {
       ck.cnt[ty]++;
     }
   }
-  ck.slot_entries = ck.n_inst <= 32 ? 16 * 32 : base + 16;
+  ck.slot_entries = base + 16;
   // per-tenant SLO multipliers replace slo_mult_fp when given
   ck.n_tenants = std::max(cluster->n_tenants, 1);
   for (int t = 0; t < HX_MAX_TENANTS; ++t)

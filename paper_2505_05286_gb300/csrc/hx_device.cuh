@@ -67,7 +67,7 @@ struct ClusterK {
   int64_t slo_mult_fp;
   int32_t prefill[HX_MAX_TYPES], decode[HX_MAX_TYPES], slots[HX_MAX_TYPES], cnt[HX_MAX_TYPES];
   int32_t ref_prompt[4], ref_out[4];
-  int32_t slot_entries;     // slot entries per warp
+  int32_t slot_entries;     // slot entries per warp, packed; the kernel's own at launch
   int32_t smem_per_warp;
   uint8_t inst_type[HX_MAX_INST];
   uint8_t inst_slots[HX_MAX_INST];
@@ -163,10 +163,19 @@ constexpr uint32_t kWindowsBit = 1u << 31;
 constexpr int kHeapCodeShift = 27;  // the arena holds at most 4 * 2^24 + 1024 entries
 constexpr uint32_t kHeapOffMask = (1u << kHeapCodeShift) - 1;
 
+// Whether every instance has 16 slot entries, so that no load gives the first; if
+// not, it has its own slots only, and 16 entries follow the last instance's.  64-bit
+// times spaced (8 KB a warp) would let 20 warps reside on an SM where the registers of
+// the full GPU's form let 32: there they are packed (64 traces x 2000 queries x 64
+// points on 8 instances 29.4 -> 21.5 ms, 32 x 2000 x 256 on 16 81.4 -> 69.4), and spaced
+// in the form for few warps (packed, 8 x 2000 x 64 takes 9.53 ms against 9.33).
+__host__ __device__ constexpr bool spaced_slots(int instances_per_lane, bool wide, bool few) {
+  return instances_per_lane == 1 && (!wide || few);
+}
+
 // Per-warp shared memory of one simulation: per-simulation constants and
 // warp-uniform state, then an InstState per lane and instance of it and the
-// slot entries: an instance's are read 16 at a time, so up to 32 instances have
-// 16 each; more have their own slots only, and 16 entries follow the last.
+// slot entries, which are read 16 at a time (spaced_slots()).
 struct __align__(16) WarpShared {
   int4 pend[HX_MAX_K];          // this event's waiting dispatches: request id, service time and
                                 // Eq. (comp) on the instance, instance

@@ -686,6 +686,7 @@ template <int J, int kFamily, bool kFew>
 __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
   constexpr bool kLog = kFamily >= kSimLog, kGeneric = kFamily >= kSimGeneric;
   constexpr bool kFaults = kFamily >= kSimFaults, kWide = kFamily == kSimWide;
+  constexpr bool kSpaced = spaced_slots(J, kWide, kFew);
   using T = typename Times<kWide>::T;
   using Slot = typename Times<kWide>::Slot;
   constexpr T kIdle = ~T(0);                        // no time
@@ -859,8 +860,7 @@ __device__ __forceinline__ void sim_body(const SimArgs& a, const ClusterK& c) {
       status = HX_ERR_BOUNDS;
 #endif
 
-    // one instance per lane: 16 slot entries each, so that no load gives the first
-    auto first_slot = [&](int m, const InstState& I) -> uint32_t { return J == 1 ? 16u * m : (kFaults ? I.cfg & ~kWindowsBit : I.cfg) >> 16; };
+    auto first_slot = [&](int m, const InstState& I) -> uint32_t { return kSpaced ? 16u * m : (kFaults ? I.cfg & ~kWindowsBit : I.cfg) >> 16; };
     // A request starts that waited in a long queue: its record's second half and
     // the records that follow have left L1 since its query arrived (3000 queries on
     // 64 instances, whose alpha = 1 queue grows past 1000: 29.0 -> 26.4 ms).  Left

@@ -137,3 +137,22 @@ def test_a_subset_is_sized_by_what_runs(n, record):
     for f in FIELDS:
         assert np.array_equal(got[f][subset], want[f]), f
     assert (np.delete(got["status"], subset) == H.HX_SKIPPED).all()
+
+
+@pytest.mark.parametrize("n_inst", [8, 32])
+def test_long_calls_keep_a_full_gpu(n_inst):
+    """A call past 2^25 us moves the whole run to 64-bit times: its slots then take
+    twice the room, which must not cost the run more than a block an SM."""
+    wl = W.make_workload(1, n_traces=80, n_queries=20)
+    wl.cluster.inst_type = (np.arange(n_inst) % 3).astype(np.uint8)  # 4 to 16 slots each
+    sim = H.Sim(wl.traces, wl.cluster, wl.grid)
+    short = sim.info()["blocks"]
+    sim.close()
+    wl.traces[3].prompt[7] = 1_000_000
+    sim = H.Sim(wl.traces, wl.cluster, wl.grid)
+    assert sim.info()["generic_kernel"] == 1 and sim.info()["blocks"] >= short * 7 // 8
+    sim.run()
+    got, want = sim.results(), oracle.run(wl)
+    sim.close()
+    for f in FIELDS:
+        assert np.array_equal(got[f], want[f]), f
