@@ -105,3 +105,28 @@ def test_logged_budgets(n_inst, kind):
         cl.faults["t1_us"] //= 4
     grid = _grid([0, 1, 2] if kind == "policies" else [0])
     assert _run(tr, cl, grid, record=list(range(grid.n_points))[::-1]) == 1
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("recipe", [0, 4])
+def test_far_first_query(recipe):
+    """A trace whose first query lies 9.5 hours before the others: the same schedule
+    and budgets as the oracle's, and the urgency keys cost the others no more than
+    without the gap (deadlines that far overdue take exact 64-bit divisions, which
+    is no business of requests that are not)."""
+    wl = W.make_workload(recipe, n_traces=1, n_queries=1000)
+    tr = wl.traces[0]
+    gap = tr.arrival_us.copy()
+    gap[1:] += 2 ** 35
+    grid = W.subset_grid(wl.grid, [wl.grid.n_points - 1])  # alpha = 1: long queues
+    cycles = []
+    for t in (tr, W.Trace(**{**tr.__dict__, "arrival_us": gap})):
+        _run(t, wl.cluster, grid, record=[0])
+        sim = H.Sim([t], wl.cluster, grid)
+        best = []
+        for _ in range(7):
+            sim.run()
+            best.append(int(sim.results()["cycles_k"][0]))
+        sim.close()
+        cycles.append(min(best))
+    assert cycles[1] < 1.1 * cycles[0], cycles
