@@ -156,3 +156,32 @@ def test_long_calls_keep_a_full_gpu(n_inst):
     sim.close()
     for f in FIELDS:
         assert np.array_equal(got[f], want[f]), f
+
+
+@pytest.mark.parametrize("n_inst", [3, 40])
+@pytest.mark.parametrize("slow,timeout", [(None, 0), (2, 0), (2, 2), (0.5, 1), (0, 2), (3, 7), (100, 0)])
+def test_times_are_64_bit_only_where_an_attempt_needs_them(n_inst, slow, timeout):
+    """The first attempt length (slowed or timed out by the fault windows) that takes
+    64-bit times is 2^25 us; told by the room that a block's slot entries take."""
+    wl = W.make_workload(1, n_traces=1, n_queries=5)
+    tr, cl = wl.traces[0], wl.cluster
+    cl.inst_type = (np.arange(n_inst) % 3).astype(np.uint8)
+    cl.prefill_tok_s[:], cl.decode_us_tok[:] = 1_000_000, 32
+    stretch = W.SCALE
+    if slow is not None:
+        cl.timeout_mult_fp = timeout * W.SCALE
+        cl.faults = np.zeros(1, W.FAULT_DTYPE)
+        cl.faults[0] = (n_inst - 1, 0, 0, 1000, int(slow * W.SCALE))
+        stretch = max(stretch, cl.timeout_mult_fp, int(slow * W.SCALE))
+    first = (2 ** 25 - 1) * W.SCALE // stretch + 1  # us of the shortest such call
+
+    def smem(cost):
+        tr.prompt[:], tr.out[:], tr.out_est[:] = 1, 1, 1
+        tr.out[3] = (cost - 1) // 32
+        tr.prompt[3] = cost - 32 * int(tr.out[3])
+        sim = H.Sim([tr], cl, wl.grid)
+        block = sim.info()["smem_per_block"]
+        sim.close()
+        return block
+    assert smem(first - 1) == smem(first // 2)
+    assert smem(first) == smem(first + 1) > smem(first - 1)
