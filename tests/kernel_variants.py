@@ -1,17 +1,12 @@
-"""Kernel variants: source edits of the simulation kernel, built beside the
-library and timed against it on the same workload, each required to give
-bit-identical results.  This is how the alternatives the design notes
-mention were measured (GPU only).
+"""Kernel variants: the library built beside itself with other compile-time
+choices of the simulation kernel and timed against it on the same workload, each
+required to give bit-identical results (GPU only).
 
     python -m tests.kernel_variants FAMILY [--traces 64] [--reps 3] [--out FILE]
 
 Family `occupancy`: 8, 7 or 6 resident 4-warp blocks per SM (the
-register budget follows).
-
-A variant is a list of edits ((anchor, replacement) in hx_kernels.cu, or
-(file, anchor, replacement)) and nvcc flags.  The families measured against
-earlier kernels (reward and key placement, record prefetch, heap sift, cache
-policies) left with the code that they edited.
+register budget follows).  A variant is a list of nvcc flags for
+hx_kernels.cu, each setting a macro that the source leaves to the build.
 """
 from __future__ import annotations
 
@@ -34,30 +29,20 @@ NVCC = ["nvcc", "-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo"
         "-fPIC", "-I", os.path.join(ROOT, "include")]
 
 VARIANTS = {
-    "occupancy": {"blocks8": ([], ["-DHX_SIM_MIN_BLOCKS(J)=8"]), "blocks7": ([], ["-DHX_SIM_MIN_BLOCKS(J)=7"]), "blocks6": ([], ["-DHX_SIM_MIN_BLOCKS(J)=6"])},
+    "occupancy": {f"blocks{n}": [f"-DHX_SIM_MIN_BLOCKS(J)={n}"] for n in (8, 7, 6)},
 }
 
 
-def make_variant(name, edits, flags=()):
-    """Copy the library sources, apply the edits ((anchor, replacement) in
-    hx_kernels.cu, or (file, anchor, replacement)), build a .so (extra nvcc
-    flags for hx_kernels.cu)."""
+def make_variant(name, flags):
+    """Build the library into a .so of its own (extra nvcc flags for hx_kernels.cu)."""
     d = os.path.join(OUT, name)
     shutil.rmtree(d, ignore_errors=True)
-    shutil.copytree(CSRC, os.path.join(d, "csrc"))
-    for e in edits:
-        f, a, b = e if len(e) == 3 else ("hx_kernels.cu", *e)
-        p = os.path.join(d, "csrc", f)
-        s = open(p).read()
-        if a not in s:
-            raise RuntimeError(f"variant {name}: anchor not found in {f}: {a[:60]!r}")
-        open(p, "w").write(s.replace(a, b))
+    os.makedirs(d)
     objs = []
     for src in ("hx_kernels.cu", "hx_api.cu"):
         o = os.path.join(d, src.replace(".cu", ".o"))
         extra = list(flags) if src == "hx_kernels.cu" else []
-        subprocess.check_call(NVCC + ["-I", os.path.join(d, "csrc"), *extra, "-c", os.path.join(d, "csrc", src),
-                                      "-o", o])
+        subprocess.check_call(NVCC + ["-I", CSRC, *extra, "-c", os.path.join(CSRC, src), "-o", o])
         objs.append(o)
     lib = os.path.join(d, "libhxsim.so")
     subprocess.check_call(NVCC[:3] + ["-shared", "-o", lib] + objs)
@@ -105,9 +90,8 @@ def main(argv=None):
     out = {"workload": f"{wl.name} cut to {args.traces} traces", "sims": wl.n_sims, "library_ms": base_ms,
            "library_all_ms": base_all, "variants": {}}
     print("library", base_ms, base_all, flush=True)
-    for name, spec in VARIANTS[args.family].items():
-        edits, flags = spec if isinstance(spec, tuple) else (spec, [])
-        ms, all_ms, r = time_lib(make_variant(name, edits, flags), wl, args.reps)
+    for name, flags in VARIANTS[args.family].items():
+        ms, all_ms, r = time_lib(make_variant(name, flags), wl, args.reps)
         same = all(np.array_equal(r[f], base[f]) for f in fields)
         out["variants"][name] = {"ms": ms, "all_ms": all_ms, "same_results": same, "speedup": base_ms / ms}
         print(name, ms, all_ms, same, round(base_ms / ms, 4), flush=True)
