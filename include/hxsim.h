@@ -221,7 +221,9 @@ typedef struct hx_extra {
 typedef struct hx_sim hx_sim;
 
 /* Validate and copy traces, cluster and grid to library-owned device memory
- * and size the per-warp scratch.  On failure *out is NULL.
+ * and size the per-warp scratch.  On failure *out is NULL.  The handle keeps a
+ * host copy of its inputs for later uploads where that makes them cheaper (many
+ * small traces; at most 64 MiB).
  *
  * Defines the simulations of Sec. 4.3's alpha tuning: every (trace, point)
  * pair replays the trace through the scheduler of Sec. 4.1 (Eq. comp for
@@ -249,8 +251,11 @@ int hx_sim_upload(hx_sim* h, const hx_trace* traces, int32_t n_traces, void* str
  * simulation (Sec. 4.1 dispatch and Sec. 4.2 local queues, event by event,
  * reduced to Sec. 4.3's T_0.95 and the SLO count), and the best-point
  * reduction (Sec. 4.3's argmin over the grid).  Asynchronous; may be called
- * repeatedly.  Errors: HX_ERR_INVALID (NULL handle), HX_ERR_CUDA (a launch
- * failed); per-simulation problems are reported in hx_result.status. */
+ * repeatedly.  A call on a capturing stream puts two simulation kernels into the
+ * graph, of which each replay gives all the work to the one that the traces
+ * uploaded by then need (attempts below or from 2^25 us).  Errors:
+ * HX_ERR_INVALID (NULL handle), HX_ERR_CUDA (a launch failed); per-simulation
+ * problems are reported in hx_result.status. */
 int hx_sim_run(hx_sim* h, void* stream);
 
 /* Wait for the last run and copy n <= n_sims results to host memory

@@ -418,9 +418,9 @@ int host_threads(int32_t n_traces, int64_t calls) {
 // Whether to stage the per-call arrays of so many traces: up to 64 MiB of inputs,
 // and 1.25 MiB a trace for every thread that stages them.  A thread stages about 19
 // GB/s and a trace's own six copies cost about 66 us, their bytes next to nothing:
-// one trace of 45k calls uploads in 0.25 ms staged and 0.28 not, one of 151k in 0.72
-// and 0.67, one of 756k in 3.3 and 3.0; four of 151k (four threads) in 0.95 and
-// 1.05, 64 of 23k in 2.4 and 4.9.
+// an upload of one trace of 45k calls takes 0.24 ms staged, 0.27 not; one of 151k
+// 0.05 ms longer staged, one of 756k 0.35 ms (of 2.7); four of 151k (four threads)
+// 0.1 ms less (of 0.9), 64 of 23k 2.4 ms instead of 4.9.
 constexpr int64_t kStageMost = int64_t(64) << 20, kStagePerThread = int64_t(1280) << 10;
 bool stage_calls_of(int32_t n_traces, int64_t calls, int64_t input_bytes, int64_t call_bytes) {
   return input_bytes <= kStageMost && call_bytes <= kStagePerThread * n_traces * host_threads(n_traces, calls);

@@ -283,7 +283,9 @@ namespace {
 // and the bit search that lengthened the event's chain (8 x 2000 queries x 64
 // points 6.80 -> 6.29 ms, 8 x 20000 x 1024 on 64 instances 431 -> 399 ms; fault
 // windows on 24 x 2000 x 64 15.5 -> 13.8 ms).  Longer attempts have 64-bit times,
-// base 0.
+// base 0, in a family that carries policies, tenants and faults too: one such
+// attempt in a grid that needs none of these costs half as much again (8 x 2000 x 64
+// 6.3 -> 9.3 ms, 64 x 2000 x 64 14.1 -> 21.3, 8 x 4000 x 1024 on 64 instances 74 -> 112).
 template <bool kWide>
 struct Times {
   using T = uint32_t;
@@ -631,9 +633,10 @@ __device__ __forceinline__ void finish_query(WarpShared* W, int64_t now, int64_t
 }  // namespace
 
 // Resident blocks per SM the register allocation aims for (4 warps each): 8
-// with one instance per lane; with two, 7, whose 72 registers hold a
-// simulation's state without spills (8 spill 48 bytes in the event loop: 8
-// traces x 20000 queries x 1024 points 503 ms against 458 ms).  The form for few
+// with one instance per lane; with two, 7, whose 72 registers hold the event
+// loop's state (8 spill 48 bytes in the event loop: 8 traces x 20000 queries x
+// 1024 points 503 ms against 458 ms).  What these forms spill, 0 to 48 bytes by
+// family, lies outside the loop: no local load per event is counted.  The form for few
 // warps aims at 5 (96 registers, no spills: 64 x 3001 x 16 25.5 -> 23.5 ms; 4 or 6
 // blocks 1 to 4 % slower).
 #ifndef HX_SIM_MIN_BLOCKS
